@@ -451,6 +451,7 @@ fh_status solve_groups(std::vector<Group*>& groups, int d, int nl, const double 
         }
       }
       for (int gi = 0; gi < ng; ++gi) {
+        if (!active[gi]) continue;  // p32->x still holds the correction of an earlier round
         Group& g = *groups[gi];
         std::vector<SolveResult> res(st[gi].size());
         g.p32->solve_results(res.data());

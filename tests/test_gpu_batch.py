@@ -115,3 +115,27 @@ def test_batch_rejects_bad_cells():
         fh.Batch([np.zeros((8, 9), np.uint8)], [micro.isotropic_table([1.0], 2)])
     with pytest.raises(fh.FhError):
         fh.Batch([np.full((9, 9), 2, np.uint8)], [micro.isotropic_table([1.0, 2.0], 2)])
+
+
+@pytest.mark.parametrize("tol", [1e-7, 1e-8, 1e-9, 1e-10])
+def test_size_groups_that_need_fewer_refinement_steps_keep_their_solution(tol):
+    """Size groups refine until their own cells are done; a group that is done
+    before the others must not receive its last correction again.  Each cell's
+    columns equal those of the same group solved alone (same kernels, same
+    arithmetic), whatever the other groups need."""
+    cuda_or_skip()
+    from paper_1004_1122_gb300 import fh
+
+    small = [micro.rsa_disks(27, 0.3, 2, 4, seed=micro.config_seed(4, 40 + k)) for k in range(3)]
+    large = [micro.rsa_disks(135, 0.35, 4, 9, seed=micro.config_seed(4, 50 + k)) for k in range(2)]
+    tab = {27: micro.isotropic_table([1.0, 8.0], 2), 135: micro.isotropic_table([1.0, 900.0], 2)}
+
+    def solve(cells):
+        with fh.Batch(cells, [tab[c.shape[0]] for c in cells], nloads=2, precision="fp32_refined") as b:
+            Leff, st, _, info = b.solve(np.eye(2), tol=tol, method="cg", max_iter=20000)
+        assert np.all(st == 0), st
+        return Leff
+
+    together = solve(small + large)
+    alone = np.concatenate([solve(small), solve(large)])
+    np.testing.assert_allclose(together, alone, rtol=1e-12, atol=0)
