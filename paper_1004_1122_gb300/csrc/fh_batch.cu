@@ -228,6 +228,7 @@ fh_status fh_batch_create(fh_batch** out, int ncells, const int* N, const uint8_
     if (!rc && precision == FH_FP32_REFINED) {
       g.p32 = new (std::nothrow) Pipeline<float>();
       if (!g.p32) rc = FH_ERR_OOM;
+      else g.p32->want_spectral = true;
       if (!rc) rc = g.p32->init(pb, nloads, true, g.st, err);
     }
     for (int l = 0; l < nloads && !rc; ++l) {
@@ -251,18 +252,15 @@ fh_status fh_batch_autotune(fh_batch* b, double* ms_before, double* ms_after) {
   for (Group& g : b->groups) {
     if (!g.p32) continue;  // float64 batches keep their default shapes
     std::string err;
-    double t, cur = 0.0;
-    for (int what = 0; what < 4; ++what) {
-      int rc = g.p32->profile(what, 10, &t, err);
-      if (rc) {
-        b->err = err;
-        return (fh_status)rc;
-      }
-      cur += t;
+    double cur = 0.0;
+    int rc = g.p32->iteration_time(&cur, err);
+    if (rc) {
+      b->err = err;
+      return (fh_status)rc;
     }
     fh::Tuning best;
     double best_ms;
-    int rc = Pipeline<float>::autotune(g.pb, b->nloads, g.st, best, best_ms, err, kBatchTuneCandidates);
+    rc = Pipeline<float>::autotune(g.pb, b->nloads, g.st, best, best_ms, err, kBatchTuneCandidates, true);
     if (rc) {
       b->err = err;
       return (fh_status)rc;
@@ -272,11 +270,13 @@ fh_status fh_batch_autotune(fh_batch* b, double* ms_before, double* ms_after) {
       cudaStreamSynchronize(g.st);
       g.p32->release();
       *g.p32 = Pipeline<float>();
+      g.p32->want_spectral = true;
       rc = g.p32->init(g.pb, b->nloads, true, g.st, err, &best);
       if (rc) {
         // fall back to the default shapes
         g.p32->release();
         *g.p32 = Pipeline<float>();
+        g.p32->want_spectral = true;
         rc = g.p32->init(g.pb, b->nloads, true, g.st, err);
         if (rc) {
           b->err = err;
@@ -601,6 +601,7 @@ int solve_all_loads(const Problem& pb, int precision, double tol, int method, in
       if (!g->p32) {
         rc = FH_ERR_OOM;
       } else {
+        g->p32->want_spectral = true;
         // launch shapes tuned for d loads per launch (fh_autotune_loads), else the defaults
         Tuning t;
         rc = -1;
@@ -609,6 +610,7 @@ int solve_all_loads(const Problem& pb, int precision, double tol, int method, in
           if (rc) {
             g->p32->release();
             *g->p32 = Pipeline<float>();
+            g->p32->want_spectral = true;
           }
         }
         if (rc) rc = g->p32->init(pb, d, true, g->st, err);

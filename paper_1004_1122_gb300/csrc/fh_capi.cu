@@ -235,8 +235,10 @@ int init_tuned(Pipeline<T>* P, const Problem& pb, bool krylov, cudaStream_t st, 
   Tuning t;
   if (cache_lookup(tune_key(pb, 1, sizeof(T) == 8), t)) {
     if (P->init(pb, 1, krylov, st, err, &t) == 0) return 0;
+    const bool spec = P->want_spectral;
     P->release();
     *P = Pipeline<T>();
+    P->want_spectral = spec;
   }
   return P->init(pb, 1, krylov, st, err);
 }
@@ -426,6 +428,7 @@ fh_status fh_create(fh_ctx** out, int d, const int* N, const double* Y, const ui
   if (!rc && (precision == FH_FP32 || precision == FH_FP32_REFINED)) {
     c->p32 = new (std::nothrow) Pipeline<float>();
     if (!c->p32) rc = FH_ERR_OOM;
+    else c->p32->want_spectral = precision == FH_FP32_REFINED;
     if (!rc) rc = init_tuned(c->p32, pb, true, c->st, err);
   }
   const size_t vbytes = (size_t)d * pb.nodes * sizeof(double);
@@ -768,7 +771,7 @@ fh_status fh_solve(fh_ctx* c, const double* E, double tol, int method, int max_i
       for (int i = 0; i < d; ++i)
         for (int j = 0; j < d; ++j) M[i * 3 + j] = c->pb.L0[i * d + j];
       double n2;
-      rc = P->matnorm2(P->p[0], M, &n2, err);
+      rc = P->spec_run_ ? P->spec_dir_norm2(M, &n2, err) : P->matnorm2(P->p[0], M, &n2, err);
       if (rc) return from_rc(c, rc, err);
       eta_r = std::fabs(last_alpha) * std::sqrt(n2 / e2);
     }
@@ -890,6 +893,7 @@ fh_status fh_project_compatible(fh_ctx* c, const double* in, double* out) {
 
 fh_status fh_profile(fh_ctx* c, int dtype, int what, int reps, double* ms) {
   if (!c || !ms || reps < 1) return FH_ERR_ARG;
+  if (what > 5) what = 4;  // no such piece
   std::string err;
   int rc;
   if (dtype == FH_FP64 && c->p64 && c->p64->x[0]) {
@@ -908,15 +912,13 @@ namespace {
 template <typename T>
 fh_status autotune_one(fh_ctx* c, Pipeline<T>*& P, bool krylov, double* ms_before, double* ms_after) {
   std::string err;
-  double before = 0.0, t;
-  for (int what = 0; what < 4; ++what) {
-    int rc = P->profile(what, 10, &t, err);
-    if (rc) return from_rc(c, rc, err);
-    before += t;
-  }
+  double before = 0.0;
+  int rc = P->iteration_time(&before, err);
+  if (rc) return from_rc(c, rc, err);
   Tuning best;
   double best_ms;
-  int rc = Pipeline<T>::autotune(c->pb, 1, c->st, best, best_ms, err);
+  const bool spec = P->want_spectral;
+  rc = Pipeline<T>::autotune(c->pb, 1, c->st, best, best_ms, err, 256, spec);
   if (rc) return from_rc(c, rc, err);
   if (ms_before) *ms_before = before;
   if (best_ms < before && !(best == P->tuning)) {
@@ -926,6 +928,7 @@ fh_status autotune_one(fh_ctx* c, Pipeline<T>*& P, bool krylov, double* ms_befor
     P->release();
     delete P;
     P = Q;
+    P->want_spectral = spec;
     rc = P->init(c->pb, 1, krylov, c->st, err, &best);
     if (rc) return from_rc(c, rc, err);
   } else {
@@ -954,20 +957,18 @@ fh_status fh_autotune_loads(fh_ctx* c, double* ms_before, double* ms_after) {
   const int d = c->pb.d;
   std::string err;
   // the default shapes' time, from a temporary pipeline
-  double before = 0.0, t;
+  double before = 0.0;
   {
     fh::Pipeline<float> P;
+    P.want_spectral = true;
     int rc = P.init(c->pb, d, true, c->st, err);
-    for (int what = 0; what < 4 && !rc; ++what) {
-      rc = P.profile(what, 10, &t, err);
-      before += t;
-    }
+    if (!rc) rc = P.iteration_time(&before, err);
     P.release();
     if (rc) return from_rc(c, rc, err);
   }
   Tuning best;
   double best_ms;
-  int rc = fh::Pipeline<float>::autotune(c->pb, d, c->st, best, best_ms, err);
+  int rc = fh::Pipeline<float>::autotune(c->pb, d, c->st, best, best_ms, err, 256, true);
   if (rc) return from_rc(c, rc, err);
   cache_store(tune_key(c->pb, d, false), best, best_ms);
   // the next fh_solve_all rebuilds its pipelines with the tuned shapes

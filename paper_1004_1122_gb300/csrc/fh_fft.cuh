@@ -151,10 +151,66 @@ template <int S, bool INV, typename T> struct RegDFT<1, S, INV, T> {
 
 template <int P, int S, bool INV, typename T, bool PRIME> struct RegDFTImpl;
 
+// odd prime P, float32: the same form on packed pairs (one instruction for the
+// real and the imaginary part).  The differences are formed with their parts
+// swapped, so that the product with i is a packed multiply-add with constants
+// (s, -s) and no register moves: 7 instructions for radix 3 instead of 14.
+template <int P, int S, bool INV> struct RegDFTPacked {
+  static __device__ __forceinline__ void run(float2* v) {
+    constexpr int h = (P - 1) / 2;
+    float2 a[h + 1], b[h + 1];
+#pragma unroll
+    for (int j = 1; j <= h; ++j) {
+      const float2 p = v[j * S], q = v[(P - j) * S];
+      a[j] = __fadd2_rn(p, q);
+      b[j] = make_float2(p.y - q.y, p.x - q.x);  // swapped
+    }
+    const float2 x0 = v[0];
+    float2 sum = x0;
+#pragma unroll
+    for (int j = 1; j <= h; ++j) sum = __fadd2_rn(sum, a[j]);
+    static_for<h>([&](auto K) {
+      constexpr int k = decltype(K)::value + 1;
+      float2 re = x0;
+      static_for<h>([&](auto J) {
+        constexpr int j = decltype(J)::value + 1;
+        constexpr float c = (float)ct::cos2pi((long long)j * k, P);
+        re = __ffma2_rn(a[j], make_float2(c, c), re);
+      });
+      // forward X_k = re - i im, X_{P-k} = re + i im; inverse swaps the signs
+      float2 m1 = re, p1 = re;
+      if constexpr (h == 1) {
+        constexpr float s = (float)ct::sin2pi(1, P);
+        m1 = __ffma2_rn(b[1], make_float2(s, -s), re);
+        p1 = __ffma2_rn(b[1], make_float2(-s, s), re);
+      } else {
+        float2 im;
+        static_for<h>([&](auto J) {
+          constexpr int j = decltype(J)::value + 1;
+          constexpr float s = (float)ct::sin2pi((long long)j * k, P);
+          if constexpr (j == 1)
+            im = __fmul2_rn(b[j], make_float2(s, -s));
+          else
+            im = __ffma2_rn(b[j], make_float2(s, -s), im);
+        });
+        m1 = __fadd2_rn(re, im);
+        p1 = __ffma2_rn(im, make_float2(-1.0f, -1.0f), re);
+      }
+      v[k * S] = INV ? p1 : m1;
+      v[(P - k) * S] = INV ? m1 : p1;
+    });
+    v[0] = sum;
+  }
+};
+
 // odd prime P: symmetric form
 template <int P, int S, bool INV, typename T> struct RegDFTImpl<P, S, INV, T, true> {
   static __device__ __forceinline__ void run(cplx<T>* v) {
     static_assert(P % 2 == 1, "odd primes only");
+    if constexpr (std::is_same<T, float>::value) {
+      RegDFTPacked<P, S, INV>::run(v);
+      return;
+    } else {
     constexpr int h = (P - 1) / 2;
     using C = cplx<T>;
     C a[h + 1], b[h + 1];
@@ -187,6 +243,7 @@ template <int P, int S, bool INV, typename T> struct RegDFTImpl<P, S, INV, T, tr
       else     { v[k * S] = m1; v[(P - k) * S] = p1; }
     });
     v[0] = sum;
+    }
   }
 };
 
@@ -321,11 +378,22 @@ __device__ __forceinline__ void stockham_stage(cplx<T> (&v)[EM], cplx<T>* sm, in
 #define FH_FOR_EACH_RADIX_X(X) \
   X(2) X(3) X(4) X(5) X(7) X(8) X(9) X(11) X(13) X(15) X(16) X(17) X(25) X(27)
 
+// The small set (DynPlan9 kernels): at most 9 values per thread, so many more
+// threads work on one sequence.
+#define FH_FOR_EACH_RADIX_S(X) X(3) X(5) X(7) X(9)
+
 // Largest prime radix of the extended set; every extended plan's register
 // array holds at least one butterfly of it.
 constexpr int kMaxPrimeX = 17;
 template <typename T> struct RegBudgetX {
   static constexpr int value = RegBudget<T>::value > kMaxPrimeX ? RegBudget<T>::value : kMaxPrimeX;
+};
+
+// Radix sets of the run-time plans and their register budgets.
+enum : int { kRadixStd = 0, kRadixExt = 1, kRadixSmall = 2 };
+constexpr int kSmallBudget = 9;
+template <typename T, int SET> struct PlanBudget {
+  static constexpr int value = SET == kRadixExt ? RegBudgetX<T>::value : SET == kRadixSmall ? kSmallBudget : RegBudget<T>::value;
 };
 
 // Maximum number of stages in a plan.
@@ -335,15 +403,15 @@ struct FFTPlan {
   int n;                    // sequence length
   int nstages;
   int radix[kMaxStages];
-  int ext;                  // 1: uses a radix of the extended set (DynPlanX kernels)
+  int ext;                  // 1: uses a radix of the extended set (DynPlanX kernels); 2: small set (DynPlan9)
 };
 
-// Run all stages of the plan on one sequence layout.  X selects the extended
-// radix set (and its register budget).
-template <bool INV, typename T, bool X = false>
+// Run all stages of the plan on one sequence layout.  SET selects the radix
+// set (and its register budget).
+template <bool INV, typename T, int SET = kRadixStd>
 __device__ __forceinline__ void run_fft(cplx<T>* sm, int is, const FFTPlan& pl, int u, int nthr,
                                         const cplx<T>* __restrict__ tw) {
-  constexpr int EM = X ? RegBudgetX<T>::value : RegBudget<T>::value;
+  constexpr int EM = PlanBudget<T, SET>::value;
   cplx<T> v[EM];
   int Ns = 1;
   for (int s = 0; s < pl.nstages; ++s) {
@@ -352,9 +420,14 @@ __device__ __forceinline__ void run_fft(cplx<T>* sm, int is, const FFTPlan& pl, 
   case RR:                                                                     \
     if constexpr (RR <= EM) stockham_stage<RR, INV, T, EM>(v, sm, is, pl.n, Ns, u, nthr, tw); \
     break;
-    if constexpr (X) {
+    if constexpr (SET == kRadixExt) {
       switch (R) {
         FH_FOR_EACH_RADIX_X(FH_STAGE_CASE)
+        default: break;
+      }
+    } else if constexpr (SET == kRadixSmall) {
+      switch (R) {
+        FH_FOR_EACH_RADIX_S(FH_STAGE_CASE)
         default: break;
       }
     } else {
@@ -368,15 +441,16 @@ __device__ __forceinline__ void run_fft(cplx<T>* sm, int is, const FFTPlan& pl, 
   }
 }
 
-// Forward FFT, a pointwise operation in the frequency domain, and the inverse
-// FFT, with the last forward stage and the first inverse stage fused in
-// registers.  The inverse runs the forward radices in reverse order, so its
-// first stage (Ns = 1) reads exactly the positions j + r n/R the last forward
-// stage produced (Ns = n/R) and no shared-memory round trip or barrier pair is
-// needed in between.  mid(v, i, active) maps the spectrum value at row i; it
-// is called by every thread of the CTA for the same (b, r) sequence, so it may
-// use warp shuffles (inactive threads pass active = false and garbage values).
-template <int R, typename T, int EM, typename F>
+// A transform, a pointwise operation, and the transform back (forward first,
+// or inverse first when INV), with the last stage of the first and the first
+// stage of the second fused in registers.  The second transform runs the
+// radices in reverse order, so its first stage (Ns = 1) reads exactly the
+// positions j + r n/R the last stage before it produced (Ns = n/R) and no
+// shared-memory round trip or barrier pair is needed in between.
+// mid(v, i, active) maps the value at position i; it is called by every thread
+// of the CTA for the same (b, r) sequence, so it may use warp shuffles
+// (inactive threads pass active = false and garbage values).
+template <int R, bool INV, typename T, int EM, typename F>
 __device__ __forceinline__ void fused_middle(cplx<T> (&v)[EM], cplx<T>* sm, int is, int n, int u, int nthr,
                                              const cplx<T>* __restrict__ tw, F& mid) {
   using C = cplx<T>;
@@ -394,11 +468,12 @@ __device__ __forceinline__ void fused_middle(cplx<T> (&v)[EM], cplx<T>* sm, int 
         int ti = j;
 #pragma unroll
         for (int r = 1; r < R; ++r) {
-          v[b * R + r] = cmul(v[b * R + r], ld_tw(tw + ti));
+          const C w = ld_tw(tw + ti);
+          v[b * R + r] = INV ? cmulc(v[b * R + r], w) : cmul(v[b * R + r], w);
           ti += j;
         }
       }
-      RegDFT<R, 1, false, T>::run(&v[b * R]);
+      RegDFT<R, 1, INV, T>::run(&v[b * R]);
     }
   }
 #pragma unroll
@@ -407,7 +482,7 @@ __device__ __forceinline__ void fused_middle(cplx<T> (&v)[EM], cplx<T>* sm, int 
     const bool act = j < nb;
 #pragma unroll
     for (int r = 0; r < R; ++r) v[b * R + r] = mid(v[b * R + r], j + r * nb, act);
-    if (act) RegDFT<R, 1, true, T>::run(&v[b * R]);
+    if (act) RegDFT<R, 1, !INV, T>::run(&v[b * R]);
   }
   __syncthreads();
 #pragma unroll
@@ -422,17 +497,22 @@ __device__ __forceinline__ void fused_middle(cplx<T> (&v)[EM], cplx<T>* sm, int 
   __syncthreads();
 }
 
-template <typename T, typename F, bool X = false>
+template <typename T, typename F, int SET = kRadixStd, bool INV = false>
 __device__ __forceinline__ void run_fft_fused(cplx<T>* sm, int is, const FFTPlan& pl, int u, int nthr,
                                               const cplx<T>* __restrict__ tw, F& mid) {
-  constexpr int EM = X ? RegBudgetX<T>::value : RegBudget<T>::value;
+  constexpr int EM = PlanBudget<T, SET>::value;
   cplx<T> v[EM];
   const int S = pl.nstages;
   int Ns = 1;
 #define FH_SWITCH(R, CASE)             \
-  if constexpr (X) {                   \
+  if constexpr (SET == kRadixExt) {    \
     switch (R) {                       \
       FH_FOR_EACH_RADIX_X(CASE)        \
+      default: break;                  \
+    }                                  \
+  } else if constexpr (SET == kRadixSmall) { \
+    switch (R) {                       \
+      FH_FOR_EACH_RADIX_S(CASE)        \
       default: break;                  \
     }                                  \
   } else {                             \
@@ -444,7 +524,7 @@ __device__ __forceinline__ void run_fft_fused(cplx<T>* sm, int is, const FFTPlan
   for (int s = 0; s + 1 < S; ++s) {
 #define FH_STAGE_CASE(RR)                                                                          \
   case RR:                                                                                         \
-    if constexpr (RR <= EM) stockham_stage<RR, false, T, EM>(v, sm, is, pl.n, Ns, u, nthr, tw); \
+    if constexpr (RR <= EM) stockham_stage<RR, INV, T, EM>(v, sm, is, pl.n, Ns, u, nthr, tw); \
     break;
     FH_SWITCH(pl.radix[s], FH_STAGE_CASE)
 #undef FH_STAGE_CASE
@@ -452,7 +532,7 @@ __device__ __forceinline__ void run_fft_fused(cplx<T>* sm, int is, const FFTPlan
   }
 #define FH_MID_CASE(RR)                                                              \
   case RR:                                                                           \
-    if constexpr (RR <= EM) fused_middle<RR, T, EM>(v, sm, is, pl.n, u, nthr, tw, mid); \
+    if constexpr (RR <= EM) fused_middle<RR, INV, T, EM>(v, sm, is, pl.n, u, nthr, tw, mid); \
     break;
   FH_SWITCH(pl.radix[S - 1], FH_MID_CASE)
 #undef FH_MID_CASE
@@ -460,7 +540,7 @@ __device__ __forceinline__ void run_fft_fused(cplx<T>* sm, int is, const FFTPlan
   for (int s = S - 2; s >= 0; --s) {
 #define FH_STAGE_CASE(RR)                                                                         \
   case RR:                                                                                        \
-    if constexpr (RR <= EM) stockham_stage<RR, true, T, EM>(v, sm, is, pl.n, Ns, u, nthr, tw); \
+    if constexpr (RR <= EM) stockham_stage<RR, !INV, T, EM>(v, sm, is, pl.n, Ns, u, nthr, tw); \
     break;
     FH_SWITCH(pl.radix[s], FH_STAGE_CASE)
 #undef FH_STAGE_CASE
@@ -479,6 +559,8 @@ __device__ __forceinline__ void run_fft_fused(cplx<T>* sm, int is, const FFTPlan
 struct DynPlan {};
 // Run-time plan over the extended radix set (primes 11, 13, 17 as well).
 struct DynPlanX {};
+// Run-time plan over the small radix set (at most 9 values per thread).
+struct DynPlan9 {};
 
 template <int... Rs> struct CPlan {
   static constexpr int S = sizeof...(Rs);
@@ -517,19 +599,19 @@ __device__ __forceinline__ void run_fft_ct(cplx<T>* sm, int is, int u, int nthr,
   });
 }
 
-template <typename T, typename P, typename F>
+template <typename T, typename P, typename F, bool INV = false>
 __device__ __forceinline__ void run_fft_fused_ct(cplx<T>* sm, int is, int u, int nthr,
                                                  const cplx<T>* __restrict__ tw, F& mid) {
   constexpr int EM = RegBudget<T>::value;
   cplx<T> v[EM];
   static_for<P::S - 1>([&](auto I) {
     constexpr int st = decltype(I)::value;
-    stockham_stage<P::r[st], false, T, EM>(v, sm, is, P::n, cplan_prefix<P>(st), u, nthr, tw);
+    stockham_stage<P::r[st], INV, T, EM>(v, sm, is, P::n, cplan_prefix<P>(st), u, nthr, tw);
   });
-  fused_middle<P::r[P::S - 1], T, EM>(v, sm, is, P::n, u, nthr, tw, mid);
+  fused_middle<P::r[P::S - 1], INV, T, EM>(v, sm, is, P::n, u, nthr, tw, mid);
   static_for<P::S - 1>([&](auto I) {
     constexpr int st = P::S - 2 - decltype(I)::value;
-    stockham_stage<P::r[st], true, T, EM>(v, sm, is, P::n, cplan_suffix<P>(st + 1), u, nthr, tw);
+    stockham_stage<P::r[st], !INV, T, EM>(v, sm, is, P::n, cplan_suffix<P>(st + 1), u, nthr, tw);
   });
 }
 
@@ -538,9 +620,11 @@ template <bool INV, typename T, typename P>
 __device__ __forceinline__ void fft_plan(cplx<T>* sm, int is, const FFTPlan& pl, int u, int nthr,
                                          const cplx<T>* __restrict__ tw) {
   if constexpr (std::is_same<P, DynPlan>::value)
-    run_fft<INV, T, false>(sm, is, pl, u, nthr, tw);
+    run_fft<INV, T>(sm, is, pl, u, nthr, tw);
   else if constexpr (std::is_same<P, DynPlanX>::value)
-    run_fft<INV, T, true>(sm, is, pl, u, nthr, tw);
+    run_fft<INV, T, kRadixExt>(sm, is, pl, u, nthr, tw);
+  else if constexpr (std::is_same<P, DynPlan9>::value)
+    run_fft<INV, T, kRadixSmall>(sm, is, pl, u, nthr, tw);
   else
     run_fft_ct<INV, T, P>(sm, is, u, nthr, tw);
 }
@@ -549,11 +633,25 @@ template <typename T, typename P, typename F>
 __device__ __forceinline__ void fft_fused_plan(cplx<T>* sm, int is, const FFTPlan& pl, int u, int nthr,
                                                const cplx<T>* __restrict__ tw, F& mid) {
   if constexpr (std::is_same<P, DynPlan>::value)
-    run_fft_fused<T, F, false>(sm, is, pl, u, nthr, tw, mid);
+    run_fft_fused<T, F>(sm, is, pl, u, nthr, tw, mid);
   else if constexpr (std::is_same<P, DynPlanX>::value)
-    run_fft_fused<T, F, true>(sm, is, pl, u, nthr, tw, mid);
+    run_fft_fused<T, F, kRadixExt>(sm, is, pl, u, nthr, tw, mid);
   else
     run_fft_fused_ct<T, P>(sm, is, u, nthr, tw, mid);
+}
+
+// The same with the inverse transform first: inverse, pointwise, forward.
+template <typename T, typename P, typename F>
+__device__ __forceinline__ void fft_mirror_plan(cplx<T>* sm, int is, const FFTPlan& pl, int u, int nthr,
+                                                const cplx<T>* __restrict__ tw, F& mid) {
+  if constexpr (std::is_same<P, DynPlan>::value)
+    run_fft_fused<T, F, kRadixStd, true>(sm, is, pl, u, nthr, tw, mid);
+  else if constexpr (std::is_same<P, DynPlanX>::value)
+    run_fft_fused<T, F, kRadixExt, true>(sm, is, pl, u, nthr, tw, mid);
+  else if constexpr (std::is_same<P, DynPlan9>::value)
+    run_fft_fused<T, F, kRadixSmall, true>(sm, is, pl, u, nthr, tw, mid);
+  else
+    run_fft_fused_ct<T, P, F, true>(sm, is, u, nthr, tw, mid);
 }
 
 // The plans the planner picks for the 3^7 = 2187 axis (81 threads), the

@@ -75,9 +75,12 @@ template <> struct PlanLen<DynPlan> {
 template <> struct PlanLen<DynPlanX> {
   static constexpr int value = 0;
 };
+template <> struct PlanLen<DynPlan9> {
+  static constexpr int value = 0;
+};
 // Axis length of a plan: a constant for compile-time plans.
 template <typename PS> __device__ __forceinline__ int plan_len(const FFTPlan& pl) {
-  if constexpr (std::is_same<PS, DynPlan>::value || std::is_same<PS, DynPlanX>::value)
+  if constexpr (PlanLen<PS>::value == 0)
     return pl.n;
   else
     return PS::n;
@@ -129,6 +132,9 @@ struct Scal {
   // buffer) while xpend is 1.
   double alpha_x;
   int xpend;
+  // frequency-domain CG (fh_spectral.cuh): alpha and beta as its kernels use them
+  float alpha_f, beta_f;
+  double ib2;      // 1 / b2
 };
 
 // kStalled: the recursive residual stopped decreasing (the working precision's

@@ -5,6 +5,7 @@
 #pragma once
 
 #include "fh_kernels.cuh"
+#include "fh_spectral.cuh"
 
 namespace fh {
 
@@ -43,6 +44,24 @@ struct LaunchTable {
   int (*ct_plan)(const FFTPlan& prow, const Launch& row, const FFTPlan& pc0, const Launch& col0,
                  const FFTPlan& pc1, const Launch& col1) = nullptr;
 };
+
+// Launchers of the frequency-domain CG iteration (fh_spectral.cuh, float32;
+// fh_spec_*.cu).  *_smem raise the shared-memory limit of the kernels these
+// arguments run; *_ct: does a compile-time plan kernel run the iteration's
+// pass with this plan and launch?
+cudaError_t spec_inv(int mode, const Launch&, const SpecArgs&, cudaStream_t);
+cudaError_t spec_fwd(int mode, const Launch&, const SpecArgs&, cudaStream_t);
+cudaError_t spec_col_set_smem(const SpecArgs&, size_t bytes);
+bool spec_col_ct(const FFTPlan&);
+cudaError_t spec_mid(bool inv, const Launch&, const SpecMidArgs&, cudaStream_t);
+cudaError_t spec_mid_set_smem(const SpecMidArgs&, size_t bytes);
+bool spec_mid_ct(const FFTPlan&);
+cudaError_t spec_row_d2(int mode, const Launch&, const SpecRowArgs&, cudaStream_t);
+cudaError_t spec_row_d3(int mode, const Launch&, const SpecRowArgs&, cudaStream_t);
+cudaError_t spec_row_d2_set_smem(const SpecRowArgs&, const Launch&);
+cudaError_t spec_row_d3_set_smem(const SpecRowArgs&, const Launch&);
+bool spec_row_d2_ct(const FFTPlan&, const Launch&);
+bool spec_row_d3_ct(const FFTPlan&, const Launch&);
 
 // Supported (D, NL): (2, 1), (2, 2), (3, 1), (3, 3).
 LaunchTable<float> launch_table_f32_d2(int nl);

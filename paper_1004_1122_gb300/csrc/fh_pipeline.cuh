@@ -153,7 +153,9 @@ struct Pipeline {
   // Time the CG-iteration pass kernels for candidate tunings (temporary
   // pipelines) and return the fastest; `ms` receives its time per iteration.
   static int autotune(const Problem& pb, int nloads, cudaStream_t stream, Tuning& best, double& ms,
-                      std::string& err, int max_candidates = 256);
+                      std::string& err, int max_candidates = 256, bool want_spectral = false);
+  // device time of one CG iteration's kernels (what autotune compares)
+  int iteration_time(double* ms, std::string& err);
   void release();
   bool device_error() const { return h_err != nullptr && *h_err != 0; }
   void set_phase(const uint8_t* d_phase) { phase = d_phase; }
@@ -194,6 +196,32 @@ struct Pipeline {
   int* d_loop = nullptr;     // device [2]: rounds run by the device-side loop, round limit
   int* h_loop = nullptr;     // pinned host mirror
   LoopCache loops;           // this pipeline's own device-side loop graphs (solve)
+  // Frequency-domain CG (fh_spectral.cuh): float32 pipelines whose owner asks
+  // for it before init (want_spectral) run CG solves without per-iteration
+  // norms through it.  x stays the field; the iteration's scalar arrays live in
+  // the r, p, ap and p2 buffers.
+  bool want_spectral = false;
+  bool spectral = false;
+  bool spec_run_ = false;      // the solve in progress uses it
+  SpecGeom sg{};
+  FFTPlan sprow{}, spcol{}, spmid{};
+  int stpl = 0, stpc = 0, stpm = 0, slpc = 0;
+  Launch scol{}, smid{}, srow{};
+  T* S2 = nullptr;             // 3-D: two-channel spectrum
+  SpecMedium* smed = nullptr;  // reference medium per cell
+  int init_spectral(const Problem& pb, std::string& err);
+  SpecArgs spec_args() const;
+  SpecRowArgs spec_row_args() const;
+  SpecMidArgs spec_mid_args() const;
+  cudaError_t spec_passes();   // one iteration's passes
+  cudaError_t spec_iter();     // ... and its scalars
+  cudaError_t spec_middle(bool inv, Scal* sc);
+  cudaError_t spec_rows(int mode, const SpecRowArgs& a);
+  cudaError_t spec_load_r();   // r: real residual fields -> scalars, in place
+  cudaError_t spec_finish();   // x += the field of the accumulated correction
+  // |M p|^2 of the last direction (single-cell, one load)
+  int spec_dir_norm2(const double* M, double* out, std::string& err);
+
   // Capture `K` iterations of `method` followed by the loop condition into
   // `body`, the body graph of a while node with handle h (on this pipeline's
   // stream).  *kernels receives the kernels one body launches.
@@ -205,6 +233,8 @@ struct Pipeline {
   cudaError_t enqueue_iter(int method, int j = 0);
   // CG items that stopped with an x step owed receive it (after the loop)
   cudaError_t enqueue_x_flush();
+  bool has_after_loop() const { return defer_x_ || spec_run_; }
+  cudaError_t enqueue_after_loop() { return spec_run_ ? spec_finish() : enqueue_x_flush(); }
   // eta_e (Eq. errE_def) of the current iterate x[0] into hist_eta_e[iter]
   cudaError_t enqueue_eta_record();
   int chunk_size(int method) const;
@@ -232,6 +262,7 @@ struct Pipeline {
   // back-to-back launches of one piece of the CG iteration:
   // 0 row_fwd (direction update + dL + FFT), 1 column passes (Green),
   // 2 row_inv (inverse FFT + A p + dot), 3 CG vector update, 5 operator apply.
+  static constexpr int kProfileSpectral = 6;  // internal: the passes of one frequency-domain iteration
   int profile(int what, int reps, double* ms, std::string& err);
 };
 

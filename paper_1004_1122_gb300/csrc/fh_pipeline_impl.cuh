@@ -346,6 +346,255 @@ int Pipeline<T>::init(const Problem& pb, int nloads_, bool krylov, cudaStream_t 
       if ((rc = dev_alloc(allocs, &rhs[l], vlen, err))) return rc;
     }
   }
+  return want_spectral && krylov ? init_spectral(pb, err) : 0;
+}
+
+// Launch shapes and buffers of the frequency-domain CG iteration.  Left off
+// (spectral = false) where a tile or line does not fit one CTA.
+template <typename T>
+int Pipeline<T>::init_spectral(const Problem& pb, std::string& err) {
+  if constexpr (std::is_same<T, float>::value) {
+    const int d = g.d, nl = nloads;
+    int dev = 0, optin = 0;
+    FH_CKS(cudaGetDevice(&dev));
+    FH_CKS(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    const size_t cap = (size_t)optin - 4096;
+    const int inner = d == 2 ? ncell : g.n1;
+    // Plans: 27 values per thread where a compile-time plan exists or the pass
+    // fills the SMs that way, else 9 values (more threads per FFT, shorter
+    // serial chains).
+    auto plan = [&](int n, long long seqs, int tile_seqs, int maxthr, bool (*has_ct)(const FFTPlan&), FFTPlan& pl,
+                    int& thr) -> bool {
+      if (!make_fft_plan(n, false, maxthr, pl, thr)) return false;
+      const bool small = !has_ct(pl) && seqs * thr < (long long)sms * 1024;
+      FFTPlan p9;
+      int t9;
+      if (small && make_fft_plan(n, false, maxthr, p9, t9, 0, true) && t9 * tile_seqs <= maxthr) {
+        pl = p9;
+        thr = t9;
+      }
+      return true;
+    };
+    const int minC = nl == 2 ? 1 : 2;  // at least one 32-byte sector of every line per column tile
+    if (!plan(g.nlast, d == 2 ? (long long)g.nlines * nl : (long long)(g.nlines + 1) / 2 * d * nl,
+              d == 2 ? nl : d * nl, kRowMaxThreads, d == 2 ? spec_col_ct : spec_mid_ct, sprow,
+              stpl) ||
+        !plan(g.n[0], (long long)g.H * inner * 2 * nl, minC * 2 * nl, kColMaxThreads, spec_col_ct, spcol, stpc) ||
+        (d == 3 && !plan(g.n1, (long long)g.H * g.n[0] * 3 * nl, minC * 3 * nl, kColMaxThreads, spec_mid_ct, spmid, stpm)))
+      return 0;
+    // Column tiles: the widest that leaves four CTAs per SM and fits 48 KB
+    auto fits = [&](int C, size_t smem) {
+      return (size_t)g.n[0] * C * 2 * nl * sizeof(float2) <= smem && C * 2 * nl * stpc <= kColMaxThreads &&
+             (d == 2 || ((size_t)g.n1 * C * 3 * nl * sizeof(float2) <= smem && C * 3 * nl * stpm <= kColMaxThreads));
+    };
+    int Cc = minC;
+    for (int cand : {16, 8, 4, 2})
+      if (cand > minC && fits(cand, 48 * 1024) && (long long)((g.H + cand - 1) / cand) * inner >= 4LL * sms) {
+        Cc = cand;
+        break;
+      }
+    if (!fits(Cc, cap)) return 0;
+    sg.C = Cc;
+    sg.csh = 0;
+    while ((1 << sg.csh) < Cc) ++sg.csh;
+    sg.Tt = (g.H + Cc - 1) / Cc;
+    if (sg.Tt * Cc % 2) ++sg.Tt;  // 16-byte aligned lines
+    sg.Hp = sg.Tt * Cc;
+    for (int k = 0; k < 3; ++k) sg.invY[k] = (float)g.invY[k];
+    sg.inv_nodes = (float)g.inv_nodes;
+    scol.block = round_up(std::max(64, Cc * 2 * nl * stpc), 32);
+    scol.grid = sg.Tt * inner;
+    scol.smem = spec_col_smem(g.n[0], Cc * 2 * nl, 2 * nl, scol.block);
+    if (d == 3) {
+      smid.block = round_up(std::max(64, Cc * 3 * nl * stpm), 32);
+      smid.grid = sg.Tt * g.n[0];
+      smid.smem = (size_t)g.n1 * Cc * 3 * nl * sizeof(float2);
+    }
+    // Lines per CTA: about 96 threads, two CTAs per SM where the grid has them
+    const int unit = d == 2 ? 1 : 2, seq = d == 2 ? nl : d * nl;  // lines and sequences that belong together
+    int k = std::max(1, 96 / (seq * stpl));
+    k = std::min<int>(k, std::max(1, g.nlines / (unit * 2 * sms)));
+    while (k > 1 && ((ncell > 1 && g.lines_cell % (k * unit)) || spec_row_smem(d, nl, k * unit, g.nlast, nphase) > 64 * 1024)) --k;
+    slpc = k * unit;
+    srow.block = round_up(std::max(32, k * seq * stpl), 32);
+    srow.grid = (g.nlines + slpc - 1) / slpc;
+    srow.smem = spec_row_smem(d, nl, slpc, g.nlast, nphase);
+    if (srow.smem > cap || srow.block > 768 || scol.smem > cap) return 0;
+    const bool more_part = scol.grid > part_stride;
+    part_stride = std::max(part_stride, scol.grid);
+    FH_CKS(spec_col_set_smem(spec_args(), scol.smem));
+    if (d == 3) FH_CKS(spec_mid_set_smem(spec_mid_args(), smid.smem));
+    FH_CKS(d == 2 ? spec_row_d2_set_smem(spec_row_args(), srow) : spec_row_d3_set_smem(spec_row_args(), srow));
+    int rc;
+    const size_t lines = (size_t)sg.Hp * g.nlines;
+    // the operator's own spectrum buffer may be smaller than the padded lines
+    if (lines * d * nl > (size_t)g.Tt * g.C * g.nlines * g.M && (rc = dev_alloc(allocs, &S, lines * d * nl, err))) return rc;
+    if (d == 3) {
+      C* buf = nullptr;
+      if ((rc = dev_alloc(allocs, &buf, lines * 2 * nl, err))) return rc;
+      S2 = reinterpret_cast<T*>(buf);
+    }
+    {
+      std::vector<SpecMedium> hm(ncell);
+      for (int c = 0; c < ncell; ++c) {
+        const double* L = pb.L0cell.empty() ? g.L0 : &pb.L0cell[9 * c];
+        SpecMedium& m = hm[c];
+        m.L00 = (float)L[0];
+        m.L11 = (float)L[4];
+        m.L22 = (float)L[8];
+        m.s01 = (float)(L[1] + L[3]);
+        m.s02 = (float)(L[2] + L[6]);
+        m.s12 = (float)(L[5] + L[7]);
+        bool iso = true;
+        for (int i = 0; i < d; ++i)
+          for (int j = 0; j < d; ++j) iso = iso && L[3 * i + j] == (i == j ? L[0] : 0.0);
+        m.iso = iso ? 1.0f : 0.0f;
+        m.scale = (float)(iso ? g.inv_nodes / L[0] : g.inv_nodes);
+      }
+      if ((rc = dev_alloc(allocs, &smed, ncell, err))) return rc;
+      FH_CKS(cudaMemcpy(smed, hm.data(), ncell * sizeof(SpecMedium), cudaMemcpyHostToDevice));
+    }
+    if (more_part && (rc = dev_alloc(allocs, &part, (size_t)3 * kMaxLoads * part_stride, err))) return rc;
+    for (int l = 0; l < nl; ++l)
+      if ((rc = dev_alloc(allocs, &p2[l], vlen, err))) return rc;
+    if (2 * lines > (size_t)vlen)  // padded scalar arrays do not fit the field buffers
+      for (int l = 0; l < nl; ++l)
+        for (T** b : {&r[l], &p[l], &ap[l], &p2[l]})
+          if ((rc = dev_alloc(allocs, b, 2 * lines, err))) return rc;
+    // the passes of an iteration all run compile-time plans of one length
+    const bool ct = (d == 2 ? spec_row_d2_ct(sprow, srow) : spec_row_d3_ct(sprow, srow)) && spec_col_ct(spcol) &&
+                    (d == 2 || spec_mid_ct(spmid));
+    ct_plan = ct && sprow.n == spcol.n && (d == 2 || spmid.n == sprow.n) ? sprow.n : 0;
+    spectral = true;
+  }
+  return 0;
+}
+
+template <typename T>
+SpecArgs Pipeline<T>::spec_args() const {
+  SpecArgs a;
+  std::memset(&a, 0, sizeof(a));
+  a.g = g;
+  a.sg = sg;
+  a.plan = spcol;
+  a.tpc = stpc;
+  a.nb_inner = g.d == 2 ? ncell : g.n1;
+  a.tw = reinterpret_cast<const float2*>(tw0);
+  a.S = g.d == 3 ? reinterpret_cast<float2*>(S2) : reinterpret_cast<float2*>(S);
+  for (int l = 0; l < nloads; ++l) {
+    a.r[l] = reinterpret_cast<float2*>(r[l]);
+    a.p[l] = reinterpret_cast<float2*>(p[l]);
+    a.ap[l] = reinterpret_cast<float2*>(ap[l]);
+    a.x[l] = reinterpret_cast<float2*>(p2[l]);
+  }
+  a.scal = scal;
+  a.nl = nloads;
+  a.three = g.d == 3;
+  a.part = reinterpret_cast<float2*>(part);
+  a.med = smed;
+  return a;
+}
+
+template <typename T>
+SpecRowArgs Pipeline<T>::spec_row_args() const {
+  SpecRowArgs a;
+  std::memset(&a, 0, sizeof(a));
+  a.g = g;
+  a.sg = sg;
+  a.plan = sprow;
+  a.tpl = stpl;
+  a.lpc = slpc;
+  a.tw = reinterpret_cast<const float2*>(tw_last);
+  a.S = reinterpret_cast<float2*>(S);
+  a.phase = phase;
+  a.tab = reinterpret_cast<const float*>(dtab);
+  a.nphase = nphase;
+  a.scal = scal;
+  return a;
+}
+
+template <typename T>
+SpecMidArgs Pipeline<T>::spec_mid_args() const {
+  SpecMidArgs m;
+  std::memset(&m, 0, sizeof(m));
+  m.g = g;
+  m.sg = sg;
+  m.plan = spmid;
+  m.tpc = stpm;
+  m.nl = nloads;
+  m.tw = reinterpret_cast<const float2*>(tw1);
+  m.S2 = reinterpret_cast<float2*>(S2);
+  m.S3 = reinterpret_cast<float2*>(S);
+  return m;
+}
+
+template <typename T>
+cudaError_t Pipeline<T>::spec_middle(bool inv, Scal* sc) {
+  if (g.d != 3) return cudaSuccess;
+  SpecMidArgs m = spec_mid_args();
+  m.scal = sc;
+  ++launches;
+  return spec_mid(inv, smid, m, st);
+}
+
+template <typename T>
+cudaError_t Pipeline<T>::spec_rows(int mode, const SpecRowArgs& a) {
+  ++launches;
+  return g.d == 2 ? spec_row_d2(mode, srow, a, st) : spec_row_d3(mode, srow, a, st);
+}
+
+template <typename T>
+cudaError_t Pipeline<T>::spec_passes() {
+  launches += 2;
+  FH_CK(spec_inv(kSpecUpdate, scol, spec_args(), st));
+  FH_CK(spec_middle(true, scal));
+  FH_CK(spec_rows(kSpecRowTau, spec_row_args()));
+  FH_CK(spec_middle(false, scal));
+  return spec_fwd(kSpecApply, scol, spec_args(), st);
+}
+
+template <typename T>
+cudaError_t Pipeline<T>::spec_iter() {
+  FH_CK(spec_passes());
+  ++launches;
+  k_scal_spec<<<item_blocks(items), kSpecScalThreads, 0, st>>>(
+      scal, reinterpret_cast<const float2*>(part), scol.grid, ncell, nloads, (double)g.cell_nodes);
+  return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t Pipeline<T>::spec_load_r() {
+  SpecRowArgs a = spec_row_args();
+  for (int l = 0; l < nloads; ++l) a.f[l] = reinterpret_cast<float*>(r[l]);
+  FH_CK(spec_rows(kSpecRowLoad, a));
+  FH_CK(spec_middle(false, nullptr));
+  ++launches;
+  return spec_fwd(kSpecProject, scol, spec_args(), st);
+}
+
+template <typename T>
+cudaError_t Pipeline<T>::spec_finish() {
+  ++launches;
+  FH_CK(spec_inv(kSpecFinish, scol, spec_args(), st));
+  FH_CK(spec_middle(true, nullptr));
+  SpecRowArgs a = spec_row_args();
+  for (int l = 0; l < nloads; ++l) a.f[l] = reinterpret_cast<float*>(x[l]);
+  return spec_rows(kSpecRowAdd, a);
+}
+
+template <typename T>
+int Pipeline<T>::spec_dir_norm2(const double* Mx, double* out, std::string& err) {
+  Mat3 m;
+  for (int i = 0; i < 9; ++i) m.v[i] = Mx[i];
+  ++launches;
+  k_spec_matnorm2<<<scol.grid, 256, 0, st>>>(spec_args(), m, part);
+  FH_CKS(cudaGetLastError());
+  ++launches;
+  k_reduce_items<<<1, kRedThreads, 0, st>>>(part, scol.grid, 1, 1, d_red);
+  FH_CKS(cudaGetLastError());
+  FH_CKS(cudaMemcpyAsync(h_red, d_red, sizeof(double), cudaMemcpyDeviceToHost, st));
+  FH_CKS(cudaStreamSynchronize(st));
+  *out = h_red[0] * (double)g.nodes;
   return 0;
 }
 
@@ -462,6 +711,7 @@ int Pipeline<T>::chunk_size(int method) const {
 
 template <typename T>
 cudaError_t Pipeline<T>::enqueue_iter(int method, int j) {
+  if (spec_run_) return spec_iter();
   RowArgs<T> a = row_args();
   a.scal = scal;
   if (method == kCG) {
@@ -802,7 +1052,7 @@ static int run_loops_host(Pipeline<T>* const* ps, int np, std::string& err) {
   }
   for (int i = 0; i < np && e == cudaSuccess; ++i) {
     Pipeline<T>& P = *ps[i];
-    if (P.defer_x_) e = P.enqueue_x_flush();
+    if (P.has_after_loop()) e = P.enqueue_after_loop();
     if (e == cudaSuccess) e = cudaMemcpyAsync(P.h_err, P.dev_err, sizeof(int), cudaMemcpyDeviceToHost, P.st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(P.st);
   }
@@ -827,7 +1077,7 @@ int run_loops(Pipeline<T>* const* ps, int np, cudaStream_t launch, LoopCache& ca
     const Pipeline<T>& P = *ps[i];
     key += std::to_string(P.uid) + ":" + std::to_string(P.run_method_) + ":" +
            std::to_string(P.run_K_) + ":" + (P.rhs_active_ ? "r" : "c") +
-           (P.hist_eta_e || P.hist_eta_r ? "h" : "-") + ";";
+           (P.hist_eta_e || P.hist_eta_r ? "h" : "-") + (P.spec_run_ ? "s;" : ";");
   }
   auto it = cache.exec.find(key);
   if (it == cache.exec.end()) {
@@ -847,18 +1097,19 @@ int run_loops(Pipeline<T>* const* ps, int np, cudaStream_t launch, LoopCache& ca
       e = cudaGraphAddNode(&node, g, nullptr, nullptr, 0, &cp);
       if (e != cudaSuccess) break;
       e = ps[i]->capture_loop_body(cp.conditional.phGraph_out[0], h, ps[i]->run_method_, ps[i]->run_K_, &kern[i]);
-      if (e == cudaSuccess && ps[i]->defer_x_) {
-        // after the loop: the x step owed by items that stopped on an even iteration
+      if (e == cudaSuccess && ps[i]->has_after_loop()) {
+        // after the loop: the x step owed by items that stopped on an even iteration,
+        // or the field of a frequency-domain solve's correction
         Pipeline<T>& P = *ps[i];
         e = cudaStreamBeginCaptureToGraph(P.st, g, &node, nullptr, 1, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) break;
         const long long before = P.launches;
-        e = P.enqueue_x_flush();
+        e = P.enqueue_after_loop();
+        kern[np + i] = P.launches - before;
         P.launches = before;
         cudaGraph_t out = nullptr;
         const cudaError_t e2 = cudaStreamEndCapture(P.st, &out);
         if (e == cudaSuccess) e = e2;
-        kern[np + i] = 1;
       }
     }
     cudaGraphExec_t exec = nullptr;
@@ -942,7 +1193,8 @@ int Pipeline<T>::solve_begin(int method, const double (*E)[kMaxD], bool rhs_fiel
       if ((rc = dev_alloc(allocs, &atps[l], vlen, err))) return rc;
     }
   }
-  defer_x_ = method == kCG && !(hist_eta_e != nullptr && items == 1);
+  spec_run_ = spectral && method == kCG && hist_eta_e == nullptr && hist_eta_r == nullptr;
+  defer_x_ = method == kCG && !spec_run_ && !(hist_eta_e != nullptr && items == 1);
   if (defer_x_ && p2[0] == nullptr) {
     for (int l = 0; l < nloads; ++l)
       if ((rc = dev_alloc(allocs, &p2[l], vlen, err))) return rc;
@@ -967,6 +1219,7 @@ int Pipeline<T>::solve_begin(int method, const double (*E)[kMaxD], bool rhs_fiel
     Scal& s = h_scal[it];
     std::memset(&s, 0, sizeof(Scal));
     s.b2 = b2[it] > 0.0 ? b2[it] : 1.0;
+    s.ib2 = 1.0 / s.b2;
     const double tl = tol_item ? tol_item[it] : tol;
     s.tol2 = tl * tl;
     s.max_iter = max_iter;
@@ -1025,7 +1278,8 @@ int Pipeline<T>::solve_begin(int method, const double (*E)[kMaxD], bool rhs_fiel
       k_scal_start<<<item_blocks(items), kRedThreads, 0, st>>>(scal, part, row.grid, ncell, nloads);
     }
     FH_CKS(cudaGetLastError());
-    for (int l = 0; l < nloads; ++l) {
+    if (spec_run_) FH_CKS(spec_load_r());
+    for (int l = 0; l < nloads && !spec_run_; ++l) {
       FH_CKS(cudaMemsetAsync(p[l], 0, vbytes, st));
       if (defer_x_) FH_CKS(cudaMemsetAsync(p2[l], 0, vbytes, st));  // the first iteration's previous p
       if (method == kBiCG) {
@@ -1043,7 +1297,7 @@ int Pipeline<T>::solve_begin(int method, const double (*E)[kMaxD], bool rhs_fiel
 
 template <typename T>
 int Pipeline<T>::autotune(const Problem& pb, int nloads_, cudaStream_t stream, Tuning& best,
-                          double& best_ms, std::string& err, int max_candidates) {
+                          double& best_ms, std::string& err, int max_candidates, bool want_spectral) {
   const bool f64 = sizeof(T) == 8;
   const int d = pb.d;
   const int nlast = pb.N[d - 1];
@@ -1092,6 +1346,7 @@ int Pipeline<T>::autotune(const Problem& pb, int nloads_, cudaStream_t stream, T
   for (const Tuning& c : cands) {
     if (tried >= max_candidates) break;
     Pipeline<T> trial;
+    trial.want_spectral = want_spectral;
     if (trial.init(pb, nloads_, true, stream, e2, &c) != 0) {
       trial.release();
       continue;
@@ -1103,10 +1358,8 @@ int Pipeline<T>::autotune(const Problem& pb, int nloads_, cudaStream_t stream, T
     ++tried;
     double total = 0.0, t;
     bool ok = true;
-    for (int what = 0; what < 4 && ok; ++what) {
-      if (trial.profile(what, 10, &t, e2) != 0) ok = false;
-      total += t;
-    }
+    if (trial.iteration_time(&t, e2) != 0) ok = false;
+    total = t;
     trial.release();
     if (ok && total < best_ms) {
       best_ms = total;
@@ -1116,6 +1369,19 @@ int Pipeline<T>::autotune(const Problem& pb, int nloads_, cudaStream_t stream, T
   if (best_ms >= 1e30) {
     err = "autotune: no candidate could be timed";
     return 9;
+  }
+  return 0;
+}
+
+template <typename T>
+int Pipeline<T>::iteration_time(double* ms, std::string& err) {
+  if (spectral) return profile(kProfileSpectral, 10, ms, err);
+  *ms = 0.0;
+  for (int what = 0; what < 4; ++what) {
+    double t = 0.0;
+    const int rc = profile(what, 10, &t, err);
+    if (rc) return rc;
+    *ms += t;
   }
   return 0;
 }
@@ -1134,6 +1400,7 @@ int Pipeline<T>::profile(int what, int reps, double* ms, std::string& err) {
     s.beta = 0.5;
     s.b2 = 1.0;
     s.max_iter = 1 << 30;
+    s.iter = 1;
   }
   FH_CKS(cudaMemcpyAsync(scal, h_scal, items * sizeof(Scal), cudaMemcpyHostToDevice, st));
   const size_t vbytes = (size_t)vlen * sizeof(T);
@@ -1179,6 +1446,7 @@ int Pipeline<T>::profile(int what, int reps, double* ms, std::string& err) {
       case 2: return launch_row_inv(kEpiDir, i);
       case 3: ++launches; return lt.cg_update(vec, v, st);
       case 5: return passes(kProApply, kEpiApply, app, app, nullptr);
+      case kProfileSpectral: return spectral ? spec_passes() : cudaErrorInvalidValue;
       default: return cudaErrorInvalidValue;
     }
   };

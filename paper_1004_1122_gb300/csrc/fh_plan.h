@@ -91,11 +91,13 @@ inline std::vector<int> plan_radices(int n, int tpl, int budget) {
 // sequence (more butterflies per thread, more independent work in flight).
 // Even lengths and lengths with a prime factor 11, 13 or 17 get an extended
 // plan (pl.ext = 1).
+// small: a plan over the small radix set (lengths that need no extended one).
 inline bool make_fft_plan(int n, bool fp64, int max_tpl, FFTPlan& pl, int& tpl,
-                          int force_tpl = 0) {
+                          int force_tpl = 0, bool small = false) {
   bool ext;
   if (!factorable(n, ext)) return false;
-  const int budget = ext ? reg_budget_x(fp64) : reg_budget(fp64);
+  small = small && !ext;
+  const int budget = small ? kSmallBudget : ext ? reg_budget_x(fp64) : reg_budget(fp64);
   int best_stages = 1 << 30, best_tpl = 0;
   std::vector<int> best_r;
   for (int t = 1; t <= max_tpl; ++t) {
@@ -112,7 +114,7 @@ inline bool make_fft_plan(int n, bool fp64, int max_tpl, FFTPlan& pl, int& tpl,
   pl.n = n;
   pl.nstages = (int)best_r.size();
   for (int s = 0; s < kMaxStages; ++s) pl.radix[s] = s < pl.nstages ? best_r[s] : 0;
-  pl.ext = ext ? 1 : 0;
+  pl.ext = ext ? kRadixExt : small ? kRadixSmall : kRadixStd;
   tpl = best_tpl;
   return true;
 }
