@@ -17,9 +17,13 @@
 //  * stage<R>() is one Stockham autosort pass over a sequence held in shared
 //    memory: butterfly j reads x[j + r n/R], applies the twiddles
 //    W_{Ns R}^{r (j mod Ns)}, transforms, and writes x[(j - j mod Ns) R + j mod Ns + r Ns]
-//    (Ns = product of the radices already applied).  Stage twiddles come from
-//    a per-length table tw[m] = exp(-2 pi i m / n) built on the host in
-//    float64.
+//    (Ns = product of the radices already applied).  The twiddles of a stage
+//    lie together, [(r - 1) Ns + k] = exp(-2 pi i r k / (Ns R)), so that the
+//    threads of a warp read consecutive entries (from one table of n roots
+//    their reads are strided by r n / (Ns R): 27 cache lines per warp instead
+//    of 2 in the second radix-27 stage).  A plan's table holds its stages in
+//    order (n - radix[0] entries), then those of the reversed radix order
+//    (n - radix[last] entries); both are built on the host in float64.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -319,7 +323,6 @@ __device__ __forceinline__ void stockham_stage(cplx<T> (&v)[EM], cplx<T>* sm, in
   constexpr int BM = EM / R;
   static_assert(BM >= 1, "radix exceeds the register budget");
   const int nb = n / R;
-  const int S = nb / Ns;
   const int in_step = nb * is, out_step = Ns * is;
   // j = u + b * nthr = q * Ns + k, advanced without divisions
   const int dq = nthr / Ns, dk = nthr - dq * Ns;
@@ -345,12 +348,10 @@ __device__ __forceinline__ void stockham_stage(cplx<T> (&v)[EM], cplx<T>* sm, in
 #pragma unroll
       for (int r = 0; r < R; ++r) v[b * R + r] = src[r * in_step];
       if (Ns > 1) {
-        const int ks = kb[b] * S;
-        int ti = ks;
+        const C* const tk = tw + kb[b];
 #pragma unroll
         for (int r = 1; r < R; ++r) {
-          const C w = ld_tw(tw + ti);
-          ti += ks;
+          const C w = ld_tw(tk + (r - 1) * Ns);
           v[b * R + r] = INV ? cmulc(v[b * R + r], w) : cmul(v[b * R + r], w);
         }
       }
@@ -437,6 +438,7 @@ __device__ __forceinline__ void run_fft(cplx<T>* sm, int is, const FFTPlan& pl, 
       }
     }
 #undef FH_STAGE_CASE
+    if (s > 0) tw += (R - 1) * Ns;
     Ns *= R;
   }
 }
@@ -465,12 +467,10 @@ __device__ __forceinline__ void fused_middle(cplx<T> (&v)[EM], cplx<T>* sm, int 
 #pragma unroll
       for (int r = 0; r < R; ++r) v[b * R + r] = src[r * in_step];
       if (nb > 1) {
-        int ti = j;
 #pragma unroll
         for (int r = 1; r < R; ++r) {
-          const C w = ld_tw(tw + ti);
+          const C w = ld_tw(tw + j + (r - 1) * nb);
           v[b * R + r] = INV ? cmulc(v[b * R + r], w) : cmul(v[b * R + r], w);
-          ti += j;
         }
       }
       RegDFT<R, 1, INV, T>::run(&v[b * R]);
@@ -504,6 +504,7 @@ __device__ __forceinline__ void run_fft_fused(cplx<T>* sm, int is, const FFTPlan
   cplx<T> v[EM];
   const int S = pl.nstages;
   int Ns = 1;
+  const cplx<T>* const twr = tw + (pl.n - pl.radix[0]);  // the reversed order's stages
 #define FH_SWITCH(R, CASE)             \
   if constexpr (SET == kRadixExt) {    \
     switch (R) {                       \
@@ -528,6 +529,7 @@ __device__ __forceinline__ void run_fft_fused(cplx<T>* sm, int is, const FFTPlan
     break;
     FH_SWITCH(pl.radix[s], FH_STAGE_CASE)
 #undef FH_STAGE_CASE
+    if (s > 0) tw += (pl.radix[s] - 1) * Ns;
     Ns *= pl.radix[s];
   }
 #define FH_MID_CASE(RR)                                                              \
@@ -537,6 +539,7 @@ __device__ __forceinline__ void run_fft_fused(cplx<T>* sm, int is, const FFTPlan
   FH_SWITCH(pl.radix[S - 1], FH_MID_CASE)
 #undef FH_MID_CASE
   Ns = pl.radix[S - 1];
+  tw = twr;
   for (int s = S - 2; s >= 0; --s) {
 #define FH_STAGE_CASE(RR)                                                                         \
   case RR:                                                                                        \
@@ -544,6 +547,7 @@ __device__ __forceinline__ void run_fft_fused(cplx<T>* sm, int is, const FFTPlan
     break;
     FH_SWITCH(pl.radix[s], FH_STAGE_CASE)
 #undef FH_STAGE_CASE
+    tw += (pl.radix[s] - 1) * Ns;
     Ns *= pl.radix[s];
   }
 #undef FH_SWITCH
@@ -579,6 +583,19 @@ template <typename P> __host__ __device__ constexpr int cplan_suffix(int s) {
   return p;
 }
 
+// Offset of stage s in the plan's twiddle table (order part), and of the stage
+// with radix r[s] in the reversed part.
+template <typename P> __host__ __device__ constexpr int cplan_tw(int s) {
+  int o = 0;
+  for (int i = 1; i < s; ++i) o += (P::r[i] - 1) * cplan_prefix<P>(i);
+  return o;
+}
+template <typename P> __host__ __device__ constexpr int cplan_twr(int s) {
+  int o = P::n - P::r[0];
+  for (int i = P::S - 2; i > s; --i) o += (P::r[i] - 1) * cplan_suffix<P>(i + 1);
+  return o;
+}
+
 // Does the run-time plan pl equal the compile-time plan P?
 template <typename P> inline bool cplan_is(const FFTPlan& pl) {
   if (pl.n != P::n || pl.nstages != P::S) return false;
@@ -595,7 +612,7 @@ __device__ __forceinline__ void run_fft_ct(cplx<T>* sm, int is, int u, int nthr,
     constexpr int st = decltype(I)::value;
     constexpr int R = P::r[st];
     static_assert(R <= EM, "radix exceeds the register budget");
-    stockham_stage<R, INV, T, EM>(v, sm, is, P::n, cplan_prefix<P>(st), u, nthr, tw);
+    stockham_stage<R, INV, T, EM>(v, sm, is, P::n, cplan_prefix<P>(st), u, nthr, tw + cplan_tw<P>(st));
   });
 }
 
@@ -606,12 +623,13 @@ __device__ __forceinline__ void run_fft_fused_ct(cplx<T>* sm, int is, int u, int
   cplx<T> v[EM];
   static_for<P::S - 1>([&](auto I) {
     constexpr int st = decltype(I)::value;
-    stockham_stage<P::r[st], INV, T, EM>(v, sm, is, P::n, cplan_prefix<P>(st), u, nthr, tw);
+    stockham_stage<P::r[st], INV, T, EM>(v, sm, is, P::n, cplan_prefix<P>(st), u, nthr, tw + cplan_tw<P>(st));
   });
-  fused_middle<P::r[P::S - 1], INV, T, EM>(v, sm, is, P::n, u, nthr, tw, mid);
+  fused_middle<P::r[P::S - 1], INV, T, EM>(v, sm, is, P::n, u, nthr, tw + cplan_tw<P>(P::S - 1), mid);
   static_for<P::S - 1>([&](auto I) {
     constexpr int st = P::S - 2 - decltype(I)::value;
-    stockham_stage<P::r[st], !INV, T, EM>(v, sm, is, P::n, cplan_suffix<P>(st + 1), u, nthr, tw);
+    stockham_stage<P::r[st], !INV, T, EM>(v, sm, is, P::n, cplan_suffix<P>(st + 1), u, nthr,
+                                            tw + cplan_twr<P>(st));
   });
 }
 

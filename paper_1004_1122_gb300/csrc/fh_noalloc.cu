@@ -46,7 +46,7 @@ constexpr int kMaxDevices = 64;
 constexpr int kTabEntries = 256 * 9;         // every uint8 phase id, d <= 3
 
 static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
-static __device__ __align__(256) double2 g_tw[3 * kMaxAxis];
+static __device__ __align__(256) double2 g_tw[3 * 2 * kMaxAxis];  // stage twiddles of up to three plans
 static __device__ __align__(256) double g_tab[kTabEntries];
 
 struct DeviceSymbols {
@@ -61,28 +61,37 @@ struct DLTable {
   double v[kTabEntries];
 };
 
-// g_tw[off_k + m] = exp(-2 pi i m / n_k) for the (up to) three axis lengths,
-// back to back; g_tab[i] = dL entry i for i < nt and 0 beyond (phase ids that
+// g_tw: the stage twiddles of the (up to) three plans, back to back (layout in
+// fh_fft.cuh); g_tab[i] = dL entry i for i < nt and 0 beyond (phase ids that
 // have no tensor act as L = L0).
-__global__ void k_fill_tables(int n0, int n1, int n2, DLTable dl, int nt) {
-  const int total = n0 + n1 + n2;
-  const int stride = gridDim.x * blockDim.x;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
-    int m = i, n = n0;
-    if (m >= n0) {
-      m -= n0;
-      n = n1;
-      if (m >= n1) {
-        m -= n1;
-        n = n2;
+struct PlanSet {
+  fh::FFTPlan pl[3];
+  int count;
+};
+
+__global__ void k_fill_tables(PlanSet ps, DLTable dl, int nt) {
+  const int stride = gridDim.x * blockDim.x, first = blockIdx.x * blockDim.x + threadIdx.x;
+  double2* out = g_tw;
+  for (int a = 0; a < ps.count; ++a) {
+    const fh::FFTPlan& pl = ps.pl[a];
+    for (int rev = 0; rev < 2; ++rev) {
+      int Ns = 1;
+      for (int s = 0; s < pl.nstages; ++s) {
+        const int R = pl.radix[rev ? pl.nstages - 1 - s : s];
+        if (s > 0) {
+          for (int i = first; i < (R - 1) * Ns; i += stride) {
+            const int r = i / Ns + 1, k = i - (r - 1) * Ns;
+            double sn, cs;
+            sincospi(2.0 * (double)(r * k) / (double)(Ns * R), &sn, &cs);
+            out[i] = make_double2(cs, -sn);
+          }
+          out += (R - 1) * Ns;
+        }
+        Ns *= R;
       }
     }
-    double sn, cs;
-    sincospi(2.0 * (double)m / (double)n, &sn, &cs);
-    g_tw[i] = make_double2(cs, -sn);
   }
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < kTabEntries; i += stride)
-    g_tab[i] = i < nt ? dl.v[i] : 0.0;
+  for (int i = first; i < kTabEntries; i += stride) g_tab[i] = i < nt ? dl.v[i] : 0.0;
 }
 
 DeviceSymbols g_dev[kMaxDevices];
@@ -303,15 +312,20 @@ extern "C" fh_status fh_apply_noalloc(int d, const int* N, const double* Y, cons
   }
 
   // ---- tables into the static arrays, filled on the device --------------
-  const int lens[3] = {g.nlast, N[0], d == 3 ? N[1] : 0};
-  const int offs[3] = {0, lens[0], lens[0] + lens[1]};
+  PlanSet ps{};
+  ps.pl[0] = prow;
+  ps.pl[1] = pc0;
+  if (d == 3) ps.pl[2] = pc1;
+  ps.count = d;
+  int offs[3] = {0, 0, 0};
+  for (int k = 1; k < 3; ++k) offs[k] = offs[k - 1] + stage_twiddle_count(ps.pl[k - 1]);
   {
     DLTable dl;
     const int nt = nphase * d * d;
     for (int p = 0; p < nphase; ++p)
       for (int i = 0; i < d * d; ++i) dl.v[p * d * d + i] = L[(size_t)p * d * d + i] - L0[i];
     for (int i = nt; i < kTabEntries; ++i) dl.v[i] = 0.0;
-    k_fill_tables<<<8, 256, 0, st>>>(lens[0], lens[1], lens[2], dl, nt);
+    k_fill_tables<<<8, 256, 0, st>>>(ps, dl, nt);
     ce = cudaGetLastError();
     if (ce != cudaSuccess) { set_err(errbuf, errlen, cudaGetErrorString(ce)); return FH_ERR_CUDA; }
   }

@@ -83,6 +83,42 @@ struct LoopCache {
   }
 };
 
+// Device allocations of one pipeline.  Small ones share blocks of 1 MiB: a
+// cudaMalloc costs far more than the kernels that fill such a buffer.
+struct DevPool {
+  std::vector<void*> blocks;
+  char* cur = nullptr;
+  size_t left = 0;
+  void push_back(void* p) { blocks.push_back(p); }
+  void release() {
+    for (void* p : blocks) cudaFree(p);
+    blocks.clear();
+    cur = nullptr;
+    left = 0;
+  }
+  cudaError_t get(void** p, size_t bytes) {
+    constexpr size_t kBlock = 1u << 20, kSmall = 64u << 10;
+    bytes = (bytes + 255) / 256 * 256;
+    if (bytes > kSmall) {
+      const cudaError_t e = cudaMalloc(p, bytes);
+      if (e == cudaSuccess) blocks.push_back(*p);
+      return e;
+    }
+    if (left < bytes) {
+      void* b = nullptr;
+      const cudaError_t e = cudaMalloc(&b, kBlock);
+      if (e != cudaSuccess) return e;
+      blocks.push_back(b);
+      cur = static_cast<char*>(b);
+      left = kBlock;
+    }
+    *p = cur;
+    cur += bytes;
+    left -= bytes;
+    return cudaSuccess;
+  }
+};
+
 template <typename T>
 struct Pipeline {
   using C = cplx<T>;
@@ -138,7 +174,8 @@ struct Pipeline {
   double l0iso = 0.0;          // L0 = l0iso I, or 0 when L0 is not isotropic
   double* eta_bufs[2] = {};    // allocations behind hist_eta_e / hist_eta_r
   cudaStream_t st = nullptr;
-  std::vector<void*> allocs;
+  DevPool allocs;
+  void* h_pinned = nullptr;    // one block behind h_scal, h_red, h_err and h_loop
   Launch vec{};
   LaunchTable<T> lt{};
   int sms = 0;
@@ -156,6 +193,7 @@ struct Pipeline {
                       std::string& err, int max_candidates = 256, bool want_spectral = false);
   // device time of one CG iteration's kernels (what autotune compares)
   int iteration_time(double* ms, std::string& err);
+  template <typename W> int upload_twiddles(const FFTPlan& pl, W** dst, std::string& err);
   void release();
   bool device_error() const { return h_err != nullptr && *h_err != 0; }
   void set_phase(const uint8_t* d_phase) { phase = d_phase; }
@@ -205,7 +243,9 @@ struct Pipeline {
   bool spec_run_ = false;      // the solve in progress uses it
   SpecGeom sg{};
   FFTPlan sprow{}, spcol{}, spmid{};
-  int stpl = 0, stpc = 0, stpm = 0, slpc = 0;
+  int stpl = 0, stpc = 0, stpm = 0, slpc = 0;  // threads per FFT, lines per CTA
+  int ssrow = 0, sscol = 0, ssmid = 0;         // distance of sequences in shared memory
+  float2 *stw_row = nullptr, *stw_col = nullptr, *stw_mid = nullptr;
   Launch scol{}, smid{}, srow{};
   T* S2 = nullptr;             // 3-D: two-channel spectrum
   SpecMedium* smed = nullptr;  // reference medium per cell

@@ -29,14 +29,13 @@ namespace fh {
 static inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
 template <typename T>
-static int dev_alloc(std::vector<void*>& allocs, T** ptr, size_t count, std::string& err) {
+static int dev_alloc(DevPool& allocs, T** ptr, size_t count, std::string& err) {
   void* p = nullptr;
-  cudaError_t e = cudaMalloc(&p, count * sizeof(T) + 16);
+  cudaError_t e = allocs.get(&p, count * sizeof(T) + 16);
   if (e != cudaSuccess) {
     err = std::string("cudaMalloc: ") + cudaGetErrorString(e);
     return 4;  // FH_ERR_OOM
   }
-  allocs.push_back(p);
   *ptr = static_cast<T*>(p);
   return 0;
 }
@@ -257,39 +256,13 @@ int Pipeline<T>::init(const Problem& pb, int nloads_, bool krylov, cudaStream_t 
   int rc;
   const size_t spec = (size_t)g.Tt * g.C * g.nlines * M;
   if ((rc = dev_alloc(allocs, &S, spec, err))) return rc;
-  auto upload_tw = [&](int n, C** dst) -> int {
-    std::vector<double> re, im;
-    twiddles(n, re, im);
-    std::vector<C> h(n);
-    for (int m = 0; m < n; ++m) {
-      h[m].x = T(re[m]);
-      h[m].y = T(im[m]);
-    }
-    int r2 = dev_alloc(allocs, dst, n, err);
-    if (r2) return r2;
-    FH_CKS(cudaMemcpy(*dst, h.data(), n * sizeof(C), cudaMemcpyHostToDevice));
-    return 0;
-  };
-  if ((rc = upload_tw(g.nlast, &tw_last))) return rc;
-  if ((rc = upload_tw(pb.N[0], &tw0))) return rc;
-  if (d == 3 && (rc = upload_tw(pb.N[1], &tw1))) return rc;
+  if ((rc = upload_twiddles(prow, &tw_last, err))) return rc;
+  if ((rc = upload_twiddles(pcol0, &tw0, err))) return rc;
+  if (d == 3 && (rc = upload_twiddles(pcol1, &tw1, err))) return rc;
   if (d == 2 && lt.col_df) {
-    // twiddles as complex double-floats: hi = fl32(w), lo = fl32(w - hi)
-    auto upload_tw_df = [&](int n, dfc** dst) -> int {
-      std::vector<double> re, im;
-      twiddles(n, re, im);
-      std::vector<dfc> h(n);
-      for (int m = 0; m < n; ++m) {
-        h[m].x = dfl(re[m]);
-        h[m].y = dfl(im[m]);
-      }
-      int r2 = dev_alloc(allocs, dst, n, err);
-      if (r2) return r2;
-      FH_CKS(cudaMemcpy(*dst, h.data(), n * sizeof(dfc), cudaMemcpyHostToDevice));
-      return 0;
-    };
-    if ((rc = upload_tw_df(pb.N[0], &tw0_df))) return rc;
-    if ((rc = upload_tw_df(g.nlast, &tw_last_df))) return rc;
+    // the same as complex double-floats: hi = fl32(w), lo = fl32(w - hi)
+    if ((rc = upload_twiddles(pcol0, &tw0_df, err))) return rc;
+    if ((rc = upload_twiddles(prow, &tw_last_df, err))) return rc;
   }
   {
     const int nt = std::max(1, nphase) * d * d * ncell;
@@ -319,34 +292,57 @@ int Pipeline<T>::init(const Problem& pb, int nloads_, bool krylov, cudaStream_t 
                       cudaMemcpyHostToDevice));
   }
   if ((rc = dev_alloc(allocs, &d_loop, 2, err))) return rc;
-  FH_CKS(cudaMallocHost(&h_loop, 2 * sizeof(int)));
   if ((rc = dev_alloc(allocs, &dev_err, 1, err))) return rc;
   FH_CKS(cudaMemset(dev_err, 0, sizeof(int)));
-  FH_CKS(cudaMallocHost(&h_err, sizeof(int)));
-  *h_err = 0;
   const int nscal = std::max(items, kMaxLoads);
   const int nred = std::max(std::max(items, ncell * d), 16);
   if ((rc = dev_alloc(allocs, &scal, nscal, err))) return rc;
   if ((rc = dev_alloc(allocs, &scal_aux, nscal, err))) return rc;
   if ((rc = dev_alloc(allocs, &part, (size_t)3 * kMaxLoads * part_stride, err))) return rc;
   if ((rc = dev_alloc(allocs, &d_red, nred, err))) return rc;
-  FH_CKS(cudaMallocHost(&h_scal, 2 * nscal * sizeof(Scal)));
-  FH_CKS(cudaMallocHost(&h_red, nred * sizeof(double)));
-  std::memset(h_scal, 0, 2 * nscal * sizeof(Scal));
+  const size_t scal_bytes = 2 * nscal * sizeof(Scal), red_bytes = nred * sizeof(double);
+  FH_CKS(cudaMallocHost(&h_pinned, scal_bytes + red_bytes + 4 * sizeof(int)));
+  std::memset(h_pinned, 0, scal_bytes + red_bytes + 4 * sizeof(int));
+  h_scal = static_cast<Scal*>(h_pinned);
+  h_red = reinterpret_cast<double*>(static_cast<char*>(h_pinned) + scal_bytes);
+  h_loop = reinterpret_cast<int*>(static_cast<char*>(h_pinned) + scal_bytes + red_bytes);
+  h_err = h_loop + 2;
   if (!pb.L0cell.empty()) {
     if ((rc = dev_alloc(allocs, &L0cell_dev, (size_t)9 * ncell, err))) return rc;
     FH_CKS(cudaMemcpy(L0cell_dev, pb.L0cell.data(), 9 * ncell * sizeof(double), cudaMemcpyHostToDevice));
   }
   if (krylov) {
-    for (int l = 0; l < nloads; ++l) {
-      if ((rc = dev_alloc(allocs, &x[l], vlen, err))) return rc;
-      if ((rc = dev_alloc(allocs, &r[l], vlen, err))) return rc;
-      if ((rc = dev_alloc(allocs, &p[l], vlen, err))) return rc;
-      if ((rc = dev_alloc(allocs, &ap[l], vlen, err))) return rc;
-      if ((rc = dev_alloc(allocs, &rhs[l], vlen, err))) return rc;
-    }
+    // one block for the field vectors, each on a 256-byte boundary (with p2,
+    // the second direction buffer of CG, where it is needed from the start)
+    const int per = want_spectral ? 6 : 5;
+    const size_t len = ((size_t)vlen + 64 + 63) / 64 * 64;
+    T* v = nullptr;
+    if ((rc = dev_alloc(allocs, &v, len * per * nloads, err))) return rc;
+    for (int l = 0; l < nloads; ++l)
+      for (T** b : {&x[l], &r[l], &p[l], &ap[l], &rhs[l], &p2[l]}) {
+        if (b == &p2[l] && per == 5) continue;
+        *b = v;
+        v += len;
+      }
   }
   return want_spectral && krylov ? init_spectral(pb, err) : 0;
+}
+
+// A plan's stage twiddles (fh_fft.cuh) on the device.
+template <typename T>
+template <typename W>
+int Pipeline<T>::upload_twiddles(const FFTPlan& pl, W** dst, std::string& err) {
+  std::vector<double> re, im;
+  stage_twiddles(pl, re, im);
+  std::vector<W> h(re.size());
+  for (size_t m = 0; m < re.size(); ++m) {
+    h[m].x = decltype(h[m].x)(re[m]);
+    h[m].y = decltype(h[m].y)(im[m]);
+  }
+  const int rc = dev_alloc(allocs, dst, h.size() + 1, err);
+  if (rc) return rc;
+  if (!h.empty()) FH_CKS(cudaMemcpy(*dst, h.data(), h.size() * sizeof(W), cudaMemcpyHostToDevice));
+  return 0;
 }
 
 // Launch shapes and buffers of the frequency-domain CG iteration.  Left off
@@ -366,16 +362,18 @@ int Pipeline<T>::init_spectral(const Problem& pb, std::string& err) {
     auto plan = [&](int n, long long seqs, int tile_seqs, int maxthr, bool (*has_ct)(const FFTPlan&), FFTPlan& pl,
                     int& thr) -> bool {
       if (!make_fft_plan(n, false, maxthr, pl, thr)) return false;
+      mirror_order(pl);
       const bool small = !has_ct(pl) && seqs * thr < (long long)sms * 1024;
       FFTPlan p9;
       int t9;
       if (small && make_fft_plan(n, false, maxthr, p9, t9, 0, true) && t9 * tile_seqs <= maxthr) {
+        mirror_order(p9);
         pl = p9;
         thr = t9;
       }
       return true;
     };
-    const int minC = nl == 2 ? 1 : 2;  // at least one 32-byte sector of every line per column tile
+    constexpr int minC = 2;  // a column tile covers at least a 32-byte sector of every line
     if (!plan(g.nlast, d == 2 ? (long long)g.nlines * nl : (long long)(g.nlines + 1) / 2 * d * nl,
               d == 2 ? nl : d * nl, kRowMaxThreads, d == 2 ? spec_col_ct : spec_mid_ct, sprow,
               stpl) ||
@@ -404,21 +402,39 @@ int Pipeline<T>::init_spectral(const Problem& pb, std::string& err) {
     sg.inv_nodes = (float)g.inv_nodes;
     scol.block = round_up(std::max(64, Cc * 2 * nl * stpc), 32);
     scol.grid = sg.Tt * inner;
-    scol.smem = spec_col_smem(g.n[0], Cc * 2 * nl, 2 * nl, scol.block);
+    // lanes of a warp on words j of rows i: element (j % w) * step * stride + i
+    auto walk = [](int threads, int w, int step, int ss) {
+      return bank_cost(std::min(threads, 128), [&](int t) { return (long long)(t % w) * step * ss + t / w; });
+    };
+    sscol = seq_stride(spcol, stpc, Cc * 2 * nl, 2, [&](int ss) {
+      return 2 * walk(scol.block, nl * Cc, 2, ss) + 2 * walk(scol.block, Cc / 2, 4 * nl, ss);
+    });
+    scol.smem = spec_col_smem(sscol, Cc * 2 * nl, 2 * nl, scol.block);
     if (d == 3) {
       smid.block = round_up(std::max(64, Cc * 3 * nl * stpm), 32);
       smid.grid = sg.Tt * g.n[0];
-      smid.smem = (size_t)g.n1 * Cc * 3 * nl * sizeof(float2);
+      ssmid = seq_stride(spmid, stpm, Cc * 3 * nl, 2, [&](int ss) {
+        return walk(smid.block, 3 * nl * Cc, 1, ss) + 3 * walk(smid.block, nl * Cc, 3, ss);
+      });
+      smid.smem = (size_t)ssmid * Cc * 3 * nl * sizeof(float2);
     }
     // Lines per CTA: about 96 threads, two CTAs per SM where the grid has them
     const int unit = d == 2 ? 1 : 2, seq = d == 2 ? nl : d * nl;  // lines and sequences that belong together
     int k = std::max(1, 96 / (seq * stpl));
     k = std::min<int>(k, std::max(1, g.nlines / (unit * 2 * sms)));
-    while (k > 1 && ((ncell > 1 && g.lines_cell % (k * unit)) || spec_row_smem(d, nl, k * unit, g.nlast, nphase) > 64 * 1024)) --k;
+    while (k > 1 && ((ncell > 1 && g.lines_cell % (k * unit)) ||
+                     spec_row_smem(d, nl, k * unit, g.nlast, g.nlast + 15, nphase) > 64 * 1024))
+      --k;
     slpc = k * unit;
     srow.block = round_up(std::max(32, k * seq * stpl), 32);
     srow.grid = (g.nlines + slpc - 1) / slpc;
-    srow.smem = spec_row_smem(d, nl, slpc, g.nlast, nphase);
+    ssrow = seq_stride(sprow, stpl, k * seq, 2, [&](int ss) {
+      return 2 * bank_cost(std::min(srow.block, 128), [&](int t) -> long long {
+        const int c = d == 2 ? t : 2 * t;  // 3-D: two elements per 16-byte word
+        return (long long)(c % seq) * ss + c / seq;
+      });
+    });
+    srow.smem = spec_row_smem(d, nl, slpc, g.nlast, ssrow, nphase);
     if (srow.smem > cap || srow.block > 768 || scol.smem > cap) return 0;
     const bool more_part = scol.grid > part_stride;
     part_stride = std::max(part_stride, scol.grid);
@@ -426,6 +442,9 @@ int Pipeline<T>::init_spectral(const Problem& pb, std::string& err) {
     if (d == 3) FH_CKS(spec_mid_set_smem(spec_mid_args(), smid.smem));
     FH_CKS(d == 2 ? spec_row_d2_set_smem(spec_row_args(), srow) : spec_row_d3_set_smem(spec_row_args(), srow));
     int rc;
+    if ((rc = upload_twiddles(sprow, &stw_row, err)) || (rc = upload_twiddles(spcol, &stw_col, err)) ||
+        (d == 3 && (rc = upload_twiddles(spmid, &stw_mid, err))))
+      return rc;
     const size_t lines = (size_t)sg.Hp * g.nlines;
     // the operator's own spectrum buffer may be smaller than the padded lines
     if (lines * d * nl > (size_t)g.Tt * g.C * g.nlines * g.M && (rc = dev_alloc(allocs, &S, lines * d * nl, err))) return rc;
@@ -455,8 +474,6 @@ int Pipeline<T>::init_spectral(const Problem& pb, std::string& err) {
       FH_CKS(cudaMemcpy(smed, hm.data(), ncell * sizeof(SpecMedium), cudaMemcpyHostToDevice));
     }
     if (more_part && (rc = dev_alloc(allocs, &part, (size_t)3 * kMaxLoads * part_stride, err))) return rc;
-    for (int l = 0; l < nl; ++l)
-      if ((rc = dev_alloc(allocs, &p2[l], vlen, err))) return rc;
     if (2 * lines > (size_t)vlen)  // padded scalar arrays do not fit the field buffers
       for (int l = 0; l < nl; ++l)
         for (T** b : {&r[l], &p[l], &ap[l], &p2[l]})
@@ -479,7 +496,8 @@ SpecArgs Pipeline<T>::spec_args() const {
   a.plan = spcol;
   a.tpc = stpc;
   a.nb_inner = g.d == 2 ? ncell : g.n1;
-  a.tw = reinterpret_cast<const float2*>(tw0);
+  a.ss = sscol;
+  a.tw = stw_col;
   a.S = g.d == 3 ? reinterpret_cast<float2*>(S2) : reinterpret_cast<float2*>(S);
   for (int l = 0; l < nloads; ++l) {
     a.r[l] = reinterpret_cast<float2*>(r[l]);
@@ -504,7 +522,8 @@ SpecRowArgs Pipeline<T>::spec_row_args() const {
   a.plan = sprow;
   a.tpl = stpl;
   a.lpc = slpc;
-  a.tw = reinterpret_cast<const float2*>(tw_last);
+  a.ss = ssrow;
+  a.tw = stw_row;
   a.S = reinterpret_cast<float2*>(S);
   a.phase = phase;
   a.tab = reinterpret_cast<const float*>(dtab);
@@ -522,7 +541,8 @@ SpecMidArgs Pipeline<T>::spec_mid_args() const {
   m.plan = spmid;
   m.tpc = stpm;
   m.nl = nloads;
-  m.tw = reinterpret_cast<const float2*>(tw1);
+  m.ss = ssmid;
+  m.tw = stw_mid;
   m.S2 = reinterpret_cast<float2*>(S2);
   m.S3 = reinterpret_cast<float2*>(S);
   return m;
@@ -600,12 +620,9 @@ int Pipeline<T>::spec_dir_norm2(const double* Mx, double* out, std::string& err)
 
 template <typename T>
 void Pipeline<T>::release() {
-  for (void* q : allocs) cudaFree(q);
-  allocs.clear();
-  if (h_scal) cudaFreeHost(h_scal);
-  if (h_red) cudaFreeHost(h_red);
-  if (h_err) cudaFreeHost(h_err);
-  if (h_loop) cudaFreeHost(h_loop);
+  allocs.release();
+  if (h_pinned) cudaFreeHost(h_pinned);
+  h_pinned = nullptr;
   loops.clear();
   h_scal = nullptr;
   h_red = nullptr;

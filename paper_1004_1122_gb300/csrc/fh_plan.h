@@ -143,4 +143,92 @@ inline void twiddles(int n, std::vector<double>& re, std::vector<double>& im) {
   }
 }
 
+// Entries of a plan's twiddle table: its stages in order, then those of the
+// reversed radix order.
+inline int stage_twiddle_count(const FFTPlan& pl) {
+  return 2 * pl.n - pl.radix[0] - pl.radix[pl.nstages - 1];
+}
+// The table (fh_fft.cuh), from the n-th roots of unity.
+inline void stage_twiddles(const FFTPlan& pl, std::vector<double>& re, std::vector<double>& im) {
+  std::vector<double> wr, wi;
+  twiddles(pl.n, wr, wi);
+  re.clear();
+  im.clear();
+  for (int rev = 0; rev < 2; ++rev) {
+    int Ns = 1;
+    for (int s = 0; s < pl.nstages; ++s) {
+      const int R = pl.radix[rev ? pl.nstages - 1 - s : s];
+      if (s > 0)
+        for (int r = 1; r < R; ++r)
+          for (int k = 0; k < Ns; ++k) {
+            const int m = (int)((long long)r * k * (pl.n / (Ns * R)) % pl.n);
+            re.push_back(wr[m]);
+            im.push_back(wi[m]);
+          }
+      Ns *= R;
+    }
+  }
+}
+
+// Stage order of plans whose transform is followed by its mirror image: the
+// smallest radix in the middle.  After a first stage of radix 3 (the mirror
+// image of 27, 27, 3) the writes of the next stage collide in shared-memory
+// banks; with 27, 3, 27 every stage's writes run along consecutive words.
+inline void mirror_order(FFTPlan& pl) {
+  if (pl.nstages < 3) return;
+  for (int s = pl.nstages - 1; s > 1; --s) std::swap(pl.radix[s], pl.radix[s - 1]);
+}
+
+// Shared-memory bank cost of 8-byte accesses: lanes t of a warp access element
+// addr(t) (negative: none); 16 banks of 8 bytes, one half warp at a time.
+template <typename F> inline int bank_cost(int threads, F&& addr) {
+  int total = 0;
+  for (int h0 = 0; h0 < threads; h0 += 16) {
+    long long seen[16][16];
+    int cnt[16] = {};
+    int worst = 0;
+    for (int t = h0; t < h0 + 16 && t < threads; ++t) {
+      const long long a = addr(t);
+      if (a < 0) continue;
+      const int b = (int)(a % 16);
+      bool dup = false;
+      for (int k = 0; k < cnt[b]; ++k) dup = dup || seen[b][k] == a;
+      if (!dup) seen[b][cnt[b]++] = a;
+      worst = std::max(worst, cnt[b]);
+    }
+    total += worst;
+  }
+  return total;
+}
+
+// Distance between sequences in shared memory (n .. n + 15 elements) with the
+// fewest bank conflicts of the plan's stages over nseq sequences of thr
+// threads, plus `weight` times the cost of io(stride).
+template <typename F>
+inline int seq_stride(const FFTPlan& pl, int thr, int nseq, int weight, F&& io) {
+  const int threads = std::min(nseq * thr, 512);
+  int best = pl.n, best_cost = 1 << 30;
+  for (int ss = pl.n; ss < pl.n + 16; ++ss) {
+    int cost = weight * io(ss);
+    int Ns = 1;
+    for (int s = 0; s < pl.nstages; ++s) {
+      const int R = pl.radix[s], nb = pl.n / R;
+      cost += R * bank_cost(threads, [&](int t) -> long long {
+        const int q = t / thr, j = t - q * thr;
+        return j < nb ? (long long)q * ss + j : -1;
+      });
+      cost += R * bank_cost(threads, [&](int t) -> long long {
+        const int q = t / thr, j = t - q * thr;
+        return j < nb ? (long long)q * ss + (j / Ns) * R * Ns + j % Ns : -1;
+      });
+      Ns *= R;
+    }
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = ss;
+    }
+  }
+  return best;
+}
+
 }  // namespace fh

@@ -3,7 +3,7 @@
 //
 // Which lengths: the odd lengths whose only prime factors are 3 and 5, from 75
 // nodes (shorter axes belong to grids that launch latency bounds); each entry
-// is the plan make_fft_plan picks for that length.  Other lengths, and the
+// is the plan make_fft_plan picks for that length, in mirror_order.  Other lengths, and the
 // small-radix plans of small grids, run the run-time-plan kernels.
 #pragma once
 
@@ -16,7 +16,7 @@ template <typename... Ps> struct PlanList {};
 using SpecPlans3D = PlanList<CPlan<25, 3>, CPlan<27, 3>, CPlan<25, 5>, CPlan<27, 5>, CPlan<25, 9>, CPlan<27, 9>>;
 using SpecPlans = PlanList<CPlan<25, 3>, CPlan<27, 3>, CPlan<25, 5>, CPlan<27, 5>, CPlan<25, 9>, CPlan<27, 9>,
                            CPlan<25, 15>, CPlan<27, 15>, CPlan<25, 25>, CPlan<27, 25>, CPlan<27, 27>,
-                           CPlan<25, 9, 5>, CPlan<27, 9, 5>, CPlan<25, 25, 3>, CPlan<27, 25, 3>, CPlan<27, 27, 3>>;
+                           CPlan<25, 5, 9>, CPlan<27, 5, 9>, CPlan<25, 3, 25>, CPlan<27, 3, 25>, CPlan<27, 3, 27>>;
 
 // Calls f(P{}) for the compile-time plan of the list that equals pl, or
 // f(DynPlan{}) when there is none.

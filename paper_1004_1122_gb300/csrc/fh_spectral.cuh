@@ -60,6 +60,7 @@ struct SpecArgs {
   SpecGeom sg;
   FFTPlan plan;                // along axis 0
   int tpc;                     // threads per column FFT
+  int ss;                      // distance between columns in shared memory
   int nb_inner;                // 2-D: cells; 3-D: lines along axis 1
   int nl, three;               // loads; 3-D
   const float2* tw;
@@ -124,13 +125,15 @@ template <typename PS> __device__ __forceinline__ int spec_threads(int rt) {
   return PlanLen<PS>::value > 0 ? spec_plan_threads<PS>() : rt;
 }
 
-// Column FFTs of a tile stored column by column (column q at sm + q n): the
-// stage addresses of a compile-time plan are then constants.
+// Column FFTs of a tile stored column by column (column q at sm + q ss): the
+// stage addresses of a compile-time plan are then constants, and ss >= n is
+// chosen for the fewest bank conflicts (seq_stride).
 template <bool INV, typename PS>
-__device__ __forceinline__ void spec_col_fft(float2* sm, int n, int Q, const FFTPlan& plan, int tpc_rt, const float2* tw) {
+__device__ __forceinline__ void spec_col_fft(float2* sm, int ss, int n, int Q, const FFTPlan& plan, int tpc_rt,
+                                             const float2* tw) {
   const int tpc = spec_threads<PS>(tpc_rt);
   const int q = threadIdx.x / tpc, u = threadIdx.x - q * tpc;
-  fft_plan<INV, float, PS>(sm + (q < Q ? q : 0) * n, 1, plan, q < Q ? u : n, tpc, tw);
+  fft_plan<INV, float, PS>(sm + (q < Q ? q : 0) * ss, 1, plan, q < Q ? u : n, tpc, tw);
 }
 
 // The scalars of one thread of a column kernel all belong to one frequency of
@@ -221,9 +224,8 @@ template <typename PS> struct SpecBounds {
 enum : int { kSpecUpdate = 0, kSpecFinish = 1 };   // spec_inv
 enum : int { kSpecApply = 0, kSpecProject = 1 };   // spec_fwd
 
-__host__ __device__ inline size_t spec_col_tile(int n, int Q) { return ((size_t)n * Q + 1) / 2 * 2; }  // float2, 16-byte multiple
-inline size_t spec_col_smem(int n, int Q, int rows, int block) {
-  return (spec_col_tile(n, Q) + (size_t)rows * block) * sizeof(float2);
+inline size_t spec_col_smem(int ss, int Q, int rows, int block) {
+  return ((size_t)ss * Q + (size_t)rows * block) * sizeof(float2);
 }
 
 // kSpecUpdate: one CG update of the tile's scalars, then the inverse FFT of
@@ -234,76 +236,89 @@ __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_inv(SpecArgs a
   float2* sm = reinterpret_cast<float2*>(smem_raw);
   const int n = plan_len<PS>(a.plan), C = a.sg.C, csh = a.sg.csh, nl = a.nl;
   const int Q = 2 * nl * C;
-  float2* const red = sm + spec_col_tile(n, Q);
+  float2* const red = sm + (size_t)a.ss * Q;
   const SpecTile tl = spec_tile(a, n);
   Scal* const sc = a.scal + tl.cell * nl;
   if (MODE == kSpecUpdate && all_done(sc, nl)) return;
-  const int e = threadIdx.x & (C - 1), row0 = threadIdx.x >> csh, drow = blockDim.x >> csh;
-  SpecFreq fq;
-  fq.init(a, a.med[tl.cell], n, tl.t * C + e, tl.inner);
-  constexpr int kUnroll = 4;
+  // a thread holds two neighbouring frequencies (16-byte words)
+  const int e = 2 * (threadIdx.x & (C / 2 - 1)), row0 = threadIdx.x >> (csh - 1), drow = blockDim.x >> (csh - 1);
+  SpecFreq fq[2];
+  fq[0].init(a, a.med[tl.cell], n, tl.t * C + e, tl.inner);
+  fq[1].init(a, a.med[tl.cell], n, tl.t * C + e + 1, tl.inner);
+  constexpr int kUnroll = 2;
   for (int l = 0; l < nl; ++l) {
     const Scal& s = sc[l];
     const bool fresh = s.iter == 0;
     const float al = MODE == kSpecUpdate || s.xpend ? s.alpha_f : 0.0f;
     const float be = s.beta_f;
     const bool live = MODE == kSpecUpdate ? s.done == kRunning : !fresh;
-    float2* const r = a.r[l] + tl.sbase + e;
-    float2* const p = a.p[l] + tl.sbase + e;
-    float2* const x = a.x[l] + tl.sbase + e;
-    const float2* const ap = a.ap[l] + tl.sbase + e;
-    float2* const ch0 = sm + (size_t)(e * nl + l) * 2 * n;
-    float2* const ch1 = ch0 + n;
-    DotAcc<float> dot;
+    float4* const r = reinterpret_cast<float4*>(a.r[l] + tl.sbase + e);
+    float4* const p = reinterpret_cast<float4*>(a.p[l] + tl.sbase + e);
+    float4* const x = reinterpret_cast<float4*>(a.x[l] + tl.sbase + e);
+    const float4* const ap = reinterpret_cast<const float4*>(a.ap[l] + tl.sbase + e);
+    float2* const ch = sm + (size_t)(e * nl + l) * 2 * a.ss;
+    const int next = 2 * nl * a.ss;  // the second frequency's columns
+    DotAcc<float> dot[2];
     for (int i0 = row0; i0 < n; i0 += kUnroll * drow) {
-      float2 vr[kUnroll], vp[kUnroll], va[kUnroll], vx[kUnroll];
+      float4 vr[kUnroll], vp[kUnroll], va[kUnroll], vx[kUnroll];
 #pragma unroll
       for (int u = 0; u < kUnroll; ++u) {
-        const int i = i0 + u * drow;
-        vr[u] = vp[u] = va[u] = vx[u] = make_float2(0.0f, 0.0f);
+        const int i = i0 + u * drow, k = i << (csh - 1);
+        vr[u] = vp[u] = va[u] = vx[u] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         if (i < n && live) {
-          if (MODE == kSpecUpdate) vr[u] = r[i << csh];
+          // r and x are touched once per iteration: kept out of the way of
+          // what the next passes read again (S, p, A p)
+          if (MODE == kSpecUpdate) vr[u] = __ldcs(r + k);
           if (!fresh) {
-            if (MODE == kSpecUpdate) va[u] = __ldg(ap + (i << csh));
-            vp[u] = p[i << csh];
-            vx[u] = x[i << csh];
+            if (MODE == kSpecUpdate) va[u] = __ldg(ap + k);
+            vp[u] = p[k];
+            vx[u] = __ldcs(x + k);
           }
         }
       }
 #pragma unroll
       for (int u = 0; u < kUnroll; ++u) {
-        const int i = i0 + u * drow;
+        const int i = i0 + u * drow, k = i << (csh - 1);
         if (i >= n) continue;
-        vx[u].x += al * vp[u].x;
-        vx[u].y += al * vp[u].y;
-        float2 v = vx[u];
+        auto axpy = [](float4& y, float c, const float4& z) {
+          y.x += c * z.x;
+          y.y += c * z.y;
+          y.z += c * z.z;
+          y.w += c * z.w;
+        };
+        axpy(vx[u], al, vp[u]);
+        float4 v = vx[u];
         if (MODE == kSpecUpdate) {
-          vr[u].x -= al * va[u].x;
-          vr[u].y -= al * va[u].y;
-          v.x = vr[u].x + be * vp[u].x;
-          v.y = vr[u].y + be * vp[u].y;
+          axpy(vr[u], -al, va[u]);
+          v = vr[u];
+          axpy(v, be, vp[u]);
           if (live) {
-            r[i << csh] = vr[u];
-            p[i << csh] = v;
-            x[i << csh] = vx[u];
+            __stcs(r + k, vr[u]);
+            p[k] = v;
+            __stcs(x + k, vx[u]);
           }
-          dot.add(vr[u].x * vr[u].x + vr[u].y * vr[u].y);
+          dot[0].add(vr[u].x * vr[u].x + vr[u].y * vr[u].y);
+          dot[1].add(vr[u].z * vr[u].z + vr[u].w * vr[u].w);
         }
-        const float x0 = fq.xi0(i), s1 = fq.rnorm(i, x0);
-        const float f0 = x0 * s1, f1 = fq.c1 * s1;
-        ch0[i] = make_float2(f0 * v.x, f0 * v.y);
-        ch1[i] = make_float2(f1 * v.x, f1 * v.y);
+        const float x0 = fq[0].xi0(i);
+        const float s0 = fq[0].rnorm(i, x0), s1 = fq[1].rnorm(i, x0);
+        const float f0 = x0 * s0, g0 = fq[0].c1 * s0, f1 = x0 * s1, g1 = fq[1].c1 * s1;
+        ch[i] = make_float2(f0 * v.x, f0 * v.y);
+        ch[a.ss + i] = make_float2(g0 * v.x, g0 * v.y);
+        ch[next + i] = make_float2(f1 * v.z, f1 * v.w);
+        ch[next + a.ss + i] = make_float2(g1 * v.z, g1 * v.w);
       }
     }
-    if (MODE == kSpecUpdate) red[l * blockDim.x + threadIdx.x] = ff_of(dot, fq.wgt);
+    if (MODE == kSpecUpdate)
+      red[l * blockDim.x + threadIdx.x] = ff_add(ff_of(dot[0], fq[0].wgt), ff_of(dot[1], fq[1].wgt));
   }
   __syncthreads();
-  spec_col_fft<true, PS>(sm, n, Q, a.plan, a.tpc, a.tw);
+  spec_col_fft<true, PS>(sm, a.ss, n, Q, a.plan, a.tpc, a.tw);
   const int wpr = nl * C;  // 16-byte words per row
   float4* const S = reinterpret_cast<float4*>(a.S) + (tl.line0 * a.sg.Hp + tl.t * C) * nl;
   const long long rs = (long long)tl.step * a.sg.Hp * nl;
   for (SpecWalk w(wpr); w.i < n; w.next()) {
-    const float2 v0 = sm[2 * w.j * n + w.i], v1 = sm[(2 * w.j + 1) * n + w.i];
+    const float2 v0 = sm[2 * w.j * a.ss + w.i], v1 = sm[(2 * w.j + 1) * a.ss + w.i];
     S[w.i * rs + w.j] = make_float4(v0.x, v0.y, v1.x, v1.y);
   }
   if (MODE == kSpecUpdate)
@@ -318,11 +333,11 @@ __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_fwd(SpecArgs a
   float2* sm = reinterpret_cast<float2*>(smem_raw);
   const int n = plan_len<PS>(a.plan), C = a.sg.C, csh = a.sg.csh, nl = a.nl;
   const int Q = 2 * nl * C;
-  float2* const red = sm + spec_col_tile(n, Q);
+  float2* const red = sm + (size_t)a.ss * Q;
   const SpecTile tl = spec_tile(a, n);
   Scal* const sc = a.scal + tl.cell * nl;
   if (MODE == kSpecApply && all_done(sc, nl)) return;
-  const int e = threadIdx.x & (C - 1), row0 = threadIdx.x >> csh, drow = blockDim.x >> csh;
+  const int e = 2 * (threadIdx.x & (C / 2 - 1)), row0 = threadIdx.x >> (csh - 1), drow = blockDim.x >> (csh - 1);
   constexpr int kUnroll = 4;
   {
     const int wpr = nl * C;
@@ -334,7 +349,7 @@ __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_fwd(SpecArgs a
       int at[kUnroll];
 #pragma unroll
       for (int u = 0; u < kUnroll; ++u) {
-        at[u] = w.i < n ? 2 * w.j * n + w.i : -1;
+        at[u] = w.i < n ? 2 * w.j * a.ss + w.i : -1;
         if (w.i < n) buf[u] = __ldg(S + w.i * rs + w.j);
         w.next();
       }
@@ -342,50 +357,57 @@ __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_fwd(SpecArgs a
       for (int u = 0; u < kUnroll; ++u)
         if (at[u] >= 0) {
           sm[at[u]] = make_float2(buf[u].x, buf[u].y);
-          sm[at[u] + n] = make_float2(buf[u].z, buf[u].w);
+          sm[at[u] + a.ss] = make_float2(buf[u].z, buf[u].w);
         }
     }
   }
-  SpecFreq fq;
-  fq.init(a, a.med[tl.cell], n, tl.t * C + e, tl.inner);
   __syncthreads();
-  spec_col_fft<false, PS>(sm, n, Q, a.plan, a.tpc, a.tw);
+  spec_col_fft<false, PS>(sm, a.ss, n, Q, a.plan, a.tpc, a.tw);
+  SpecFreq fq[2];
+  fq[0].init(a, a.med[tl.cell], n, tl.t * C + e, tl.inner);
+  fq[1].init(a, a.med[tl.cell], n, tl.t * C + e + 1, tl.inner);
   for (int l = 0; l < nl; ++l) {
-    DotAcc<float> d1, d2;
+    DotAcc<float> d1[2], d2[2];
     if (MODE == kSpecProject || sc[l].done == kRunning) {
-      const float2* const p = a.p[l] + tl.sbase + e;
-      float2* const out = (MODE == kSpecApply ? a.ap[l] : a.r[l]) + tl.sbase + e;
-      const float2* const ch0 = sm + (size_t)(e * nl + l) * 2 * n;
-      const float2* const ch1 = ch0 + n;
+      const float4* const p = reinterpret_cast<const float4*>(a.p[l] + tl.sbase + e);
+      float4* const out = reinterpret_cast<float4*>((MODE == kSpecApply ? a.ap[l] : a.r[l]) + tl.sbase + e);
+      const float2* const ch = sm + (size_t)(e * nl + l) * 2 * a.ss;
+      const int next = 2 * nl * a.ss;
       for (int i0 = row0; i0 < n; i0 += kUnroll * drow) {
-        float2 vp[kUnroll];
+        float4 vp[kUnroll];
 #pragma unroll
         for (int u = 0; u < kUnroll; ++u) {
           const int i = i0 + u * drow;
-          vp[u] = (MODE == kSpecApply && i < n) ? __ldg(p + (i << csh)) : make_float2(0.0f, 0.0f);
+          vp[u] = (MODE == kSpecApply && i < n) ? __ldg(p + (i << (csh - 1))) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         }
 #pragma unroll
         for (int u = 0; u < kUnroll; ++u) {
           const int i = i0 + u * drow;
           if (i >= n) continue;
-          const float2 v0 = ch0[i], v1 = ch1[i];
-          const float x0 = fq.xi0(i), rn = fq.rnorm(i, x0);
-          const float w = MODE == kSpecApply ? fq.project(x0, rn) : rn * a.sg.inv_nodes;
-          const float w0 = x0 * w, w1 = fq.c1 * w;
-          float2 y = make_float2(w0 * v0.x + w1 * v1.x, w0 * v0.y + w1 * v1.y);
-          if (MODE == kSpecApply) {
-            y.x += vp[u].x;
-            y.y += vp[u].y;
-            d1.add(vp[u].x * y.x + vp[u].y * y.y);
-            d2.add(y.x * y.x + y.y * y.y);
+          const float x0 = fq[0].xi0(i);
+          float2 y[2];
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const float2 v0 = ch[h * next + i], v1 = ch[h * next + a.ss + i];
+            const float rn = fq[h].rnorm(i, x0);
+            const float w = MODE == kSpecApply ? fq[h].project(x0, rn) : rn * a.sg.inv_nodes;
+            const float w0 = x0 * w, w1 = fq[h].c1 * w;
+            y[h] = make_float2(w0 * v0.x + w1 * v1.x, w0 * v0.y + w1 * v1.y);
+            if (MODE == kSpecApply) {
+              const float2 q = h ? make_float2(vp[u].z, vp[u].w) : make_float2(vp[u].x, vp[u].y);
+              y[h].x += q.x;
+              y[h].y += q.y;
+              d1[h].add(q.x * y[h].x + q.y * y[h].y);
+              d2[h].add(y[h].x * y[h].x + y[h].y * y[h].y);
+            }
           }
-          out[i << csh] = y;
+          out[i << (csh - 1)] = make_float4(y[0].x, y[0].y, y[1].x, y[1].y);
         }
       }
     }
     if (MODE == kSpecApply) {
-      red[l * blockDim.x + threadIdx.x] = ff_of(d1, fq.wgt);
-      red[(nl + l) * blockDim.x + threadIdx.x] = ff_of(d2, fq.wgt);
+      red[l * blockDim.x + threadIdx.x] = ff_add(ff_of(d1[0], fq[0].wgt), ff_of(d1[1], fq[1].wgt));
+      red[(nl + l) * blockDim.x + threadIdx.x] = ff_add(ff_of(d2[0], fq[0].wgt), ff_of(d2[1], fq[1].wgt));
     }
   }
   if (MODE == kSpecApply) {
@@ -405,6 +427,7 @@ struct SpecMidArgs {
   SpecGeom sg;
   FFTPlan plan;                // along axis 1
   int tpc;
+  int ss;                      // distance between columns in shared memory
   int nl;
   const float2* tw;
   float2* S2;                  // two channels per load
@@ -445,15 +468,15 @@ __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_mid(SpecMidArg
         if (wi[u] >= n) continue;
         const float xi1 = (float)signed_freq(wi[u], n) * invY1;
         const float xi2 = (float)(t * C + (nl == 1 ? wj[u] : wj[u] / 3)) * invY2;
-        float2* d = sm + wj[u] * 3 * n + wi[u];
+        float2* d = sm + wj[u] * 3 * a.ss + wi[u];
         d[0] = make_float2(v[u].x, v[u].y);
-        d[n] = make_float2(xi1 * v[u].z, xi1 * v[u].w);
-        d[2 * n] = make_float2(xi2 * v[u].z, xi2 * v[u].w);
+        d[a.ss] = make_float2(xi1 * v[u].z, xi1 * v[u].w);
+        d[2 * a.ss] = make_float2(xi2 * v[u].z, xi2 * v[u].w);
       }
     }
     __syncthreads();
-    spec_col_fft<true, PS>(sm, n, Q, a.plan, a.tpc, a.tw);
-    for (SpecWalk o(Q); o.i < n; o.next()) S3[o.i * rs * 3 + o.j] = sm[o.j * n + o.i];
+    spec_col_fft<true, PS>(sm, a.ss, n, Q, a.plan, a.tpc, a.tw);
+    for (SpecWalk o(Q); o.i < n; o.next()) S3[o.i * rs * 3 + o.j] = sm[o.j * a.ss + o.i];
   } else {
     SpecWalk w(Q);
     while (w.i < n) {
@@ -461,7 +484,7 @@ __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_mid(SpecMidArg
       int at[kUnroll];
 #pragma unroll
       for (int u = 0; u < kUnroll; ++u) {
-        at[u] = w.i < n ? w.j * n + w.i : -1;
+        at[u] = w.i < n ? w.j * a.ss + w.i : -1;
         if (w.i < n) v[u] = S3[w.i * rs * 3 + w.j];
         w.next();
       }
@@ -470,12 +493,12 @@ __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_mid(SpecMidArg
         if (at[u] >= 0) sm[at[u]] = v[u];
     }
     __syncthreads();
-    spec_col_fft<false, PS>(sm, n, Q, a.plan, a.tpc, a.tw);
+    spec_col_fft<false, PS>(sm, a.ss, n, Q, a.plan, a.tpc, a.tw);
     for (SpecWalk o(rc); o.i < n; o.next()) {
       const float xi1 = (float)signed_freq(o.i, n) * invY1;
       const float xi2 = (float)(t * C + (nl == 1 ? o.j : o.j / 3)) * invY2;
-      const float2* s = sm + o.j * 3 * n + o.i;
-      const float2 s0 = s[0], s1 = s[n], s2 = s[2 * n];
+      const float2* s = sm + o.j * 3 * a.ss + o.i;
+      const float2 s0 = s[0], s1 = s[a.ss], s2 = s[2 * a.ss];
       S2[o.i * rs + o.j] = make_float4(s0.x, s0.y, xi1 * s1.x + xi2 * s2.x, xi1 * s1.y + xi2 * s2.y);
     }
   }
@@ -490,6 +513,7 @@ struct SpecRowArgs {
   FFTPlan plan;                // along the last axis
   int tpl;                     // threads per line FFT
   int lpc;                     // lines per CTA (3-D: even)
+  int ss;                      // distance between sequences in shared memory
   const float2* tw;
   float2* S;                   // D components per load, in place
   const uint8_t* phase;
@@ -509,16 +533,17 @@ enum : int {
 // imaginary part; 3-D, one per (pair of lines, load, component), the two lines
 // as real and imaginary part (no channel is left unpaired).
 // Thread and residency limits of the row kernels: 80 registers for the 27
-// complex values of a thread.
+// complex values of a thread of a compile-time plan; the run-time plans'
+// kernels, which hold every radix twice, spill at 80.
 constexpr int kSpecRowCtThreads = 192;
 template <typename PS> struct SpecRowBounds {
-  static constexpr int threads = PlanLen<PS>::value > 0 ? kSpecRowCtThreads : 768;
+  static constexpr int threads = PlanLen<PS>::value > 0 ? kSpecRowCtThreads : kRowMaxThreads;
   static constexpr int blocks = PlanLen<PS>::value > 0 ? 4 : 1;
 };
 
-inline size_t spec_row_smem(int d, int nl, int lpc, int n, int nphase) {
+inline size_t spec_row_smem(int d, int nl, int lpc, int n, int ss, int nphase) {
   const size_t nseq = d == 2 ? lpc * nl : lpc / 2 * d * nl;
-  return (nseq * n + 1) / 2 * 16 + (size_t)nphase * d * d * sizeof(float) + (size_t)lpc * n;
+  return (nseq * ss + 1) / 2 * 16 + (size_t)nphase * d * d * sizeof(float) + (size_t)lpc * n;
 }
 
 template <int D, int NL, int MODE, typename PS = DynPlan>
@@ -528,12 +553,12 @@ __global__ void __launch_bounds__(SpecRowBounds<PS>::threads, SpecRowBounds<PS>:
   const Geom& g = a.g;
   constexpr int M = D * NL;
   const int n = plan_len<PS>(a.plan);
-  const int nthr = blockDim.x, tpl = spec_threads<PS>(a.tpl), lpc = a.lpc, H = g.H, Hp = a.sg.Hp;
+  const int nthr = blockDim.x, tpl = spec_threads<PS>(a.tpl), lpc = a.lpc, H = g.H, Hp = a.sg.Hp, ss = a.ss;
   const int nseq = D == 2 ? lpc * NL : (lpc / 2) * M;
   const int line0 = blockIdx.x * lpc;
   const int cell = g.ncell > 1 ? line0 / g.lines_cell : 0;
   if (MODE == kSpecRowTau && all_done(a.scal + cell * NL, NL)) return;
-  float* const stab = reinterpret_cast<float*>(sm + (((size_t)nseq * n + 1) & ~(size_t)1));  // 16-byte aligned
+  float* const stab = reinterpret_cast<float*>(sm + (((size_t)nseq * ss + 1) & ~(size_t)1));  // 16-byte aligned
   uint8_t* const sph = reinterpret_cast<uint8_t*>(stab + a.nphase * D * D);
   if (MODE == kSpecRowTau) {
     const float* const tabc = a.tab + (size_t)cell * g.tab_stride;
@@ -563,7 +588,7 @@ __global__ void __launch_bounds__(SpecRowBounds<PS>::threads, SpecRowBounds<PS>:
             const int w = w0 + u * nthr;
             if (w >= H * NL) continue;
             const int kx = w / NL, l = w - kx * NL;
-            float2* const seq = sm + (size_t)(ll * NL + l) * n;
+            float2* const seq = sm + (size_t)(ll * NL + l) * ss;
             if (kx == 0 || 2 * kx == n) {  // bins that are their own Hermitian partner
               seq[kx] = make_float2(v[u].x, v[u].z);
             } else {
@@ -597,7 +622,7 @@ __global__ void __launch_bounds__(SpecRowBounds<PS>::threads, SpecRowBounds<PS>:
               if (kx >= H) continue;
               const float2 ya = h ? make_float2(va[u].z, va[u].w) : make_float2(va[u].x, va[u].y);
               const float2 yb = h ? make_float2(vb[u].z, vb[u].w) : make_float2(vb[u].x, vb[u].y);
-              float2* const seq = sm + (size_t)(lp * M + m) * n;
+              float2* const seq = sm + (size_t)(lp * M + m) * ss;
               if (kx == 0 || 2 * kx == n) {
                 seq[kx] = make_float2(ya.x, yb.x);
               } else {
@@ -618,7 +643,7 @@ __global__ void __launch_bounds__(SpecRowBounds<PS>::threads, SpecRowBounds<PS>:
         const float* const src = a.f[m / D] + (m % D) * g.nodes + lo;
         const int s = D == 2 ? ll * NL + m / 2 : (ll / 2) * M + m, half = D == 2 ? m & 1 : ll & 1;
         for (int i = threadIdx.x; i < n; i += nthr)
-          reinterpret_cast<float*>(sm + (size_t)s * n + i)[half] = ok ? src[i] : 0.0f;
+          reinterpret_cast<float*>(sm + (size_t)s * ss + i)[half] = ok ? src[i] : 0.0f;
       }
     }
   }
@@ -626,7 +651,7 @@ __global__ void __launch_bounds__(SpecRowBounds<PS>::threads, SpecRowBounds<PS>:
 
   const int s = threadIdx.x / tpl;
   const int u = s < nseq ? threadIdx.x - s * tpl : n;  // idle threads never touch smem
-  float2* const seq = sm + (size_t)(s < nseq ? s : 0) * n;
+  float2* const seq = sm + (size_t)(s < nseq ? s : 0) * ss;
   if constexpr (MODE == kSpecRowLoad) {
     fft_plan<false, float, PS>(seq, 1, a.plan, u, tpl, a.tw);
   } else if constexpr (MODE == kSpecRowAdd) {
@@ -639,7 +664,7 @@ __global__ void __launch_bounds__(SpecRowBounds<PS>::threads, SpecRowBounds<PS>:
         float* const dst = a.f[m / D] + (m % D) * g.nodes + lo;
         const int q = D == 2 ? ll * NL + m / 2 : (ll / 2) * M + m, half = D == 2 ? m & 1 : ll & 1;
         for (int i = threadIdx.x; i < n; i += nthr)
-          dst[i] += reinterpret_cast<const float*>(sm + (size_t)q * n + i)[half];
+          dst[i] += reinterpret_cast<const float*>(sm + (size_t)q * ss + i)[half];
       }
     }
     return;
@@ -659,7 +684,7 @@ __global__ void __launch_bounds__(SpecRowBounds<PS>::threads, SpecRowBounds<PS>:
       if (line0 + 2 * lp >= g.nlines) break;
       const uint8_t* const pa = sph + 2 * lp * n;
       const uint8_t* const pb = line0 + 2 * lp + 1 < g.nlines ? pa + n : pa;
-      float2* const base = sm + (size_t)lp * M * n;
+      float2* const base = sm + (size_t)lp * M * ss;
       for (int i = threadIdx.x; i < n; i += nthr) {
         const float* const ta = stab + pa[i] * 9;
         const float* const tb = stab + pb[i] * 9;
@@ -667,10 +692,10 @@ __global__ void __launch_bounds__(SpecRowBounds<PS>::threads, SpecRowBounds<PS>:
         for (int l = 0; l < NL; ++l) {
           float2 v[3];
 #pragma unroll
-          for (int c = 0; c < 3; ++c) v[c] = base[(l * 3 + c) * n + i];
+          for (int c = 0; c < 3; ++c) v[c] = base[(l * 3 + c) * ss + i];
 #pragma unroll
           for (int c = 0; c < 3; ++c)
-            base[(l * 3 + c) * n + i] = make_float2(ta[3 * c] * v[0].x + ta[3 * c + 1] * v[1].x + ta[3 * c + 2] * v[2].x,
+            base[(l * 3 + c) * ss + i] = make_float2(ta[3 * c] * v[0].x + ta[3 * c + 1] * v[1].x + ta[3 * c + 2] * v[2].x,
                                                     tb[3 * c] * v[0].y + tb[3 * c + 1] * v[1].y + tb[3 * c + 2] * v[2].y);
         }
       }
@@ -688,7 +713,7 @@ __global__ void __launch_bounds__(SpecRowBounds<PS>::threads, SpecRowBounds<PS>:
         const int kx = w / NL, l = w - kx * NL;
         float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         if (kx < H) {
-          const float2* const sq = sm + (size_t)(ll * NL + l) * n;
+          const float2* const sq = sm + (size_t)(ll * NL + l) * ss;
           const float2 z1 = sq[kx], z2 = sq[kx == 0 ? 0 : n - kx];
           v = make_float4(0.5f * (z1.x + z2.x), 0.5f * (z1.y - z2.y), 0.5f * (z1.y + z2.y), 0.5f * (z2.x - z1.x));
         }
@@ -710,7 +735,7 @@ __global__ void __launch_bounds__(SpecRowBounds<PS>::threads, SpecRowBounds<PS>:
           const int kx = c / M, m = c - kx * M;
           float2 ya = make_float2(0.0f, 0.0f), yb = ya;
           if (kx < H) {
-            const float2* const sq = sm + (size_t)(lp * M + m) * n;
+            const float2* const sq = sm + (size_t)(lp * M + m) * ss;
             const float2 z1 = sq[kx], z2 = sq[kx == 0 ? 0 : n - kx];
             ya = make_float2(0.5f * (z1.x + z2.x), 0.5f * (z1.y - z2.y));
             yb = make_float2(0.5f * (z1.y + z2.y), 0.5f * (z2.x - z1.x));
