@@ -109,7 +109,10 @@ int Pipeline<T>::init(const Problem& pb, int nloads_, bool krylov, cudaStream_t 
   }
   const int M = g.M;
   const size_t smem_green = std::min<size_t>(150 * 1024, (size_t)optin - 4096);
-  // tile width C of the half spectrum
+  // Tile width C of the half spectrum: the widest (up to 15 % padding) that
+  // still leaves two column CTAs per SM, else the narrowest.  Wide tiles move
+  // longer runs of memory, but on small grids they leave most SMs without a
+  // CTA (255^2 float64, C = 16: 8 CTAs, Green pass 244 us).
   int Cc = 0;
   for (int cand : {16, 8, 4, 2, 1}) {
     if (w.C && cand != w.C) continue;
@@ -126,7 +129,8 @@ int Pipeline<T>::init(const Problem& pb, int nloads_, bool krylov, cudaStream_t 
       if (round_up(cand * M * tpc0, 32) > kColMaxThreads) continue;
     }
     Cc = cand;
-    break;
+    const long long ctas = (long long)Tt * (d == 2 ? ncell : std::min(pb.N[0], pb.N[1]));
+    if (ctas >= 2LL * sms) break;
   }
   if (Cc == 0) {
     err = "grid too large for the column tiling";
@@ -169,6 +173,7 @@ int Pipeline<T>::init(const Problem& pb, int nloads_, bool krylov, cudaStream_t 
         if (g.n1 % cand) continue;
         if ((size_t)pb.N[0] * cand * CM * esz > std::min<size_t>(100 * 1024, smem_green)) continue;
         if (round_up((int)(cand * CM) * tpc0, 32) > kColMaxThreads) continue;
+        if (cand > 1 && (long long)g.Tt * (g.n1 / cand) < 2LL * sms) continue;
         G = cand;
         break;
       }

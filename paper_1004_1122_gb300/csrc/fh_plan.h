@@ -206,7 +206,7 @@ template <typename F> inline int bank_cost(int threads, F&& addr) {
 // threads, plus `weight` times the cost of io(stride).
 template <typename F>
 inline int seq_stride(const FFTPlan& pl, int thr, int nseq, int weight, F&& io) {
-  const int threads = std::min(nseq * thr, 512);
+  const int threads = std::min(nseq * thr, 96);  // the pattern repeats
   int best = pl.n, best_cost = 1 << 30;
   for (int ss = pl.n; ss < pl.n + 16; ++ss) {
     int cost = weight * io(ss);
