@@ -13,10 +13,12 @@
 //   y  = conv10(u0)
 // conv = 3x3x3 with periodic padding (the unit cell is periodic), pool = mean
 // over 3x3x3 blocks, up = nearest-neighbour upsampling by 3.
-// The forward convolutions run on the tensor cores (fh_conv_tc.cuh: tcgen05
-// implicit GEMM, bfloat16 weights, float32 activations split into two
-// bfloat16 halves); the backward ones (data and weight gradients) on the
-// CUDA cores in float32.
+// All convolutions -- forward, data gradient and weight gradient -- run on the
+// tensor cores (fh_conv_planes.cuh: tcgen05, bfloat16 weights, float32
+// activations and gradients split into two bfloat16 halves).  The split, the
+// pooling, upsampling and skip sums and the leaky ReLU's derivative are one
+// pass that writes the operand planes of the next convolution; the forward
+// ReLU is the convolution's epilogue.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -27,7 +29,7 @@
 #include <vector>
 
 #include "../../include/fh_nn.h"
-#include "fh_conv_tc.cuh"
+#include "fh_conv_planes.cuh"
 
 namespace {
 
@@ -38,139 +40,6 @@ struct Dims {
   int n0, n1, n2;
   __host__ __device__ long long v() const { return (long long)n0 * n1 * n2; }
 };
-
-// dW[o][c][t] = sum_z gy[o](z) x[c](z + t);  db[o] = sum_z gy[o](z).
-// CTA (o, c, s) sums the 27 taps and the bias over voxel slice s of S; the
-// partials go to part[((s * O + o) * C + c) * 28 + t] and k_wgrad_reduce adds
-// the slices in a fixed order (no atomics, deterministic).
-__global__ void __launch_bounds__(kThreads) k_conv_wgrad(const float* __restrict__ x, int C,
-                                                         const float* __restrict__ gy, int O, int S,
-                                                         float* __restrict__ part, Dims dm) {
-  const int pair = blockIdx.x % (O * C), sl = blockIdx.x / (O * C);
-  const int o = pair / C, c = pair - (pair / C) * C;
-  const long long V = dm.v();
-  const long long v0 = V * sl / S, v1 = V * (sl + 1) / S;
-  const float* xc = x + (long long)c * V;
-  const float* go = gy + (long long)o * V;
-  const int plane = dm.n1 * dm.n2;
-  float acc[27];
-#pragma unroll
-  for (int t = 0; t < 27; ++t) acc[t] = 0.0f;
-  float accb = 0.0f;
-  for (long long vox = v0 + threadIdx.x; vox < v1; vox += blockDim.x) {
-    const int z = (int)(vox / plane);
-    const int rem = (int)(vox - (long long)z * plane);
-    const int yy = rem / dm.n2, xx = rem - yy * dm.n2;
-    const float g = __ldg(go + vox);
-    accb += g;
-    int xs[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      int x2 = xx + k - 1;
-      x2 += x2 < 0 ? dm.n2 : (x2 >= dm.n2 ? -dm.n2 : 0);
-      xs[k] = x2;
-    }
-#pragma unroll
-    for (int dz = 0; dz < 3; ++dz) {
-      int zz = z + dz - 1;
-      zz += zz < 0 ? dm.n0 : (zz >= dm.n0 ? -dm.n0 : 0);
-#pragma unroll
-      for (int dy = 0; dy < 3; ++dy) {
-        int y2 = yy + dy - 1;
-        y2 += y2 < 0 ? dm.n1 : (y2 >= dm.n1 ? -dm.n1 : 0);
-        const float* row = xc + (long long)(zz * dm.n1 + y2) * dm.n2;
-#pragma unroll
-        for (int k = 0; k < 3; ++k) acc[dz * 9 + dy * 3 + k] = fmaf(g, __ldg(row + xs[k]), acc[dz * 9 + dy * 3 + k]);
-      }
-    }
-  }
-  __shared__ float red[kThreads / 32][28];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int t = 0; t < 28; ++t) {
-    float v = t < 27 ? acc[t] : accb;
-#pragma unroll
-    for (int k = 16; k > 0; k >>= 1) v += __shfl_down_sync(0xffffffffu, v, k);
-    if (lane == 0) red[warp][t] = v;
-  }
-  __syncthreads();
-  if (threadIdx.x < 28) {
-    float v = 0.0f;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v += red[w][threadIdx.x];
-    part[((long long)(sl * O + o) * C + c) * 28 + threadIdx.x] = v;
-  }
-}
-
-// gW[o][c][t] = sum_s part[s][o][c][t];  gb[o] = sum_s part[s][o][0][27]
-__global__ void k_wgrad_reduce(const float* __restrict__ part, int O, int C, int S, float* __restrict__ gW,
-                               float* __restrict__ gb) {
-  const long long n = (long long)O * C * 28;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const int t = (int)(i % 28);
-    const long long oc = i / 28;
-    float v = 0.0f;
-    for (int sl = 0; sl < S; ++sl) v += part[((long long)sl * O * C + oc) * 28 + t];
-    if (t < 27) {
-      gW[oc * 27 + t] = v;
-    } else if (oc % C == 0) {
-      gb[oc / C] = v;
-    }
-  }
-}
-
-__global__ void k_leaky(const float* __restrict__ z, float* __restrict__ a, long long n) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const float v = z[i];
-    a[i] = v > 0.0f ? v : kSlope * v;
-  }
-}
-
-// g <- g * leaky'(z)
-__global__ void k_leaky_bwd(const float* __restrict__ z, float* __restrict__ g, long long n) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    if (!(z[i] > 0.0f)) g[i] *= kSlope;
-}
-
-// coarse[c][Z][Y][X] = mean of the 3x3x3 fine block (fine dims = 3 * coarse dims)
-__global__ void k_pool(const float* __restrict__ fine, float* __restrict__ coarse, int C, Dims cd) {
-  const long long Vc = cd.v();
-  const long long n = Vc * C;
-  const int f1 = 3 * cd.n1, f2 = 3 * cd.n2;
-  const long long Vf = 27 * Vc;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const int c = (int)(i / Vc);
-    const long long v = i - (long long)c * Vc;
-    const int Z = (int)(v / ((long long)cd.n1 * cd.n2));
-    const int rem = (int)(v - (long long)Z * cd.n1 * cd.n2);
-    const int Y = rem / cd.n2, X = rem - Y * cd.n2;
-    const float* fc = fine + (long long)c * Vf;
-    float s = 0.0f;
-    for (int a = 0; a < 3; ++a)
-      for (int bb = 0; bb < 3; ++bb)
-        for (int e = 0; e < 3; ++e) s += fc[((long long)(3 * Z + a) * f1 + 3 * Y + bb) * f2 + 3 * X + e];
-    coarse[i] = s * (1.0f / 27.0f);
-  }
-}
-
-// fine[c][z][y][x] = scale * coarse[c][z/3][y/3][x/3] (+ add[c][z][y][x] if add, + fine if accumulate)
-__global__ void k_up(const float* __restrict__ coarse, float* __restrict__ fine, const float* __restrict__ add,
-                     int C, Dims fd, float scale, int accumulate) {
-  const long long Vf = fd.v();
-  const long long n = Vf * C;
-  const int c1 = fd.n1 / 3, c2 = fd.n2 / 3;
-  const long long Vc = Vf / 27;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const int c = (int)(i / Vf);
-    const long long v = i - (long long)c * Vf;
-    const int z = (int)(v / ((long long)fd.n1 * fd.n2));
-    const int rem = (int)(v - (long long)z * fd.n1 * fd.n2);
-    const int y = rem / fd.n2, x = rem - y * fd.n2;
-    float s = scale * coarse[(long long)c * Vc + ((long long)(z / 3) * c1 + y / 3) * c2 + x / 3];
-    if (add) s += add[i];
-    if (accumulate) s += fine[i];
-    fine[i] = s;
-  }
-}
 
 // coarse[c][Z][Y][X] = sum of the fine block (adjoint of nearest upsampling)
 __global__ void k_up_bwd(const float* __restrict__ fine, float* __restrict__ coarse, int C, Dims cd) {
@@ -223,35 +92,6 @@ __global__ void k_adam(float* __restrict__ p, const float* __restrict__ g, float
     m[i] = mi;
     v[i] = vi;
     p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-  }
-}
-
-// Tensor-core weight layout of one layer: wt[o][t * Cp + c] = bf16(w[o][c][t]),
-// zero for o >= O or c >= C (NT rows, 27 * Cp columns).
-__global__ void k_to_bf16_tc(const float* __restrict__ w, int O, int C, int Cp, int NT,
-                             __nv_bfloat16* __restrict__ wt) {
-  const long long n = (long long)NT * 27 * Cp;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const int o = (int)(i / (27 * Cp));
-    const int k = (int)(i - (long long)o * 27 * Cp);
-    const int t = k / Cp, c = k - t * Cp;
-    const float v = (o < O && c < C) ? w[((long long)o * C + c) * 27 + t] : 0.0f;
-    wt[i] = __float2bfloat16_rn(v);
-  }
-}
-
-// Transposed layout for the data gradient gx[c] = sum_o sum_t w[o][c][t] gy[o](. - t):
-// wt[c][t * Op + o] = bf16(w[o][c][26 - t]), zero for c >= C or o >= O (NT rows
-// = C padded to 16, 27 * Op columns).
-__global__ void k_to_bf16_tc_t(const float* __restrict__ w, int O, int C, int Op, int NT,
-                               __nv_bfloat16* __restrict__ wt) {
-  const long long n = (long long)NT * 27 * Op;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const int c = (int)(i / (27 * Op));
-    const int k = (int)(i - (long long)c * 27 * Op);
-    const int t = k / Op, o = k - t * Op;
-    const float v = (o < O && c < C) ? w[((long long)o * C + c) * 27 + (26 - t)] : 0.0f;
-    wt[i] = __float2bfloat16_rn(v);
   }
 }
 
@@ -327,109 +167,182 @@ int grid1(long long n) {
 }  // namespace
 
 constexpr int kLayers = 11;
+constexpr int kStaticSmem = 10 * 1024;  // at least the convolution kernels' static shared memory
+
+using fh::tc::PlaneGeom;
 
 struct fh_nn {
   Dims lv[4];
+  PlaneGeom pg[4];                             // padded grids of the levels
   int cin = 0, cout = 0;
   int ch[4] = {16, 32, 48, 64};
   int lo[kLayers], li[kLayers], ll[kLayers];  // layer out / in channels, level
   long long woff[kLayers], boff[kLayers];      // offsets in the flat parameter vector
   long long nparam = 0;
   cudaStream_t st = nullptr;
+  int sms = 0;
+  size_t smem_cap = 0;
   float *P = nullptr, *G = nullptr, *Mo = nullptr, *Ve = nullptr;
-  __nv_bfloat16* Wtc = nullptr;                 // tensor-core weight layout, all layers
-  __nv_bfloat16* WtcT = nullptr;                // transposed (data-gradient) layout
-  long long wtc_off[kLayers], wtct_off[kLayers];// offsets (multiples of 8 elements)
-  int cpad[kLayers], ntile[kLayers];             // forward: in channels padded to 8, N tile
-  int opad[kLayers], ntile_t[kLayers];           // data gradient: out channels padded to 8, N tile
+  __nv_bfloat16* W[2][kLayers] = {};            // operand layouts: forward, data gradient
   int* dev_err = nullptr;                        // bounded waits that expired
-  float* wpart = nullptr;                        // weight-gradient partials per voxel slice
-  // forward: pre-activations z[k] (k < 10), encoder a[l], pooled pl[l],
-  // decoder sums v[l] and activations u[l], output y; tmp = leaky(up conv)
-  float *x = nullptr, *z[kLayers - 1] = {}, *a[4] = {}, *pl[3] = {}, *v[3] = {}, *u[3] = {}, *y = nullptr;
-  float* tmp = nullptr;
-  // backward
+  float* wpart[kLayers] = {};                    // weight-gradient partials
+  // the weight gradients run beside the chain of data gradients on their own stream
+  cudaStream_t side = nullptr;
+  cudaEvent_t fork[kLayers] = {}, join = nullptr;
+  // act[k]: output of layer k after the leaky ReLU; in[k]: operand planes of
+  // its input (kept for the weight gradient); y: output
+  float* act[kLayers - 1] = {};
+  uint4* in[kLayers] = {};
+  float* y = nullptr;
+  // backward: gradients, planes with periodic padding (one layer at a time)
+  // and with zero padding (per layer: the padding stays zero)
   float *gy = nullptr, *gu[3] = {}, *gv[3] = {}, *ga3 = nullptr, *gp[3] = {}, *gt = nullptr;
+  uint4 *GA = nullptr, *GB[kLayers] = {};
   double* part = nullptr;
   double* h_part = nullptr;
   int npart = 0;
-  std::vector<void*> allocs;
+  void* slab = nullptr;                          // the one allocation behind all of it
   long long launches = 0;
 };
 
 namespace {
 
-template <typename T>
-int nn_alloc(fh_nn* n, T** p, long long count) {
-  void* q = nullptr;
-  if (cudaMalloc(&q, (size_t)count * sizeof(T) + 16) != cudaSuccess) return FH_ERR_OOM;
-  n->allocs.push_back(q);
-  *p = static_cast<T*>(q);
-  return 0;
+struct ConvShape {
+  int T, sy, rows, tiles_z, grid, resident, cps, nstage;
+  size_t smem;
+};
+
+// Compiled (T, NT): two accumulators of T NT columns per CTA.
+#define FH_FOR_EACH_CONV(X) \
+  X(4, 16) X(2, 16) X(1, 16) X(4, 32) X(2, 32) X(1, 32) X(4, 48) X(2, 48) X(1, 48) X(4, 64) X(2, 64) X(1, 64)
+
+// Tile of a convolution: as many 128-voxel MMA tiles per CTA tile (4, 2, 1) as
+// still give every SM a tile -- longer tiles copy their neighbouring rows less
+// often -- with all chunks of channels in one stage where they fit and the
+// weights beside them, and two stages where those fit.
+ConvShape conv_shape(const fh_nn* n, const PlaneGeom& g, int chunks, int NT) {
+  for (int cps : {chunks, 1})
+    for (int nstage : {2, 1})
+      for (int T : {4, 2, 1})
+        for (int resident : {1, 0}) {
+          if (!resident && cps > 1) continue;
+          ConvShape c{};
+          c.T = T;
+          c.cps = cps;
+          c.nstage = nstage;
+          c.resident = resident;
+          c.rows = std::min(128 * T, g.n1 * g.px);
+          c.sy = std::min(g.px, c.rows + 2);
+          c.tiles_z = (g.n1 * g.px + 128 * T - 1) / (128 * T);
+          const long long tiles = (long long)c.tiles_z * g.n0;
+          c.grid = (int)std::min<long long>(tiles, n->sms);
+          c.smem = fh::tc::conv_smem(T, c.sy, c.rows, NT, chunks, resident != 0, cps, nstage);
+          if (c.smem <= n->smem_cap && (tiles >= n->sms || T == 1)) return c;
+        }
+  return ConvShape{};
 }
 
-cudaError_t conv(fh_nn* n, int layer, const float* in, float* out, bool trans) {
-  const int O = trans ? n->li[layer] : n->lo[layer];
-  const int C = trans ? n->lo[layer] : n->li[layer];
-  const Dims d = n->lv[n->ll[layer]];
+// y = leaky(conv(x; W) + b), or the data gradient gx = conv(gy; W^T, taps
+// reversed) of layer k; slope 1: no ReLU
+cudaError_t conv(fh_nn* n, int k, const uint4* planes, float* out, bool trans, float slope) {
+  const PlaneGeom& g = n->pg[n->ll[k]];
+  fh::tc::ConvPlanesArgs a;
+  a.g = g;
+  a.x = planes;
+  a.nblk = fh::tc::chan_blocks(trans ? n->lo[k] : n->li[k]);
+  a.w = n->W[trans][k];
+  a.O = trans ? n->li[k] : n->lo[k];
+  const int NT = (a.O + 15) / 16 * 16;
+  a.y = out;
+  a.b = trans ? nullptr : n->P + n->boff[k];
+  a.slope = slope;
+  const ConvShape c = conv_shape(n, g, a.nblk / 2, NT);
+  a.sy = c.sy;
+  a.rows = c.rows;
+  a.tiles_z = c.tiles_z;
+  a.resident = c.resident;
+  a.cps = c.cps;
+  a.nstage = c.nstage;
+  a.err = n->dev_err;
+  a.wait_ns = fh::tma::wait_limit_ns();
   ++n->launches;
-  {
-    // forward: y = conv(x; W) + b;  data gradient: gx = conv(gy; W^T, taps
-    // reversed), the same implicit GEMM with the transposed weight layout
-    fh::tc::ConvTcArgs ta;
-    ta.x = in;
-    ta.C = C;
-    ta.Cp = trans ? n->opad[layer] : n->cpad[layer];
-    ta.y = out;
-    ta.O = O;
-    ta.NT = trans ? n->ntile_t[layer] : n->ntile[layer];
-    ta.w = trans ? n->WtcT + n->wtct_off[layer] : n->Wtc + n->wtc_off[layer];
-    ta.b = trans ? nullptr : n->P + n->boff[layer];
-    ta.n0 = d.n0;
-    ta.n1 = d.n1;
-    ta.n2 = d.n2;
-    ta.err = n->dev_err;
-    ta.wait_ns = fh::tma::wait_limit_ns();
-    const unsigned g = (unsigned)((d.v() + fh::tc::kM - 1) / fh::tc::kM);
-    fh::tc::k_conv_tc<<<g, fh::tc::kThreads, fh::tc::kSmemBytes, n->st>>>(ta);
+#define FH_CONV(TT, NN) \
+  if (c.T == TT && NT == NN) fh::tc::k_conv_planes<TT, NN><<<c.grid, fh::tc::kConvThreads, c.smem, n->st>>>(a);
+  FH_FOR_EACH_CONV(FH_CONV)
+#undef FH_CONV
+  return cudaGetLastError();
+}
+
+template <int MODE>
+cudaError_t split(fh_nn* n, int level, int C, const float* src, uint4* out, const float* coarse = nullptr,
+                  const float* act = nullptr, uint4* out0 = nullptr) {
+  fh::tc::SplitArgs a;
+  a.g = n->pg[level];
+  a.C = C;
+  a.src = src;
+  a.coarse = coarse;
+  a.act = act;
+  a.out = out;
+  a.out0 = out0;
+  a.slope = kSlope;
+  const long long pv = (long long)(a.g.n0 + 2) * a.g.py * a.g.px;
+  const dim3 grid((unsigned)std::min<long long>((pv + 255) / 256, 65535), fh::tc::chan_blocks(C));
+  ++n->launches;
+  fh::tc::k_split<MODE><<<grid, 256, 0, n->st>>>(a);
+  return cudaGetLastError();
+}
+
+// CTAs of a layer's weight gradient along the voxels: one per SM and
+// (16-channel chunk, 16 outputs), at most one per voxel tile
+int wgrad_slices(const fh_nn* n, int k) {
+  const PlaneGeom& g = n->pg[n->ll[k]];
+  const int per = fh::tc::chan_blocks(n->li[k]) / 2 * (fh::tc::chan_blocks(n->lo[k]) / 2);
+  return (int)std::max<long long>(1, std::min<long long>(n->sms / per, g.v() / fh::tc::kWgK + 1));
+}
+
+cudaError_t wgrad(fh_nn* n, int k) {
+  const PlaneGeom& g = n->pg[n->ll[k]];
+  fh::tc::WgradArgs a;
+  a.g = g;
+  a.x = n->in[k];
+  a.nblk = fh::tc::chan_blocks(n->li[k]);
+  a.gy = n->GB[k];
+  a.oblk = fh::tc::chan_blocks(n->lo[k]);
+  a.O = n->lo[k];
+  a.C = n->li[k];
+  a.slices = wgrad_slices(n, k);
+  a.sy = std::min(g.px, fh::tc::kWgK);
+  a.vox = (long long)(g.n0 - 1) * g.py * g.px + (long long)(g.n1 - 1) * g.px + g.n2 + 2;
+  a.part = n->wpart[k];
+  a.err = n->dev_err;
+  a.wait_ns = fh::tma::wait_limit_ns();
+  const int chunks = a.nblk / 2;
+  ++n->launches;
+  cudaError_t e = cudaEventRecord(n->fork[k], n->st);  // GB[k] is written
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(n->side, n->fork[k], 0);
+  if (e != cudaSuccess) return e;
+  fh::tc::k_wgrad_planes<16><<<dim3(a.slices, chunks, a.oblk / 2), fh::tc::kWgThreads, fh::tc::wg_smem(a.sy, 16), n->side>>>(a);
+  return cudaGetLastError();
+}
+
+// Every layer's weight gradient from its partials; n->st waits for them.
+cudaError_t wgrad_finish(fh_nn* n) {
+  fh::tc::WgradSumArgs a;
+  for (int k = 0; k < kLayers; ++k) {
+    a.part[k] = n->wpart[k];
+    a.gW[k] = n->G + n->woff[k];
+    a.gb[k] = n->G + n->boff[k];
+    a.O[k] = n->lo[k];
+    a.C[k] = n->li[k];
+    a.slices[k] = wgrad_slices(n, k);
   }
-  return cudaGetLastError();
+  ++n->launches;
+  fh::tc::k_wgrad_sum<<<dim3(64, kLayers), 128, 0, n->side>>>(a);
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) e = cudaEventRecord(n->join, n->side);
+  return e == cudaSuccess ? cudaStreamWaitEvent(n->st, n->join, 0) : e;
 }
 
-// voxel slices per (o, c) pair: enough CTAs for ~4 per SM, at least 2048 voxels a slice
-int wgrad_slices(int O, int C, long long V) {
-  long long s = (608 + (long long)O * C - 1) / ((long long)O * C);
-  s = std::min<long long>(s, std::max<long long>(1, V / 2048));
-  return (int)std::max<long long>(1, std::min<long long>(s, 64));
-}
-
-cudaError_t wgrad(fh_nn* n, int layer, const float* in, const float* gy) {
-  const Dims d = n->lv[n->ll[layer]];
-  const int O = n->lo[layer], C = n->li[layer];
-  const int S = wgrad_slices(O, C, d.v());
-  n->launches += 2;
-  k_conv_wgrad<<<O * C * S, kThreads, 0, n->st>>>(in, C, gy, O, S, n->wpart, d);
-  k_wgrad_reduce<<<grid1((long long)O * C * 28), kThreads, 0, n->st>>>(n->wpart, O, C, S, n->G + n->woff[layer],
-                                                                       n->G + n->boff[layer]);
-  return cudaGetLastError();
-}
-
-void leaky(fh_nn* n, const float* z, float* a, long long cnt) {
-  ++n->launches;
-  k_leaky<<<grid1(cnt), kThreads, 0, n->st>>>(z, a, cnt);
-}
-void leaky_bwd(fh_nn* n, const float* z, float* g, long long cnt) {
-  ++n->launches;
-  k_leaky_bwd<<<grid1(cnt), kThreads, 0, n->st>>>(z, g, cnt);
-}
-void pool(fh_nn* n, const float* f, float* c, int C, Dims cd) {
-  ++n->launches;
-  k_pool<<<grid1(cd.v() * C), kThreads, 0, n->st>>>(f, c, C, cd);
-}
-void up(fh_nn* n, const float* c, float* f, const float* add, int C, Dims fd, float scale, int accum) {
-  ++n->launches;
-  k_up<<<grid1(fd.v() * C), kThreads, 0, n->st>>>(c, f, add, C, fd, scale, accum);
-}
 void up_bwd(fh_nn* n, const float* f, float* c, int C, Dims cd) {
   ++n->launches;
   k_up_bwd<<<grid1(cd.v() * C), kThreads, 0, n->st>>>(f, c, C, cd);
@@ -439,68 +352,76 @@ void up_bwd(fh_nn* n, const float* f, float* c, int C, Dims cd) {
 constexpr int kUp[3] = {8, 6, 4};
 constexpr int kPost[3] = {9, 7, 5};
 
-cudaError_t forward(fh_nn* n) {
-  cudaError_t e;
+#define FH_NN(call)                                  \
+  do {                                               \
+    const cudaError_t e_ = (call);                   \
+    if (e_ != cudaSuccess) return e_;                \
+  } while (0)
+
+// y = net(x), both [channels][V] on the device
+cudaError_t forward(fh_nn* n, const float* x, float* y) {
+  using namespace fh::tc;
+  WeightArgs wa;
   for (int k = 0; k < kLayers; ++k) {
-    n->launches += 2;
-    k_to_bf16_tc<<<grid1((long long)n->ntile[k] * 27 * n->cpad[k]), kThreads, 0, n->st>>>(
-        n->P + n->woff[k], n->lo[k], n->li[k], n->cpad[k], n->ntile[k], n->Wtc + n->wtc_off[k]);
-    k_to_bf16_tc_t<<<grid1((long long)n->ntile_t[k] * 27 * n->opad[k]), kThreads, 0, n->st>>>(
-        n->P + n->woff[k], n->lo[k], n->li[k], n->opad[k], n->ntile_t[k], n->WtcT + n->wtct_off[k]);
+    wa.w[k] = n->P + n->woff[k];
+    wa.out[0][k] = n->W[0][k];
+    wa.out[1][k] = n->W[1][k];
+    wa.O[k] = n->lo[k];
+    wa.C[k] = n->li[k];
   }
-  if ((e = conv(n, 0, n->x, n->z[0], false))) return e;
-  leaky(n, n->z[0], n->a[0], n->lv[0].v() * n->ch[0]);
+  ++n->launches;
+  k_weight_planes<<<dim3(32, 2 * kLayers), kThreads, 0, n->st>>>(wa);
+  FH_NN(cudaGetLastError());
+  FH_NN(split<kSplitPlain>(n, 0, n->cin, x, n->in[0]));
+  FH_NN(conv(n, 0, n->in[0], n->act[0], false, kSlope));
   for (int l = 1; l < 4; ++l) {
-    pool(n, n->a[l - 1], n->pl[l - 1], n->ch[l - 1], n->lv[l]);
-    if ((e = conv(n, l, n->pl[l - 1], n->z[l], false))) return e;
-    leaky(n, n->z[l], n->a[l], n->lv[l].v() * n->ch[l]);
+    FH_NN(split<kSplitPool>(n, l, n->ch[l - 1], n->act[l - 1], n->in[l]));
+    FH_NN(conv(n, l, n->in[l], n->act[l], false, kSlope));
   }
-  const float* in = n->a[3];
+  const float* cur = n->act[3];
   for (int l = 2; l >= 0; --l) {
     const int ku = kUp[l], kp = kPost[l];
-    // v_l = up(leaky(conv_ku(in))) + a_l ; u_l = leaky(conv_kp(v_l))
-    if ((e = conv(n, ku, in, n->z[ku], false))) return e;
-    leaky(n, n->z[ku], n->tmp, n->lv[l + 1].v() * n->ch[l]);
-    up(n, n->tmp, n->v[l], n->a[l], n->ch[l], n->lv[l], 1.0f, 0);
-    if ((e = conv(n, kp, n->v[l], n->z[kp], false))) return e;
-    leaky(n, n->z[kp], n->u[l], n->lv[l].v() * n->ch[l]);
-    in = n->u[l];
+    // v_l = up(leaky(conv_ku(cur))) + a_l ; u_l = leaky(conv_kp(v_l))
+    FH_NN(split<kSplitPlain>(n, l + 1, n->li[ku], cur, n->in[ku]));
+    FH_NN(conv(n, ku, n->in[ku], n->act[ku], false, kSlope));
+    FH_NN(split<kSplitUp>(n, l, n->ch[l], n->act[l], n->in[kp], n->act[ku]));
+    FH_NN(conv(n, kp, n->in[kp], n->act[kp], false, kSlope));
+    cur = n->act[kp];
   }
-  if ((e = conv(n, 10, n->u[0], n->y, false))) return e;
-  return cudaGetLastError();
+  FH_NN(split<kSplitPlain>(n, 0, n->ch[0], cur, n->in[10]));
+  return conv(n, 10, n->in[10], y, false, 1.0f);
 }
 
 // gradients of sum(gy * y) (gy already in n->gy)
 cudaError_t backward(fh_nn* n) {
-  cudaError_t e;
-  if ((e = wgrad(n, 10, n->u[0], n->gy))) return e;
-  if ((e = conv(n, 10, n->gy, n->gu[0], true))) return e;        // g_u0
+  using namespace fh::tc;
+  FH_NN(split<kSplitPlain>(n, 0, n->cout, n->gy, n->GA, nullptr, nullptr, n->GB[10]));
+  FH_NN(wgrad(n, 10));
+  FH_NN(conv(n, 10, n->GA, n->gu[0], true, 1.0f));               // g_u0
   for (int l = 0; l < 3; ++l) {
     const int ku = kUp[l], kp = kPost[l];
-    const long long Vl = n->lv[l].v(), Vc = n->lv[l + 1].v();
-    leaky_bwd(n, n->z[kp], n->gu[l], Vl * n->ch[l]);               // -> g_z(post)
-    if ((e = wgrad(n, kp, n->v[l], n->gu[l]))) return e;
-    if ((e = conv(n, kp, n->gu[l], n->gv[l], true))) return e;     // g_v_l (= skip part of g_a_l)
-    up_bwd(n, n->gv[l], n->gt, n->ch[l], n->lv[l + 1]);             // c_l at level l+1
-    leaky_bwd(n, n->z[ku], n->gt, Vc * n->ch[l]);                   // -> g_z(up)
-    const float* up_in = l < 2 ? n->u[l + 1] : n->a[3];
-    if ((e = wgrad(n, ku, up_in, n->gt))) return e;
-    float* g_in = l < 2 ? n->gu[l + 1] : n->ga3;
-    if ((e = conv(n, ku, n->gt, g_in, true))) return e;            // g_u_{l+1} (or g_a3)
+    FH_NN(split<kSplitGrad>(n, l, n->ch[l], n->gu[l], n->GA, nullptr, n->act[kp], n->GB[kp]));  // g_z(post)
+    FH_NN(wgrad(n, kp));
+    FH_NN(conv(n, kp, n->GA, n->gv[l], true, 1.0f));              // g_v_l (= skip part of g_a_l)
+    up_bwd(n, n->gv[l], n->gt, n->ch[l], n->lv[l + 1]);           // c_l at level l+1
+    FH_NN(split<kSplitGrad>(n, l + 1, n->ch[l], n->gt, n->GA, nullptr, n->act[ku], n->GB[ku]));  // g_z(up)
+    FH_NN(wgrad(n, ku));
+    FH_NN(conv(n, ku, n->GA, l < 2 ? n->gu[l + 1] : n->ga3, true, 1.0f));  // g_u_{l+1} (or g_a3)
   }
   // encoder: g_a3 in ga3; g_a_l = g_v_l + poolT(g_p_l)
-  float* g_a = n->ga3;
   for (int l = 3; l >= 1; --l) {
-    leaky_bwd(n, n->z[l], g_a, n->lv[l].v() * n->ch[l]);          // -> g_z_l
-    if ((e = wgrad(n, l, n->pl[l - 1], g_a))) return e;
-    if ((e = conv(n, l, g_a, n->gp[l - 1], true))) return e;      // g_p_{l-1}
-    up(n, n->gp[l - 1], n->gv[l - 1], nullptr, n->ch[l - 1], n->lv[l - 1], 1.0f / 27.0f, 1);
-    g_a = n->gv[l - 1];
+    if (l == 3)
+      FH_NN(split<kSplitGrad>(n, 3, n->ch[3], n->ga3, n->GA, nullptr, n->act[3], n->GB[3]));
+    else
+      FH_NN(split<kSplitGradUp>(n, l, n->ch[l], n->gv[l], n->GA, n->gp[l], n->act[l], n->GB[l]));
+    FH_NN(wgrad(n, l));
+    FH_NN(conv(n, l, n->GA, n->gp[l - 1], true, 1.0f));           // g_p_{l-1}
   }
-  leaky_bwd(n, n->z[0], g_a, n->lv[0].v() * n->ch[0]);            // -> g_z0
-  if ((e = wgrad(n, 0, n->x, g_a))) return e;
-  return cudaGetLastError();
+  FH_NN(split<kSplitGradUp>(n, 0, n->ch[0], n->gv[0], nullptr, n->gp[0], n->act[0], n->GB[0]));
+  FH_NN(wgrad(n, 0));
+  return wgrad_finish(n);
 }
+#undef FH_NN
 
 // true when a kernel's bounded wait expired (synchronises the stream)
 bool device_error(fh_nn* n) {
@@ -532,7 +453,12 @@ extern "C" {
 void fh_nn_destroy(fh_nn* n) {
   if (!n) return;
   if (n->st) cudaStreamSynchronize(n->st);
-  for (void* p : n->allocs) cudaFree(p);
+  if (n->side) cudaStreamSynchronize(n->side);
+  if (n->slab) cudaFree(n->slab);
+  for (cudaEvent_t e : n->fork)
+    if (e) cudaEventDestroy(e);
+  if (n->join) cudaEventDestroy(n->join);
+  if (n->side) cudaStreamDestroy(n->side);
   if (n->h_part) cudaFreeHost(n->h_part);
   delete n;
 }
@@ -574,57 +500,89 @@ fh_status fh_nn_create(fh_nn** out, const int* N, int cin, int cout, const int* 
     off += n->lo[k];
   }
   n->nparam = off;
-  long long toff = 0, ttoff = 0;
-  for (int k = 0; k < kLayers; ++k) {
-    n->cpad[k] = (n->li[k] + 7) / 8 * 8;
-    n->ntile[k] = (n->lo[k] + 15) / 16 * 16;
-    n->opad[k] = (n->lo[k] + 7) / 8 * 8;
-    n->ntile_t[k] = (n->li[k] + 15) / 16 * 16;
-    n->wtc_off[k] = toff;
-    toff += (long long)n->ntile[k] * 27 * n->cpad[k];
-    n->wtct_off[k] = ttoff;
-    ttoff += (long long)n->ntile_t[k] * 27 * n->opad[k];
-    if (n->ntile[k] > fh::tc::kNmax || n->ntile_t[k] > fh::tc::kNmax) {
+  for (int k = 0; k < kLayers; ++k)
+    if (n->lo[k] > fh::tc::kNmax || n->li[k] > fh::tc::kNmax) {
       delete n;
       return FH_ERR_ARG;  // more than 64 channels on one side of a layer
     }
-  }
+  for (int l = 0; l < 4; ++l) n->pg[l] = fh::tc::plane_geom(n->lv[l].n0, n->lv[l].n1, n->lv[l].n2);
   n->st = (cudaStream_t)stream;
-  int rc = 0;
+  int dev = 0, optin = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&n->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+#define FH_CONV(TT, NN)                                                                          \
+  cudaFuncSetAttribute(fh::tc::k_conv_planes<TT, NN>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
+                       optin - kStaticSmem) != cudaSuccess ||
+      FH_FOR_EACH_CONV(FH_CONV)
+#undef FH_CONV
+      cudaFuncSetAttribute(fh::tc::k_wgrad_planes<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - kStaticSmem) !=
+          cudaSuccess) {
+    delete n;
+    return FH_ERR_CUDA;
+  }
+  n->smem_cap = (size_t)optin - kStaticSmem;
   const long long V[4] = {n->lv[0].v(), n->lv[1].v(), n->lv[2].v(), n->lv[3].v()};
   long long coarse_max = 0;  // largest c_l * |level l+1|
   for (int l = 0; l < 3; ++l) coarse_max = std::max(coarse_max, (long long)n->ch[l] * V[l + 1]);
-  rc |= nn_alloc(n, &n->P, off);
-  rc |= nn_alloc(n, &n->G, off);
-  rc |= nn_alloc(n, &n->Mo, off);
-  rc |= nn_alloc(n, &n->Ve, off);
-  rc |= nn_alloc(n, &n->Wtc, toff);
-  rc |= nn_alloc(n, &n->WtcT, ttoff);
-  {
-    long long wp = 0;
-    for (int k = 0; k < kLayers; ++k)
-      wp = std::max(wp, (long long)wgrad_slices(n->lo[k], n->li[k], V[n->ll[k]]) * n->lo[k] * n->li[k] * 28);
-    rc |= nn_alloc(n, &n->wpart, wp);
+  // one allocation; the operand planes come first (their padding and slack
+  // start as zeros, and the zero-padded planes' padding stays zero)
+  struct Want {
+    void** p;
+    size_t bytes;
+  };
+  std::vector<Want> want;
+  size_t total = 0, planes = 0;
+  auto need = [&](auto** p, long long count) {
+    const size_t bytes = ((size_t)count * sizeof(**p) + 255) / 256 * 256;
+    want.push_back({reinterpret_cast<void**>(p), bytes});
+    total += bytes;
+  };
+  long long ga = 0;
+  for (int k = 0; k < kLayers; ++k) {
+    const PlaneGeom& g = n->pg[n->ll[k]];
+    need(&n->in[k], fh::tc::plane_elems(g, n->li[k]));
+    need(&n->GB[k], fh::tc::plane_elems(g, n->lo[k]));
+    ga = std::max(ga, fh::tc::plane_elems(g, n->lo[k]));
   }
-  rc |= nn_alloc(n, &n->dev_err, 1);
-  rc |= nn_alloc(n, &n->x, V[0] * cin);
-  for (int k = 0; k < kLayers - 1; ++k) rc |= nn_alloc(n, &n->z[k], V[n->ll[k]] * (long long)n->lo[k]);
-  for (int k = 0; k < 4; ++k) rc |= nn_alloc(n, &n->a[k], V[k] * n->ch[k]);
-  for (int k = 0; k < 3; ++k) rc |= nn_alloc(n, &n->pl[k], V[k + 1] * n->ch[k]);
-  for (int k = 0; k < 3; ++k) rc |= nn_alloc(n, &n->v[k], V[k] * n->ch[k]);
-  for (int k = 0; k < 3; ++k) rc |= nn_alloc(n, &n->u[k], V[k] * n->ch[k]);
-  rc |= nn_alloc(n, &n->y, V[0] * cout);
-  rc |= nn_alloc(n, &n->tmp, coarse_max);
-  rc |= nn_alloc(n, &n->gy, V[0] * cout);
-  for (int k = 0; k < 3; ++k) rc |= nn_alloc(n, &n->gu[k], V[k] * n->ch[k]);
-  for (int k = 0; k < 3; ++k) rc |= nn_alloc(n, &n->gv[k], V[k] * n->ch[k]);
-  rc |= nn_alloc(n, &n->ga3, V[3] * n->ch[3]);
-  for (int k = 0; k < 3; ++k) rc |= nn_alloc(n, &n->gp[k], V[k + 1] * n->ch[k]);
-  rc |= nn_alloc(n, &n->gt, coarse_max);
+  need(&n->GA, ga);
+  planes = total;
+  for (int k = 0; k < kLayers; ++k) {
+    need(&n->wpart[k], (long long)wgrad_slices(n, k) * (fh::tc::chan_blocks(n->li[k]) / 2) * 9 * 128 *
+                           (fh::tc::chan_blocks(n->lo[k]) * 8));
+    const int o16 = (n->lo[k] + 15) / 16 * 16, i16 = (n->li[k] + 15) / 16 * 16;
+    need(&n->W[0][k], (long long)27 * o16 * i16);
+    need(&n->W[1][k], (long long)27 * o16 * i16);
+  }
+  need(&n->P, off);
+  need(&n->G, off);
+  need(&n->Mo, off);
+  need(&n->Ve, off);
+  need(&n->dev_err, 1);
+  for (int k = 0; k < kLayers - 1; ++k) need(&n->act[k], V[n->ll[k]] * (long long)n->lo[k]);
+  need(&n->y, V[0] * cout);
+  need(&n->gy, V[0] * cout);
+  for (int k = 0; k < 3; ++k) need(&n->gu[k], V[k] * n->ch[k]);
+  for (int k = 0; k < 3; ++k) need(&n->gv[k], V[k] * n->ch[k]);
+  need(&n->ga3, V[3] * n->ch[3]);
+  for (int k = 0; k < 3; ++k) need(&n->gp[k], V[k + 1] * n->ch[k]);
+  need(&n->gt, coarse_max);
   n->npart = 4096;
-  rc |= nn_alloc(n, &n->part, n->npart);
+  need(&n->part, n->npart);
+  int rc = cudaMalloc(&n->slab, total) == cudaSuccess ? 0 : FH_ERR_OOM;
+  if (!rc) {
+    char* q = static_cast<char*>(n->slab);
+    for (const Want& w : want) {
+      *w.p = q;
+      q += w.bytes;
+    }
+  }
+  for (int k = 0; k <= kLayers && !rc; ++k)
+    if (cudaEventCreateWithFlags(k < kLayers ? &n->fork[k] : &n->join, cudaEventDisableTiming) != cudaSuccess) rc = FH_ERR_CUDA;
+  if (!rc && cudaStreamCreateWithFlags(&n->side, cudaStreamNonBlocking) != cudaSuccess) rc = FH_ERR_CUDA;
   if (!rc && cudaMallocHost(&n->h_part, n->npart * sizeof(double)) != cudaSuccess) rc = FH_ERR_OOM;
-  if (!rc && (cudaMemsetAsync(n->dev_err, 0, sizeof(int), n->st) != cudaSuccess ||
+  if (!rc && (cudaMemsetAsync(n->slab, 0, planes, n->st) != cudaSuccess ||
+              cudaMemsetAsync(n->dev_err, 0, sizeof(int), n->st) != cudaSuccess ||
               cudaMemsetAsync(n->Mo, 0, off * sizeof(float), n->st) != cudaSuccess ||
               cudaMemsetAsync(n->Ve, 0, off * sizeof(float), n->st) != cudaSuccess ||
               cudaMemsetAsync(n->P, 0, off * sizeof(float), n->st) != cudaSuccess))
@@ -661,21 +619,12 @@ fh_status fh_nn_get_params(fh_nn* n, float* host, long long count) {
 
 fh_status fh_nn_forward(fh_nn* n, const float* x, float* y) {
   if (!n || !x || !y) return FH_ERR_ARG;
-  const long long Vx = n->lv[0].v() * n->cin, Vy = n->lv[0].v() * n->cout;
-  if (cudaMemcpyAsync(n->x, x, Vx * sizeof(float), cudaMemcpyDeviceToDevice, n->st) != cudaSuccess)
-    return FH_ERR_CUDA;
-  if (forward(n) != cudaSuccess) return FH_ERR_CUDA;
-  if (cudaMemcpyAsync(y, n->y, Vy * sizeof(float), cudaMemcpyDeviceToDevice, n->st) != cudaSuccess)
-    return FH_ERR_CUDA;
-  return FH_OK;
+  return forward(n, x, y) == cudaSuccess ? FH_OK : FH_ERR_CUDA;
 }
 
 fh_status fh_nn_gradients(fh_nn* n, const float* x, const float* target, double* loss, float* grad_host) {
   if (!n || !x || !target) return FH_ERR_ARG;
-  const long long Vx = n->lv[0].v() * n->cin;
-  if (cudaMemcpyAsync(n->x, x, Vx * sizeof(float), cudaMemcpyDeviceToDevice, n->st) != cudaSuccess)
-    return FH_ERR_CUDA;
-  if (forward(n) != cudaSuccess) return FH_ERR_CUDA;
+  if (forward(n, x, n->y) != cudaSuccess) return FH_ERR_CUDA;
   int rc = loss_grad(n, target, loss);
   if (rc) return (fh_status)rc;
   if (backward(n) != cudaSuccess) return FH_ERR_CUDA;
