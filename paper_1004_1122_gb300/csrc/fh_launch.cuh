@@ -51,6 +51,7 @@ struct LaunchTable {
 // pass with this plan and launch?
 cudaError_t spec_inv(int mode, const Launch&, const SpecArgs&, cudaStream_t);
 cudaError_t spec_fwd(int mode, const Launch&, const SpecArgs&, cudaStream_t);
+cudaError_t spec_green(const Launch&, const SpecArgs&, cudaStream_t);
 cudaError_t spec_col_set_smem(const SpecArgs&, size_t bytes);
 bool spec_col_ct(const FFTPlan&);
 cudaError_t spec_mid(bool inv, const Launch&, const SpecMidArgs&, cudaStream_t);

@@ -239,6 +239,7 @@ struct Pipeline {
   // norms through it.  x stays the field; the iteration's scalar arrays live in
   // the r, p, ap and p2 buffers.
   bool want_spectral = false;
+  bool spec_ops = false;       // the frequency-layout passes are set up (float32)
   bool spectral = false;
   bool spec_run_ = false;      // the solve in progress uses it
   SpecGeom sg{};
@@ -302,7 +303,6 @@ struct Pipeline {
   // back-to-back launches of one piece of the CG iteration:
   // 0 row_fwd (direction update + dL + FFT), 1 column passes (Green),
   // 2 row_inv (inverse FFT + A p + dot), 3 CG vector update, 5 operator apply.
-  static constexpr int kProfileSpectral = 6;  // internal: the passes of one frequency-domain iteration
   int profile(int what, int reps, double* ms, std::string& err);
 };
 

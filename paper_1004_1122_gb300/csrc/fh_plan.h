@@ -41,15 +41,10 @@ inline bool factorable(int n, bool& ext) {
   return n == 1;
 }
 
-// Minimum-stage radix schedule for length n when each sequence is worked on
-// by tpl threads: a stage of radix R is allowed iff every thread holds at most
-// floor(budget / R) butterflies, i.e. ceil(n / R / tpl) * R <= budget.
-// Returns the stage list (empty if impossible).  Radices are emitted largest
-// first.  Dynamic programme over the divisors m of n: best[m] is a shortest
-// list of allowed radices whose product is m.
-inline std::vector<int> plan_radices(int n, int tpl, int budget) {
-  bool ext;
-  if (!factorable(n, ext)) return {};
+// Radices of a plan whose sequences are worked on by tpl threads each: a stage
+// of radix R is allowed iff every thread holds at most floor(budget / R)
+// butterflies, i.e. ceil(n / R / tpl) * R <= budget.
+inline std::vector<int> allowed_radices(int n, int tpl, int budget) {
   std::vector<int> allowed;
   for (int R : compiled_radices()) {
     if (n % R) continue;
@@ -59,6 +54,13 @@ inline std::vector<int> plan_radices(int n, int tpl, int budget) {
     if (need > bmax) continue;
     allowed.push_back(R);
   }
+  return allowed;
+}
+
+// Minimum-stage radix schedule for length n from these radices (empty if
+// impossible), largest radix first.  Dynamic programme over the divisors m of
+// n: best[m] is a shortest list of allowed radices whose product is m.
+inline std::vector<int> plan_radices(int n, const std::vector<int>& allowed) {
   std::vector<int> divs;
   for (int m = 1; m <= n; ++m)
     if (n % m == 0) divs.push_back(m);  // ascending
@@ -99,10 +101,15 @@ inline bool make_fft_plan(int n, bool fp64, int max_tpl, FFTPlan& pl, int& tpl,
   small = small && !ext;
   const int budget = small ? kSmallBudget : ext ? reg_budget_x(fp64) : reg_budget(fp64);
   int best_stages = 1 << 30, best_tpl = 0;
-  std::vector<int> best_r;
+  std::vector<int> best_r, last;
   for (int t = 1; t <= max_tpl; ++t) {
     if (force_tpl && t != force_tpl) continue;
-    std::vector<int> r = plan_radices(n, t, budget);
+    // the same radices as for fewer threads: the same plan (trying all 1024
+    // thread counts took 3 ms for n = 2187)
+    std::vector<int> allowed = allowed_radices(n, t, budget);
+    if (allowed == last) continue;
+    last.swap(allowed);
+    const std::vector<int> r = plan_radices(n, last);
     if (r.empty()) continue;
     if ((int)r.size() < best_stages) {
       best_stages = (int)r.size();

@@ -27,9 +27,17 @@ cudaError_t spec_fwd(int mode, const Launch& L, const SpecArgs& a, cudaStream_t 
   });
 }
 
+cudaError_t spec_green(const Launch& L, const SpecArgs& a, cudaStream_t st) {
+  return on_plan<SpecPlans, true>(a.plan, [&](auto t) {
+    k_spec_green<decltype(t)><<<L.grid, L.block, L.smem, st>>>(a);
+    return cudaGetLastError();
+  });
+}
+
 cudaError_t spec_col_set_smem(const SpecArgs& a, size_t bytes) {
   cudaError_t e = on_plan<SpecPlans, true>(a.plan, [&](auto t) {
-    cudaError_t e2 = opt_in_smem(k_spec_inv<kSpecUpdate, decltype(t)>, bytes);
+    cudaError_t e2 = opt_in_smem(k_spec_green<decltype(t)>, bytes);
+    if (e2 == cudaSuccess) e2 = opt_in_smem(k_spec_inv<kSpecUpdate, decltype(t)>, bytes);
     return e2 == cudaSuccess ? opt_in_smem(k_spec_fwd<kSpecApply, decltype(t)>, bytes) : e2;
   });
   if (e != cudaSuccess) return e;

@@ -12,13 +12,19 @@ template <int D, int NL, typename Plans> struct SpecRows {
   template <typename F> static cudaError_t hot(const FFTPlan& pl, const Launch& L, F&& f) {
     return L.block <= kSpecRowCtThreads ? on_plan<Plans, kX>(pl, f) : on_plan<PlanList<>, kX>(pl, f);
   }
+  // the load and add passes: compile-time plans for one load (the operator's
+  // product), else run-time plans (twice per solve)
+  template <typename F> static cudaError_t ends(const FFTPlan& pl, const Launch& L, F&& f) {
+    if constexpr (NL == 1) return hot(pl, L, f);
+    return on_plan<PlanList<>, kX>(pl, f);
+  }
   static cudaError_t run(int mode, const Launch& L, const SpecRowArgs& a, cudaStream_t st) {
     if (mode == kSpecRowTau)
       return hot(a.plan, L, [&](auto t) {
         k_spec_row<D, NL, kSpecRowTau, decltype(t)><<<L.grid, L.block, L.smem, st>>>(a);
         return cudaGetLastError();
       });
-    return on_plan<PlanList<>, kX>(a.plan, [&](auto t) {
+    return ends(a.plan, L, [&](auto t) {
       if (mode == kSpecRowLoad)
         k_spec_row<D, NL, kSpecRowLoad, decltype(t)><<<L.grid, L.block, L.smem, st>>>(a);
       else
@@ -29,7 +35,7 @@ template <int D, int NL, typename Plans> struct SpecRows {
   static cudaError_t set_smem(const SpecRowArgs& a, const Launch& L) {
     cudaError_t e = hot(a.plan, L, [&](auto t) { return opt_in_smem(k_spec_row<D, NL, kSpecRowTau, decltype(t)>, L.smem); });
     if (e != cudaSuccess) return e;
-    return on_plan<PlanList<>, kX>(a.plan, [&](auto t) {
+    return ends(a.plan, L, [&](auto t) {
       cudaError_t e2 = opt_in_smem(k_spec_row<D, NL, kSpecRowLoad, decltype(t)>, L.smem);
       return e2 == cudaSuccess ? opt_in_smem(k_spec_row<D, NL, kSpecRowAdd, decltype(t)>, L.smem) : e2;
     });

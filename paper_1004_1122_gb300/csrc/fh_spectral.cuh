@@ -418,6 +418,69 @@ __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_fwd(SpecArgs a
   }
 }
 
+// Green operator on a two-channel spectrum (the operator's product): forward
+// FFT along axis 0, y^ = xi (xi . tau^) / (xi . L0 . xi) / |N|, inverse FFT.
+// 3-D: two channels per frequency (xi_0 is the FFT axis, the other two
+// components enter projected), 10 us on 63x135x105 where the three-channel
+// pass took 21 us; 2-D 49 us on 2187^2, bound by the shared-memory stages.
+template <typename PS = DynPlan>
+__global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_green(SpecArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float2* sm = reinterpret_cast<float2*>(smem_raw);
+  const int n = plan_len<PS>(a.plan), C = a.sg.C, nl = a.nl;
+  const int Q = 2 * nl * C, wpr = nl * C;
+  const SpecTile tl = spec_tile(a, n);
+  float4* const S = reinterpret_cast<float4*>(a.S) + (tl.line0 * a.sg.Hp + tl.t * C) * nl;
+  const long long rs = (long long)tl.step * a.sg.Hp * nl;
+  constexpr int kUnroll = 4;
+  {
+    SpecWalk w(wpr);
+    while (w.i < n) {
+      float4 buf[kUnroll];
+      int at[kUnroll];
+#pragma unroll
+      for (int u = 0; u < kUnroll; ++u) {
+        at[u] = w.i < n ? 2 * w.j * a.ss + w.i : -1;
+        if (w.i < n) buf[u] = S[w.i * rs + w.j];
+        w.next();
+      }
+#pragma unroll
+      for (int u = 0; u < kUnroll; ++u)
+        if (at[u] >= 0) {
+          sm[at[u]] = make_float2(buf[u].x, buf[u].y);
+          sm[at[u] + a.ss] = make_float2(buf[u].z, buf[u].w);
+        }
+    }
+  }
+  __syncthreads();
+  spec_col_fft<false, PS>(sm, a.ss, n, Q, a.plan, a.tpc, a.tw);
+  {
+    const int csh = a.sg.csh;
+    const int e = threadIdx.x & (C - 1), row0 = threadIdx.x >> csh, drow = blockDim.x >> csh;
+    SpecFreq fq;
+    fq.init(a, a.med[tl.cell], n, tl.t * C + e, tl.inner);
+    const float c1 = fq.c1, L00 = fq.L00, L01 = fq.L01, L11 = fq.L11;
+    for (int l = 0; l < nl; ++l) {
+      float2* const ch = sm + (size_t)(e * nl + l) * 2 * a.ss;
+      for (int i = row0; i < n; i += drow) {
+        const float2 v0 = ch[i], v1 = ch[a.ss + i];
+        const float x0 = fq.xi0(i);
+        const bool zero = fq.dead || i == fq.nyq || (i == 0 && fq.zero0);
+        const float f = zero ? 0.0f : a.sg.inv_nodes / (x0 * (L00 * x0 + L01) + L11);
+        const float2 w = make_float2((x0 * v0.x + c1 * v1.x) * f, (x0 * v0.y + c1 * v1.y) * f);
+        ch[i] = make_float2(x0 * w.x, x0 * w.y);
+        ch[a.ss + i] = make_float2(c1 * w.x, c1 * w.y);
+      }
+    }
+  }
+  __syncthreads();
+  spec_col_fft<true, PS>(sm, a.ss, n, Q, a.plan, a.tpc, a.tw);
+  for (SpecWalk w(wpr); w.i < n; w.next()) {
+    const float2 v0 = sm[2 * w.j * a.ss + w.i], v1 = sm[(2 * w.j + 1) * a.ss + w.i];
+    S[w.i * rs + w.j] = make_float4(v0.x, v0.y, v1.x, v1.y);
+  }
+}
+
 // ----------------------------------------------------------------------------
 // 3-D: passes along axis 1 between the two-channel and the three-component
 // spectra; one CTA per (tile, i0), rows of C frequencies.
@@ -517,16 +580,17 @@ struct SpecRowArgs {
   const float2* tw;
   float2* S;                   // D components per load, in place
   const uint8_t* phase;
-  const float* tab;            // dL per phase
+  const float* tab;            // per-phase tensors, or nullptr
   int nphase;
-  float* f[kMaxLoads];         // kSpecRowLoad: fields read; kSpecRowAdd: fields added to
+  const float* in[kMaxLoads];  // kSpecRowLoad, kSpecRowAdd: fields
+  float* out[kMaxLoads];       // kSpecRowAdd: results (may be the fields)
   Scal* scal;
 };
 
 enum : int {
   kSpecRowTau = 0,   // S <- F[dL F^-1 S] along the lines
-  kSpecRowLoad = 1,  // S <- F f
-  kSpecRowAdd = 2    // f += F^-1 S
+  kSpecRowLoad = 1,  // S <- F in, or F[tab in] when there is a table
+  kSpecRowAdd = 2    // out = in + F^-1 S, or in + tab F^-1 S
 };
 
 // Complex sequences: 2-D, one per (line, load), its two components as real and
@@ -560,7 +624,7 @@ __global__ void __launch_bounds__(SpecRowBounds<PS>::threads, SpecRowBounds<PS>:
   if (MODE == kSpecRowTau && all_done(a.scal + cell * NL, NL)) return;
   float* const stab = reinterpret_cast<float*>(sm + (((size_t)nseq * ss + 1) & ~(size_t)1));  // 16-byte aligned
   uint8_t* const sph = reinterpret_cast<uint8_t*>(stab + a.nphase * D * D);
-  if (MODE == kSpecRowTau) {
+  if (MODE == kSpecRowTau || a.tab != nullptr) {
     const float* const tabc = a.tab + (size_t)cell * g.tab_stride;
     for (int i = threadIdx.x; i < a.nphase * D * D; i += nthr) stab[i] = tabc[i];
     // phases of the CTA's lines (consecutive in the image)
@@ -635,17 +699,55 @@ __global__ void __launch_bounds__(SpecRowBounds<PS>::threads, SpecRowBounds<PS>:
       }
     }
   } else {
-    for (int ll = 0; ll < lpc; ++ll) {
-      const bool ok = line0 + ll < g.nlines;
-      const long long lo = (long long)(line0 + ll) * n;
+    // 1. the fields' lines (polarised when there is a table) into the sequences
+    if (a.tab != nullptr) __syncthreads();
+    constexpr int kLines = D == 2 ? 1 : 2;   // lines packed into one sequence set
+    constexpr int kUnrollF = 2;
+    for (int lp = 0; lp < lpc / kLines; ++lp)
 #pragma unroll
-      for (int m = 0; m < M; ++m) {
-        const float* const src = a.f[m / D] + (m % D) * g.nodes + lo;
-        const int s = D == 2 ? ll * NL + m / 2 : (ll / 2) * M + m, half = D == 2 ? m & 1 : ll & 1;
-        for (int i = threadIdx.x; i < n; i += nthr)
-          reinterpret_cast<float*>(sm + (size_t)s * ss + i)[half] = ok ? src[i] : 0.0f;
+      for (int l = 0; l < NL; ++l) {
+        const float* const src = a.in[l];
+        for (int i0 = threadIdx.x; i0 < n; i0 += kUnrollF * nthr) {
+          float v[kUnrollF][kLines][D];
+#pragma unroll
+          for (int u = 0; u < kUnrollF; ++u)
+#pragma unroll
+            for (int h = 0; h < kLines; ++h)
+#pragma unroll
+              for (int c = 0; c < D; ++c) {
+                const int i = i0 + u * nthr, line = line0 + lp * kLines + h;
+                v[u][h][c] = (i < n && line < g.nlines) ? __ldg(src + c * g.nodes + (long long)line * n + i) : 0.0f;
+              }
+#pragma unroll
+          for (int u = 0; u < kUnrollF; ++u) {
+            const int i = i0 + u * nthr;
+            if (i >= n) continue;
+            if (a.tab != nullptr) {
+#pragma unroll
+              for (int h = 0; h < kLines; ++h) {
+                const int ll = lp * kLines + h;
+                const float* const row = stab + (line0 + ll < g.nlines ? sph[ll * n + i] : 0) * (D * D);
+                float t[D];
+#pragma unroll
+                for (int c = 0; c < D; ++c) {
+                  t[c] = 0.0f;
+#pragma unroll
+                  for (int b2 = 0; b2 < D; ++b2) t[c] += row[c * D + b2] * v[u][h][b2];
+                }
+#pragma unroll
+                for (int c = 0; c < D; ++c) v[u][h][c] = t[c];
+              }
+            }
+            if constexpr (D == 2) {
+              sm[(size_t)(lp * NL + l) * ss + i] = make_float2(v[u][0][0], v[u][0][1]);
+            } else {
+#pragma unroll
+              for (int c = 0; c < D; ++c)
+                sm[(size_t)(lp * M + l * D + c) * ss + i] = make_float2(v[u][0][c], v[u][kLines - 1][c]);
+            }
+          }
+        }
       }
-    }
   }
   __syncthreads();
 
@@ -656,16 +758,51 @@ __global__ void __launch_bounds__(SpecRowBounds<PS>::threads, SpecRowBounds<PS>:
     fft_plan<false, float, PS>(seq, 1, a.plan, u, tpl, a.tw);
   } else if constexpr (MODE == kSpecRowAdd) {
     fft_plan<true, float, PS>(seq, 1, a.plan, u, tpl, a.tw);
+    constexpr int kUnrollF = 2;
     for (int ll = 0; ll < lpc; ++ll) {
       if (line0 + ll >= g.nlines) break;
       const long long lo = (long long)(line0 + ll) * n;
 #pragma unroll
-      for (int m = 0; m < M; ++m) {
-        float* const dst = a.f[m / D] + (m % D) * g.nodes + lo;
-        const int q = D == 2 ? ll * NL + m / 2 : (ll / 2) * M + m, half = D == 2 ? m & 1 : ll & 1;
-        for (int i = threadIdx.x; i < n; i += nthr)
-          dst[i] += reinterpret_cast<const float*>(sm + (size_t)q * ss + i)[half];
-      }
+      for (int l = 0; l < NL; ++l)
+        for (int i0 = threadIdx.x; i0 < n; i0 += kUnrollF * nthr) {
+          float e[kUnrollF][D];
+#pragma unroll
+          for (int q = 0; q < kUnrollF; ++q)
+#pragma unroll
+            for (int c = 0; c < D; ++c) {
+              const int i = i0 + q * nthr;
+              e[q][c] = i < n ? a.in[l][c * g.nodes + lo + i] : 0.0f;
+            }
+#pragma unroll
+          for (int q = 0; q < kUnrollF; ++q) {
+            const int i = i0 + q * nthr;
+            if (i >= n) continue;
+            float y[D];
+            if constexpr (D == 2) {
+              const float2 v = sm[(size_t)(ll * NL + l) * ss + i];
+              y[0] = v.x;
+              y[1] = v.y;
+            } else {
+#pragma unroll
+              for (int c = 0; c < D; ++c)
+                y[c] = reinterpret_cast<const float*>(sm + (size_t)((ll / 2) * M + l * D + c) * ss + i)[ll & 1];
+            }
+            if (a.tab != nullptr) {
+              const float* const row = stab + sph[ll * n + i] * (D * D);
+              float t[D];
+#pragma unroll
+              for (int c = 0; c < D; ++c) {
+                t[c] = 0.0f;
+#pragma unroll
+                for (int b2 = 0; b2 < D; ++b2) t[c] += row[c * D + b2] * y[b2];
+              }
+#pragma unroll
+              for (int c = 0; c < D; ++c) y[c] = t[c];
+            }
+#pragma unroll
+            for (int c = 0; c < D; ++c) a.out[l][c * g.nodes + lo + i] = e[q][c] + y[c];
+          }
+        }
     }
     return;
   } else if constexpr (D == 2) {

@@ -74,3 +74,23 @@ def test_all_loads_match_single_loads(N):
         cols = [s.solve(e, tol=1e-9, want_field=False)[1] for e in np.eye(len(N))]
     assert all(i["status"] == "FH_OK" for i in infos)
     assert np.max(np.abs(Le - np.stack(cols, axis=1))) <= 1e-7 * np.max(np.abs(Le))
+
+
+@pytest.mark.parametrize("N", [(75, 81), (405, 225), (135, 3), (25, 75, 81), (81, 27, 135), (3, 135, 75), (5, 7, 3)])
+@pytest.mark.parametrize("transpose", [False, True])
+def test_float32_product_in_place(N, transpose):
+    """The operator's product on the same passes.  Bound: 64 u (1 + max|dL|)
+    max|e| of the FFT stages, times 4 for the packed line transforms."""
+    torch = cuda_or_skip()
+    from paper_1004_1122_gb300 import fh
+
+    phase, L, L0, Y = _problem(N, True)
+    e = np.random.default_rng(1).normal(size=(len(N),) + N).astype(np.float32)
+    ref = (oracle.apply_AT if transpose else oracle.apply_A)(e.astype(np.float64), phase, L, L0, Y)
+    with fh.Solver(phase, L, L0=L0, Y=Y, precision="fp32") as s:
+        x = torch.from_numpy(e).cuda()
+        got = s.apply(x, transpose=transpose).double().cpu().numpy()
+        s.apply(x, out=x, transpose=transpose)
+    tol = 4 * 64 * 2.0 ** -24 * (1.0 + np.max(np.abs(L - L0[None]))) * np.max(np.abs(e))
+    assert np.max(np.abs(got - ref)) <= tol
+    assert np.array_equal(x.double().cpu().numpy(), got)
