@@ -383,6 +383,13 @@ __device__ __forceinline__ void stockham_stage(cplx<T> (&v)[EM], cplx<T>* sm, in
 // threads work on one sequence.
 #define FH_FOR_EACH_RADIX_S(X) X(3) X(5) X(7) X(9)
 
+// The spread set (DynPlanW kernels): every thread of a sequence works on one
+// radix-2 to radix-7 butterfly or one output pair of a radix-11, 13 or 17
+// butterfly per stage.
+#define FH_FOR_EACH_RADIX_W(X) X(2) X(3) X(4) X(5) X(7)
+#define FH_FOR_EACH_SPLIT_W(X) X(11) X(13) X(17)
+constexpr int kMaxWholeW = 7;  // larger (prime) radices are split over threads
+
 // Largest prime radix of the extended set; every extended plan's register
 // array holds at least one butterfly of it.
 constexpr int kMaxPrimeX = 17;
@@ -391,7 +398,7 @@ template <typename T> struct RegBudgetX {
 };
 
 // Radix sets of the run-time plans and their register budgets.
-enum : int { kRadixStd = 0, kRadixExt = 1, kRadixSmall = 2 };
+enum : int { kRadixStd = 0, kRadixExt = 1, kRadixSmall = 2, kRadixSpread = 3 };
 constexpr int kSmallBudget = 9;
 template <typename T, int SET> struct PlanBudget {
   static constexpr int value = SET == kRadixExt ? RegBudgetX<T>::value : SET == kRadixSmall ? kSmallBudget : RegBudget<T>::value;
@@ -404,8 +411,109 @@ struct FFTPlan {
   int n;                    // sequence length
   int nstages;
   int radix[kMaxStages];
-  int ext;                  // 1: uses a radix of the extended set (DynPlanX kernels); 2: small set (DynPlan9)
+  int ext;                  // radix set: kRadixStd (0), kRadixExt (DynPlanX kernels), kRadixSmall (DynPlan9), kRadixSpread (DynPlanW)
 };
+
+// cos and sin of 2 pi m / R.
+template <int R> struct UnitRoots {
+  double c[R], s[R];
+};
+template <int R> __host__ __device__ constexpr UnitRoots<R> unit_roots() {
+  UnitRoots<R> w{};
+  for (int m = 0; m < R; ++m) {
+    const ct::cs v = ct::cossin2pi(m, R);
+    w.c[m] = v.c;
+    w.s[m] = v.s;
+  }
+  return w;
+}
+template <int R> __device__ constexpr UnitRoots<R> kUnitRoots = unit_roots<R>();
+
+// Work items per sequence of a stage of radix R of a spread plan.
+__host__ __device__ constexpr int spread_items(int n, int R) { return n / R * (R > kMaxWholeW ? (R + 1) / 2 : 1); }
+
+// Stockham stage of odd prime radix R with each butterfly spread over
+// (R + 1) / 2 threads: thread k > 0 forms the sum and the difference of inputs
+// k and R - k, then every thread sums one output pair,
+//   y_k, y_{R-k} = (x_0 + sum_i cos(2 pi i k / R) s_i) -+ i sum_i sin(2 pi i k / R) d_i.
+// A whole radix-17 butterfly is a chain of 320 float64 operations in one
+// thread, 64 cycles each on this part; here it is 44.  nthr >= spread_items.
+template <int R, bool INV, typename T>
+__device__ __forceinline__ void stockham_stage_split(cplx<T>* sm, int is, int n, int Ns, int u,
+                                                     const cplx<T>* __restrict__ tw) {
+  using C = cplx<T>;
+  constexpr int K = (R + 1) / 2;
+  const int nb = n / R;
+  const int k = u / nb, j = u - k * nb;
+  const bool act = k < K;
+  const int step = nb * is;
+  C* const src = sm + j * is;
+  const int q = j / Ns, kk = j - q * Ns;
+  if (act && k > 0) {
+    C a = src[k * step], b = src[(R - k) * step];
+    if (Ns > 1) {
+      const C wa = ld_tw(tw + kk + (k - 1) * Ns), wb = ld_tw(tw + kk + (R - k - 1) * Ns);
+      a = INV ? cmulc(a, wa) : cmul(a, wa);
+      b = INV ? cmulc(b, wb) : cmul(b, wb);
+    }
+    src[k * step] = cadd(a, b);
+    src[(R - k) * step] = csub(a, b);
+  }
+  __syncthreads();
+  C A, B;
+  A.x = A.y = B.x = B.y = T(0);
+  if (act) {
+    A = src[0];
+    int m = 0;
+#pragma unroll
+    for (int i = 1; i < K; ++i) {
+      m += k;
+      if (m >= R) m -= R;
+      const T c = T(__ldg(&kUnitRoots<R>.c[m])), s = T(__ldg(&kUnitRoots<R>.s[m]));
+      const C sum = src[i * step], dif = src[(R - i) * step];
+      A.x += c * sum.x;
+      A.y += c * sum.y;
+      B.x += s * dif.x;
+      B.y += s * dif.y;
+    }
+  }
+  __syncthreads();
+  if (act) {
+    C* const dst = sm + (q * R * Ns + kk) * is;
+    const int out = Ns * is;
+    const C lo = cmk<T>(A.x + B.y, A.y - B.x), hi = cmk<T>(A.x - B.y, A.y + B.x);
+    dst[k * out] = INV ? hi : lo;
+    if (k > 0) dst[(R - k) * out] = INV ? lo : hi;
+  }
+  __syncthreads();
+}
+
+// `stages` stages of a spread plan from stage `first` on, upwards or (REV)
+// downwards; Ns and tw belong to the first of them.
+template <bool INV, bool REV, typename T>
+__device__ __forceinline__ void run_fft_spread(cplx<T>* sm, int is, const FFTPlan& pl, int u, int nthr, int first,
+                                               int Ns, const cplx<T>* __restrict__ tw, int stages) {
+  for (int i = 0; i < stages; ++i) {
+    const int R = pl.radix[REV ? first - i : first + i];
+    switch (R) {
+#define FH_STAGE_CASE(RR)                                                    \
+  case RR: {                                                                 \
+    cplx<T> v[RR];                                                           \
+    stockham_stage<RR, INV, T, RR>(v, sm, is, pl.n, Ns, u, nthr, tw);        \
+    break;                                                                   \
+  }
+      FH_FOR_EACH_RADIX_W(FH_STAGE_CASE)
+#undef FH_STAGE_CASE
+#define FH_STAGE_CASE(RR) \
+  case RR: stockham_stage_split<RR, INV, T>(sm, is, pl.n, Ns, u, tw); break;
+      FH_FOR_EACH_SPLIT_W(FH_STAGE_CASE)
+#undef FH_STAGE_CASE
+      default: break;
+    }
+    if (Ns > 1) tw += (R - 1) * Ns;
+    Ns *= R;
+  }
+}
 
 // Run all stages of the plan on one sequence layout.  SET selects the radix
 // set (and its register budget).
@@ -553,6 +661,28 @@ __device__ __forceinline__ void run_fft_fused(cplx<T>* sm, int is, const FFTPlan
 #undef FH_SWITCH
 }
 
+// Transform, pointwise operation and transform back of a spread plan; its last
+// radix is a whole butterfly.
+template <typename T, typename F>
+__device__ __forceinline__ void run_fft_spread_fused(cplx<T>* sm, int is, const FFTPlan& pl, int u, int nthr,
+                                                     const cplx<T>* __restrict__ tw, F& mid) {
+  const int S = pl.nstages, R = pl.radix[S - 1];
+  run_fft_spread<false, false, T>(sm, is, pl, u, nthr, 0, 1, tw, S - 1);
+  const cplx<T>* const twm = S > 1 ? tw + (pl.n / R - pl.radix[0]) : tw;
+  switch (R) {
+#define FH_MID_CASE(RR)                                                          \
+  case RR: {                                                                     \
+    cplx<T> v[RR];                                                               \
+    fused_middle<RR, false, T, RR>(v, sm, is, pl.n, u, nthr, twm, mid);          \
+    break;                                                                       \
+  }
+    FH_FOR_EACH_RADIX_W(FH_MID_CASE)
+#undef FH_MID_CASE
+    default: break;
+  }
+  run_fft_spread<true, true, T>(sm, is, pl, u, nthr, S - 2, R, tw + (pl.n - pl.radix[0]), S - 1);
+}
+
 // ----------------------------------------------------------------------------
 // compile-time plans
 // ----------------------------------------------------------------------------
@@ -565,6 +695,8 @@ struct DynPlan {};
 struct DynPlanX {};
 // Run-time plan over the small radix set (at most 9 values per thread).
 struct DynPlan9 {};
+// Run-time plan over the spread set (one small butterfly per thread and stage).
+struct DynPlanW {};
 
 template <int... Rs> struct CPlan {
   static constexpr int S = sizeof...(Rs);
@@ -643,6 +775,8 @@ __device__ __forceinline__ void fft_plan(cplx<T>* sm, int is, const FFTPlan& pl,
     run_fft<INV, T, kRadixExt>(sm, is, pl, u, nthr, tw);
   else if constexpr (std::is_same<P, DynPlan9>::value)
     run_fft<INV, T, kRadixSmall>(sm, is, pl, u, nthr, tw);
+  else if constexpr (std::is_same<P, DynPlanW>::value)
+    run_fft_spread<INV, false, T>(sm, is, pl, u, nthr, 0, 1, tw, pl.nstages);
   else
     run_fft_ct<INV, T, P>(sm, is, u, nthr, tw);
 }
@@ -654,6 +788,8 @@ __device__ __forceinline__ void fft_fused_plan(cplx<T>* sm, int is, const FFTPla
     run_fft_fused<T, F>(sm, is, pl, u, nthr, tw, mid);
   else if constexpr (std::is_same<P, DynPlanX>::value)
     run_fft_fused<T, F, kRadixExt>(sm, is, pl, u, nthr, tw, mid);
+  else if constexpr (std::is_same<P, DynPlanW>::value)
+    run_fft_spread_fused<T, F>(sm, is, pl, u, nthr, tw, mid);
   else
     run_fft_fused_ct<T, P>(sm, is, u, nthr, tw, mid);
 }

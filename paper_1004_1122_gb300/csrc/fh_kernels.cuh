@@ -75,6 +75,9 @@ template <> struct PlanLen<DynPlan> {
 template <> struct PlanLen<DynPlanX> {
   static constexpr int value = 0;
 };
+template <> struct PlanLen<DynPlanW> {
+  static constexpr int value = 0;
+};
 template <> struct PlanLen<DynPlan9> {
   static constexpr int value = 0;
 };
@@ -95,6 +98,10 @@ template <typename PS> struct ColBounds {
 };
 template <> struct ColBounds<DynPlan> {
   static constexpr int threads = kColMaxThreads, blocks = 1;
+};
+constexpr int kColSpreadMaxThreads = 512;  // column passes with a spread plan: <= 128 registers per thread
+template <> struct ColBounds<DynPlanW> {
+  static constexpr int threads = kColSpreadMaxThreads, blocks = 1;
 };
 constexpr int kColPipeMaxThreads = 512;  // persistent Green pass: <= 128 registers per thread
 

@@ -47,6 +47,11 @@ using CtPlan = typename std::conditional<D == 2, typename std::conditional<NL ==
 template <typename T, int D>
 constexpr bool kHasDf = std::is_same<T, double>::value && D == 2;
 
+// Spread plans: float64, one load per launch (grids too small to give every
+// SM scheduler a warp; see spread_plans in the pipeline).
+template <typename T, int NL>
+constexpr bool kHasSpread = std::is_same<T, double>::value && NL == 1;
+
 // The 2187^2 Green pass also exists with its tuned tile shape compiled in:
 // tiles of 2 frequencies x 2 components (Q = 4 columns), 81 threads per
 // 2187-point column FFT.
@@ -143,6 +148,22 @@ struct Launchers {
       FH_SM((k_col<T, D, kColFwd, DynPlanX>), c1)
       FH_SM((k_col<T, D, kColInv, DynPlanX>), c1)
     }
+    if constexpr (kHasSpread<T, NL>) {
+      FH_SM((k_row_fwd<T, D, NL, kProApply, DynPlanW>), rs)
+      FH_SM((k_row_fwd<T, D, NL, kProPlain, DynPlanW>), rs)
+      FH_SM((k_row_fwd<T, D, NL, kProDir, DynPlanW>), rs)
+      FH_SM((k_row_fwd<T, D, NL, kProDirPlain, DynPlanW>), rs)
+      FH_SM((k_row_inv<T, D, NL, kEpiApply, DynPlanW>), rs)
+      FH_SM((k_row_inv<T, D, NL, kEpiApplyT, DynPlanW>), rs)
+      FH_SM((k_row_inv<T, D, NL, kEpiDir, DynPlanW>), rs)
+      FH_SM((k_row_inv<T, D, NL, kEpiDirShadow, DynPlanW>), rs)
+      FH_SM((k_row_inv<T, D, NL, kEpiFixed, DynPlanW>), rs)
+      FH_SM((k_row_inv<T, D, NL, kEpiResid, DynPlanW>), rs)
+      FH_SM((k_col<T, D, kColGreen, DynPlanW>), c0)
+      FH_SM((k_col<T, D, kColEta, DynPlanW>), c0)
+      FH_SM((k_col<T, D, kColFwd, DynPlanW>), c1)
+      FH_SM((k_col<T, D, kColInv, DynPlanW>), c1)
+    }
     if constexpr (kHasDf<T, D>) {
       FH_SM((k_col_green_df<>), c0)
       FH_SM((k_row_fwd<T, D, NL, kProApply, DynPlan, true>), rs)
@@ -171,6 +192,19 @@ struct Launchers {
         k_row_fwd<T, D, NL, kProDir, P><<<L.grid, L.block, L.smem, st>>>(a);
         return cudaGetLastError();
       }
+    }
+    if (a.plan.ext == kRadixSpread) {
+      if constexpr (kHasSpread<T, NL>) {
+        switch (pro) {
+          case kProApply: k_row_fwd<T, D, NL, kProApply, DynPlanW><<<L.grid, L.block, L.smem, st>>>(a); break;
+          case kProPlain: k_row_fwd<T, D, NL, kProPlain, DynPlanW><<<L.grid, L.block, L.smem, st>>>(a); break;
+          case kProDir: k_row_fwd<T, D, NL, kProDir, DynPlanW><<<L.grid, L.block, L.smem, st>>>(a); break;
+          case kProDirPlain: k_row_fwd<T, D, NL, kProDirPlain, DynPlanW><<<L.grid, L.block, L.smem, st>>>(a); break;
+          default: return cudaErrorInvalidValue;
+        }
+        return cudaGetLastError();
+      }
+      return cudaErrorInvalidValue;
     }
     if (a.plan.ext) {  // a length with a prime factor 11, 13 or 17
       if constexpr (NL == 1) {
@@ -220,6 +254,23 @@ struct Launchers {
         k_row_inv<T, D, NL, kEpiDir, P><<<L.grid, L.block, L.smem, st>>>(a);
         return cudaGetLastError();
       }
+    }
+    if (a.plan.ext == kRadixSpread) {
+      if constexpr (kHasSpread<T, NL>) {
+        switch (epi) {
+          case kEpiApply: k_row_inv<T, D, NL, kEpiApply, DynPlanW><<<L.grid, L.block, L.smem, st>>>(a); break;
+          case kEpiApplyT: k_row_inv<T, D, NL, kEpiApplyT, DynPlanW><<<L.grid, L.block, L.smem, st>>>(a); break;
+          case kEpiDir: k_row_inv<T, D, NL, kEpiDir, DynPlanW><<<L.grid, L.block, L.smem, st>>>(a); break;
+          case kEpiDirShadow:
+            k_row_inv<T, D, NL, kEpiDirShadow, DynPlanW><<<L.grid, L.block, L.smem, st>>>(a);
+            break;
+          case kEpiFixed: k_row_inv<T, D, NL, kEpiFixed, DynPlanW><<<L.grid, L.block, L.smem, st>>>(a); break;
+          case kEpiResid: k_row_inv<T, D, NL, kEpiResid, DynPlanW><<<L.grid, L.block, L.smem, st>>>(a); break;
+          default: return cudaErrorInvalidValue;
+        }
+        return cudaGetLastError();
+      }
+      return cudaErrorInvalidValue;
     }
     if (a.plan.ext) {  // a length with a prime factor 11, 13 or 17
       if constexpr (NL == 1) {
@@ -297,6 +348,19 @@ struct Launchers {
           }
         }
       }
+    }
+    if (a.b.plan.ext == kRadixSpread) {
+      if constexpr (kHasSpread<T, NL>) {
+        switch (mode) {
+          case kColFwd: k_col<T, D, kColFwd, DynPlanW><<<L.grid, L.block, L.smem, st>>>(a); break;
+          case kColInv: k_col<T, D, kColInv, DynPlanW><<<L.grid, L.block, L.smem, st>>>(a); break;
+          case kColGreen: k_col<T, D, kColGreen, DynPlanW><<<L.grid, L.block, L.smem, st>>>(a); break;
+          case kColEta: k_col<T, D, kColEta, DynPlanW><<<L.grid, L.block, L.smem, st>>>(a); break;
+          default: return cudaErrorInvalidValue;
+        }
+        return cudaGetLastError();
+      }
+      return cudaErrorInvalidValue;
     }
     if (a.b.plan.ext) {  // a length with a prime factor 11, 13 or 17
       if constexpr (NL == 1) {

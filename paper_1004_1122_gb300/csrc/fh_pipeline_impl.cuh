@@ -102,6 +102,25 @@ int Pipeline<T>::init(const Problem& pb, int nloads_, bool krylov, cudaStream_t 
     err = "no FFT plan for this grid (axis lengths must factor into 2, 3, 5, 7, 11, 13 and 17)";
     return 9;  // FH_ERR_UNSUPPORTED
   }
+  // Spread plans (one small butterfly per thread and stage) for float64
+  // pipelines whose passes would leave SM schedulers without a warp.  A float64
+  // warp instruction occupies its scheduler's unit for 64 cycles on this part,
+  // so a pass then takes one thread's chain of float64 operations: the more
+  // threads share a sequence, the shorter.
+  auto spread = [&](int n, long long seqs, int tile_seqs, int max_thr, int forced, FFTPlan& pl, int& t) {
+    FFTPlan ps;
+    int ts = 0;
+    if (!f64 || !krylov || nloads != 1 || (want && want->pipe) || seqs * t >= 128LL * sms) return;
+    if (!make_spread_plan(n, ps, ts) || ts * tile_seqs > max_thr || (forced && forced != ts)) return;
+    pl = ps;
+    t = ts;
+  };
+  spread(g.nlast, ((long long)g.nlines * g.M + 1) / 2, (g.M + 1) / 2, kRowMaxThreads, w.tpl, prow, tpl);
+  spread(pb.N[0], (long long)g.H * g.n1 * ncell * g.M, g.M * std::max(1, w.C), kColSpreadMaxThreads, w.tpc0, pcol0, tpc0);
+  if (d == 3) spread(pb.N[1], (long long)g.H * pb.N[0] * g.M, g.M * std::max(1, w.C), kColSpreadMaxThreads,
+                     w.tpc1, pcol1, tpc1);
+  const int colmax0 = pcol0.ext == kRadixSpread ? kColSpreadMaxThreads : kColMaxThreads;
+  const int colmax1 = pcol1.ext == kRadixSpread ? kColSpreadMaxThreads : kColMaxThreads;
   const bool ext = prow.ext || pcol0.ext || (d == 3 && pcol1.ext);
   if (ext && nloads != 1) {
     err = "even axis lengths and lengths with a prime factor 11, 13 or 17 run one load per launch only";
@@ -121,12 +140,12 @@ int Pipeline<T>::init(const Problem& pb, int nloads_, bool krylov, cudaStream_t 
     if (cand > 1 && pad > 0.15 && !w.C) continue;
     if (d == 2) {
       if ((size_t)pb.N[0] * cand * M * esz > smem_green) continue;
-      if (round_up(cand * M * tpc0, 32) > kColMaxThreads) continue;
+      if (round_up(cand * M * tpc0, 32) > colmax0) continue;
     } else {
       if ((size_t)pb.N[1] * cand * M * esz > smem_green) continue;
-      if (round_up(cand * M * tpc1, 32) > kColMaxThreads) continue;
+      if (round_up(cand * M * tpc1, 32) > colmax1) continue;
       if ((size_t)pb.N[0] * cand * M * esz > smem_green) continue;
-      if (round_up(cand * M * tpc0, 32) > kColMaxThreads) continue;
+      if (round_up(cand * M * tpc0, 32) > colmax0) continue;
     }
     Cc = cand;
     const long long ctas = (long long)Tt * (d == 2 ? ncell : std::min(pb.N[0], pb.N[1]));
@@ -172,7 +191,7 @@ int Pipeline<T>::init(const Problem& pb, int nloads_, bool krylov, cudaStream_t 
       for (int cand = g.n1; cand >= 1; --cand) {
         if (g.n1 % cand) continue;
         if ((size_t)pb.N[0] * cand * CM * esz > std::min<size_t>(100 * 1024, smem_green)) continue;
-        if (round_up((int)(cand * CM) * tpc0, 32) > kColMaxThreads) continue;
+        if (round_up((int)(cand * CM) * tpc0, 32) > colmax0) continue;
         if (cand > 1 && (long long)g.Tt * (g.n1 / cand) < 2LL * sms) continue;
         G = cand;
         break;

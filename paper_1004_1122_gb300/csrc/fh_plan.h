@@ -126,6 +126,30 @@ inline bool make_fft_plan(int n, bool fp64, int max_tpl, FFTPlan& pl, int& tpl,
   return true;
 }
 
+// Spread plan (kRadixSpread) of length n: every stage gives each thread at most
+// one butterfly of radix 2 to 7 or one output pair of a radix-11, 13 or 17
+// butterfly; the split radices come first.  False where the last stage would
+// be a split one.
+inline bool make_spread_plan(int n, FFTPlan& pl, int& tpl) {
+  std::vector<int> r;
+  int m = n;
+  for (int R : {17, 13, 11, 7, 5, 4, 3, 2})
+    while (m % R == 0) {
+      r.push_back(R);
+      m /= R;
+    }
+  if (m != 1 || r.empty() || (int)r.size() > kMaxStages || r.back() > kMaxWholeW) return false;
+  pl.n = n;
+  pl.nstages = (int)r.size();
+  tpl = 1;
+  for (int s = 0; s < kMaxStages; ++s) {
+    pl.radix[s] = s < pl.nstages ? r[s] : 0;
+    if (s < pl.nstages) tpl = std::max(tpl, spread_items(n, r[s]));
+  }
+  pl.ext = kRadixSpread;
+  return true;
+}
+
 // exp(-2 pi i m / n) for m in [0, n), float64.  The angle is reduced exactly
 // on the rational m / n (octant symmetry) before calling the C library, so
 // every entry is within an ulp or two of the true value.
