@@ -297,6 +297,12 @@ __device__ __forceinline__ void block_reduce_store(double (&v)[NV], int nv, doub
   }
 }
 
+// First statement of the kernels of a chain (seq_launch): wait for the kernel
+// before this one and its writes, then let the next one's CTAs in.
+__device__ __forceinline__ void seq_begin() {
+  cudaGridDependencySynchronize();
+}
+
 __device__ __forceinline__ void prefetch_l2(const void* p) {
   asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
@@ -340,6 +346,7 @@ enum : int {
 // RS: compile-time launch shape (RowShape) or RowDyn.
 template <typename T, int D, int NL, int PRO, typename PS = DynPlan, bool DF = false, typename RS = RowDyn>
 __global__ void __launch_bounds__(RowBounds<PS>::threads, RowBounds<PS>::blocks) k_row_fwd(RowArgs<T> a) {
+  seq_begin();
   using C = cplx<T>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* sm = reinterpret_cast<C*>(smem_raw);
@@ -653,6 +660,7 @@ __device__ __forceinline__ void green_tile(const ColArgs<T>& a, cplx<T>* sm, int
 // offsets instead of run-time index arithmetic.
 template <typename T, int D, int CM_, typename PS = DynPlan, int QC = 0, int TC = 0>
 __global__ void __launch_bounds__(ColBounds<PS>::threads, ColBounds<PS>::blocks) k_col(ColArgs<T> a) {
+  seq_begin();
   using C = cplx<T>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* sm = reinterpret_cast<C*>(smem_raw);
@@ -814,6 +822,7 @@ struct GreenPointDF {
 // whole double2 values (16-byte aligned), so the tile moves as 16-byte words.
 template <typename PS = DynPlan>
 __global__ void __launch_bounds__(kColMaxThreads) k_col_green_df(ColArgs<double> a, const dfc* __restrict__ twdf) {
+  seq_begin();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   dfc* sm = reinterpret_cast<dfc*>(smem_raw);
   const ColArgsBase& b = a.b;
@@ -951,6 +960,7 @@ enum : int {
 // RS: compile-time launch shape (RowShape) or RowDyn.
 template <typename T, int D, int NL, int EPI, typename PS = DynPlan, bool DF = false, typename RS = RowDyn>
 __global__ void __launch_bounds__(RowBounds<PS>::threads, RowBounds<PS>::blocks) k_row_inv(RowArgs<T> a) {
+  seq_begin();
   using C = cplx<T>;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   C* sm = reinterpret_cast<C*>(smem_raw);
@@ -1337,6 +1347,7 @@ __device__ __forceinline__ void cell_ranges(const VecArgs<T>& a, Mk&& mk) {
 // history)
 template <typename T, int NL, bool PP = false, int XM = 1>
 __global__ void k_cg_update(VecArgs<T> a) {
+  seq_begin();
   const int bpc = gridDim.x / a.b.ncell;
   const int cell = blockIdx.x / bpc;
   Scal* const sc = a.scal + cell * NL;
@@ -1363,6 +1374,7 @@ __global__ void k_cg_update(VecArgs<T> a) {
 // receive it, x += alpha_x p.
 template <typename T, int NL>
 __global__ void k_cg_flush(VecArgs<T> a) {
+  seq_begin();
   const int bpc = gridDim.x / a.b.ncell;
   const int cell = blockIdx.x / bpc;
   const Scal* const sc = a.scal + cell * NL;
@@ -1381,6 +1393,7 @@ __global__ void k_cg_flush(VecArgs<T> a) {
 // (p, p) at slot 2 kMaxLoads + l.
 template <typename T, int NL>
 __global__ void k_bicg_update(VecArgs<T> a) {
+  seq_begin();
   const int bpc = gridDim.x / a.b.ncell;
   const int cell = blockIdx.x / bpc;
   Scal* const sc = a.scal + cell * NL;
@@ -1465,6 +1478,7 @@ __device__ __forceinline__ void record_hist(Scal& s) {
 // After the initial residual (kEpiResid partials or a copied rhs):
 // rr = sum, rel = sqrt(rr / b2), beta = 0, iter = 0.
 static __global__ void k_scal_start(Scal* scal, const double* part, int np, int ncell, int nl) {
+  seq_begin();
   const ItemRef r = item_ref(np, ncell, nl);
   if (!r.valid) return;
   const double rr = block_sum(item_part(part, r.l, np, r), r.bpc);
@@ -1489,6 +1503,7 @@ static __global__ void k_scal_start(Scal* scal, const double* part, int np, int 
 
 // alpha = (r, r) / (A p, p) for CG; alpha = (r, r*) / (A p, p*) for BiCG
 static __global__ void k_scal_alpha(Scal* scal, const double* part, int np, int ncell, int nl, int bicg) {
+  seq_begin();
   const ItemRef r = item_ref(np, ncell, nl);
   if (!r.valid) return;
   const double den = block_sum(item_part(part, r.l, np, r), r.bpc);
@@ -1508,6 +1523,7 @@ static __global__ void k_scal_alpha(Scal* scal, const double* part, int np, int 
 // step owed, 1 after one that settled it, -1 when x moves every iteration.
 static __global__ void k_scal_beta(Scal* scal, const double* part, int np, int ncell, int nl, int bicg,
                                    int xpar) {
+  seq_begin();
   const ItemRef r = item_ref(np, ncell, nl);
   if (!r.valid) return;
   double rho_new = 0.0, rr_new, pp = 0.0;
@@ -1553,6 +1569,7 @@ static __global__ void k_scal_beta(Scal* scal, const double* part, int np, int n
 
 // Fixed point: the epilogue produced ||e_new - e||^2 = ||r(e)||^2.
 static __global__ void k_scal_fixed(Scal* scal, const double* part, int np, int ncell, int nl) {
+  seq_begin();
   const ItemRef r = item_ref(np, ncell, nl);
   if (!r.valid) return;
   const double rr = block_sum(item_part(part, r.l, np, r), r.bpc);
@@ -1587,6 +1604,7 @@ static __global__ void k_eta_record(const double* part, int np, const Scal* scal
 
 // out[cell * nv + v] = sum of row v of the partials over the cell's slots.
 static __global__ void k_reduce_items(const double* part, int np, int ncell, int nv, double* out) {
+  seq_begin();
   const ItemRef r = item_ref(np, ncell, nv);
   if (!r.valid) return;
   const double x = block_sum(item_part(part, r.l, np, r), r.bpc);

@@ -176,7 +176,7 @@ struct Launchers {
     if constexpr (kHasDf<T, D>) {
       if (a.twdf != nullptr) {  // float64 residual: double-float line FFTs
         if (pro != kProApply) return cudaErrorInvalidValue;
-        k_row_fwd<T, D, NL, kProApply, DynPlan, true><<<L.grid, L.block, L.smem, st>>>(a);
+        seq_launch(k_row_fwd<T, D, NL, kProApply, DynPlan, true>, L, L.smem, st, a);
         return cudaGetLastError();
       }
     }
@@ -185,21 +185,21 @@ struct Launchers {
       if (pro == kProDir && L.block <= RowBounds<P>::threads && cplan_is<P>(a.plan)) {
         if constexpr (D == 3 && NL == 3) {
           if (row_shape_is<RowShape243x3, D * NL>(L, a)) {
-            k_row_fwd<T, D, NL, kProDir, P, false, RowShape243x3><<<L.grid, L.block, L.smem, st>>>(a);
+            seq_launch(k_row_fwd<T, D, NL, kProDir, P, false, RowShape243x3>, L, L.smem, st, a);
             return cudaGetLastError();
           }
         }
-        k_row_fwd<T, D, NL, kProDir, P><<<L.grid, L.block, L.smem, st>>>(a);
+        seq_launch(k_row_fwd<T, D, NL, kProDir, P>, L, L.smem, st, a);
         return cudaGetLastError();
       }
     }
     if (a.plan.ext == kRadixSpread) {
       if constexpr (kHasSpread<T, NL>) {
         switch (pro) {
-          case kProApply: k_row_fwd<T, D, NL, kProApply, DynPlanW><<<L.grid, L.block, L.smem, st>>>(a); break;
-          case kProPlain: k_row_fwd<T, D, NL, kProPlain, DynPlanW><<<L.grid, L.block, L.smem, st>>>(a); break;
-          case kProDir: k_row_fwd<T, D, NL, kProDir, DynPlanW><<<L.grid, L.block, L.smem, st>>>(a); break;
-          case kProDirPlain: k_row_fwd<T, D, NL, kProDirPlain, DynPlanW><<<L.grid, L.block, L.smem, st>>>(a); break;
+          case kProApply: seq_launch(k_row_fwd<T, D, NL, kProApply, DynPlanW>, L, L.smem, st, a); break;
+          case kProPlain: seq_launch(k_row_fwd<T, D, NL, kProPlain, DynPlanW>, L, L.smem, st, a); break;
+          case kProDir: seq_launch(k_row_fwd<T, D, NL, kProDir, DynPlanW>, L, L.smem, st, a); break;
+          case kProDirPlain: seq_launch(k_row_fwd<T, D, NL, kProDirPlain, DynPlanW>, L, L.smem, st, a); break;
           default: return cudaErrorInvalidValue;
         }
         return cudaGetLastError();
@@ -209,10 +209,10 @@ struct Launchers {
     if (a.plan.ext) {  // a length with a prime factor 11, 13 or 17
       if constexpr (NL == 1) {
         switch (pro) {
-          case kProApply: k_row_fwd<T, D, NL, kProApply, DynPlanX><<<L.grid, L.block, L.smem, st>>>(a); break;
-          case kProPlain: k_row_fwd<T, D, NL, kProPlain, DynPlanX><<<L.grid, L.block, L.smem, st>>>(a); break;
-          case kProDir: k_row_fwd<T, D, NL, kProDir, DynPlanX><<<L.grid, L.block, L.smem, st>>>(a); break;
-          case kProDirPlain: k_row_fwd<T, D, NL, kProDirPlain, DynPlanX><<<L.grid, L.block, L.smem, st>>>(a); break;
+          case kProApply: seq_launch(k_row_fwd<T, D, NL, kProApply, DynPlanX>, L, L.smem, st, a); break;
+          case kProPlain: seq_launch(k_row_fwd<T, D, NL, kProPlain, DynPlanX>, L, L.smem, st, a); break;
+          case kProDir: seq_launch(k_row_fwd<T, D, NL, kProDir, DynPlanX>, L, L.smem, st, a); break;
+          case kProDirPlain: seq_launch(k_row_fwd<T, D, NL, kProDirPlain, DynPlanX>, L, L.smem, st, a); break;
           default: return cudaErrorInvalidValue;
         }
         return cudaGetLastError();
@@ -220,10 +220,10 @@ struct Launchers {
       return cudaErrorInvalidValue;
     }
     switch (pro) {
-      case kProApply: k_row_fwd<T, D, NL, kProApply><<<L.grid, L.block, L.smem, st>>>(a); break;
-      case kProPlain: k_row_fwd<T, D, NL, kProPlain><<<L.grid, L.block, L.smem, st>>>(a); break;
-      case kProDir: k_row_fwd<T, D, NL, kProDir><<<L.grid, L.block, L.smem, st>>>(a); break;
-      case kProDirPlain: k_row_fwd<T, D, NL, kProDirPlain><<<L.grid, L.block, L.smem, st>>>(a); break;
+      case kProApply: seq_launch(k_row_fwd<T, D, NL, kProApply>, L, L.smem, st, a); break;
+      case kProPlain: seq_launch(k_row_fwd<T, D, NL, kProPlain>, L, L.smem, st, a); break;
+      case kProDir: seq_launch(k_row_fwd<T, D, NL, kProDir>, L, L.smem, st, a); break;
+      case kProDirPlain: seq_launch(k_row_fwd<T, D, NL, kProDirPlain>, L, L.smem, st, a); break;
       default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
@@ -232,7 +232,7 @@ struct Launchers {
     if constexpr (kHasDf<T, D>) {
       if (a.twdf != nullptr) {  // float64 residual: double-float line FFTs
         if (epi != kEpiResid) return cudaErrorInvalidValue;
-        k_row_inv<T, D, NL, kEpiResid, DynPlan, true><<<L.grid, L.block, L.smem, st>>>(a);
+        seq_launch(k_row_inv<T, D, NL, kEpiResid, DynPlan, true>, L, L.smem, st, a);
         return cudaGetLastError();
       }
     }
@@ -241,31 +241,31 @@ struct Launchers {
       if (epi == kEpiDir && L.block <= RowBounds<P>::threads && cplan_is<P>(a.plan)) {
         if constexpr (D == 3 && NL == 3) {
           if (row_shape_is<RowShape243x3, D * NL>(L, a)) {
-            k_row_inv<T, D, NL, kEpiDir, P, false, RowShape243x3><<<L.grid, L.block, L.smem, st>>>(a);
+            seq_launch(k_row_inv<T, D, NL, kEpiDir, P, false, RowShape243x3>, L, L.smem, st, a);
             return cudaGetLastError();
           }
         }
         if constexpr (D == 2 && NL == 1) {
           if (row_shape_is_2187(L, a)) {
-            k_row_inv<T, D, NL, kEpiDir, P, false, RowShape2187><<<L.grid, L.block, L.smem, st>>>(a);
+            seq_launch(k_row_inv<T, D, NL, kEpiDir, P, false, RowShape2187>, L, L.smem, st, a);
             return cudaGetLastError();
           }
         }
-        k_row_inv<T, D, NL, kEpiDir, P><<<L.grid, L.block, L.smem, st>>>(a);
+        seq_launch(k_row_inv<T, D, NL, kEpiDir, P>, L, L.smem, st, a);
         return cudaGetLastError();
       }
     }
     if (a.plan.ext == kRadixSpread) {
       if constexpr (kHasSpread<T, NL>) {
         switch (epi) {
-          case kEpiApply: k_row_inv<T, D, NL, kEpiApply, DynPlanW><<<L.grid, L.block, L.smem, st>>>(a); break;
-          case kEpiApplyT: k_row_inv<T, D, NL, kEpiApplyT, DynPlanW><<<L.grid, L.block, L.smem, st>>>(a); break;
-          case kEpiDir: k_row_inv<T, D, NL, kEpiDir, DynPlanW><<<L.grid, L.block, L.smem, st>>>(a); break;
+          case kEpiApply: seq_launch(k_row_inv<T, D, NL, kEpiApply, DynPlanW>, L, L.smem, st, a); break;
+          case kEpiApplyT: seq_launch(k_row_inv<T, D, NL, kEpiApplyT, DynPlanW>, L, L.smem, st, a); break;
+          case kEpiDir: seq_launch(k_row_inv<T, D, NL, kEpiDir, DynPlanW>, L, L.smem, st, a); break;
           case kEpiDirShadow:
-            k_row_inv<T, D, NL, kEpiDirShadow, DynPlanW><<<L.grid, L.block, L.smem, st>>>(a);
+            seq_launch(k_row_inv<T, D, NL, kEpiDirShadow, DynPlanW>, L, L.smem, st, a);
             break;
-          case kEpiFixed: k_row_inv<T, D, NL, kEpiFixed, DynPlanW><<<L.grid, L.block, L.smem, st>>>(a); break;
-          case kEpiResid: k_row_inv<T, D, NL, kEpiResid, DynPlanW><<<L.grid, L.block, L.smem, st>>>(a); break;
+          case kEpiFixed: seq_launch(k_row_inv<T, D, NL, kEpiFixed, DynPlanW>, L, L.smem, st, a); break;
+          case kEpiResid: seq_launch(k_row_inv<T, D, NL, kEpiResid, DynPlanW>, L, L.smem, st, a); break;
           default: return cudaErrorInvalidValue;
         }
         return cudaGetLastError();
@@ -275,14 +275,14 @@ struct Launchers {
     if (a.plan.ext) {  // a length with a prime factor 11, 13 or 17
       if constexpr (NL == 1) {
         switch (epi) {
-          case kEpiApply: k_row_inv<T, D, NL, kEpiApply, DynPlanX><<<L.grid, L.block, L.smem, st>>>(a); break;
-          case kEpiApplyT: k_row_inv<T, D, NL, kEpiApplyT, DynPlanX><<<L.grid, L.block, L.smem, st>>>(a); break;
-          case kEpiDir: k_row_inv<T, D, NL, kEpiDir, DynPlanX><<<L.grid, L.block, L.smem, st>>>(a); break;
+          case kEpiApply: seq_launch(k_row_inv<T, D, NL, kEpiApply, DynPlanX>, L, L.smem, st, a); break;
+          case kEpiApplyT: seq_launch(k_row_inv<T, D, NL, kEpiApplyT, DynPlanX>, L, L.smem, st, a); break;
+          case kEpiDir: seq_launch(k_row_inv<T, D, NL, kEpiDir, DynPlanX>, L, L.smem, st, a); break;
           case kEpiDirShadow:
-            k_row_inv<T, D, NL, kEpiDirShadow, DynPlanX><<<L.grid, L.block, L.smem, st>>>(a);
+            seq_launch(k_row_inv<T, D, NL, kEpiDirShadow, DynPlanX>, L, L.smem, st, a);
             break;
-          case kEpiFixed: k_row_inv<T, D, NL, kEpiFixed, DynPlanX><<<L.grid, L.block, L.smem, st>>>(a); break;
-          case kEpiResid: k_row_inv<T, D, NL, kEpiResid, DynPlanX><<<L.grid, L.block, L.smem, st>>>(a); break;
+          case kEpiFixed: seq_launch(k_row_inv<T, D, NL, kEpiFixed, DynPlanX>, L, L.smem, st, a); break;
+          case kEpiResid: seq_launch(k_row_inv<T, D, NL, kEpiResid, DynPlanX>, L, L.smem, st, a); break;
           default: return cudaErrorInvalidValue;
         }
         return cudaGetLastError();
@@ -290,12 +290,12 @@ struct Launchers {
       return cudaErrorInvalidValue;
     }
     switch (epi) {
-      case kEpiApply: k_row_inv<T, D, NL, kEpiApply><<<L.grid, L.block, L.smem, st>>>(a); break;
-      case kEpiApplyT: k_row_inv<T, D, NL, kEpiApplyT><<<L.grid, L.block, L.smem, st>>>(a); break;
-      case kEpiDir: k_row_inv<T, D, NL, kEpiDir><<<L.grid, L.block, L.smem, st>>>(a); break;
-      case kEpiDirShadow: k_row_inv<T, D, NL, kEpiDirShadow><<<L.grid, L.block, L.smem, st>>>(a); break;
-      case kEpiFixed: k_row_inv<T, D, NL, kEpiFixed><<<L.grid, L.block, L.smem, st>>>(a); break;
-      case kEpiResid: k_row_inv<T, D, NL, kEpiResid><<<L.grid, L.block, L.smem, st>>>(a); break;
+      case kEpiApply: seq_launch(k_row_inv<T, D, NL, kEpiApply>, L, L.smem, st, a); break;
+      case kEpiApplyT: seq_launch(k_row_inv<T, D, NL, kEpiApplyT>, L, L.smem, st, a); break;
+      case kEpiDir: seq_launch(k_row_inv<T, D, NL, kEpiDir>, L, L.smem, st, a); break;
+      case kEpiDirShadow: seq_launch(k_row_inv<T, D, NL, kEpiDirShadow>, L, L.smem, st, a); break;
+      case kEpiFixed: seq_launch(k_row_inv<T, D, NL, kEpiFixed>, L, L.smem, st, a); break;
+      case kEpiResid: seq_launch(k_row_inv<T, D, NL, kEpiResid>, L, L.smem, st, a); break;
       default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
@@ -307,9 +307,9 @@ struct Launchers {
         if constexpr (D == 3 && NL == 3) {
           if (a.b.Q == kCol3Q && a.b.tpc == kCol3T) {  // the tuned 243^3 three-load tile shape
             switch (mode) {
-              case kColFwd: k_col<T, D, kColFwd, P, kCol3Q, kCol3T><<<L.grid, L.block, L.smem, st>>>(a); break;
-              case kColInv: k_col<T, D, kColInv, P, kCol3Q, kCol3T><<<L.grid, L.block, L.smem, st>>>(a); break;
-              case kColGreen: k_col<T, D, kColGreen, P, kCol3Q, kCol3T><<<L.grid, L.block, L.smem, st>>>(a); break;
+              case kColFwd: seq_launch(k_col<T, D, kColFwd, P, kCol3Q, kCol3T>, L, L.smem, st, a); break;
+              case kColInv: seq_launch(k_col<T, D, kColInv, P, kCol3Q, kCol3T>, L, L.smem, st, a); break;
+              case kColGreen: seq_launch(k_col<T, D, kColGreen, P, kCol3Q, kCol3T>, L, L.smem, st, a); break;
               default: return cudaErrorInvalidValue;
             }
             return cudaGetLastError();
@@ -319,31 +319,31 @@ struct Launchers {
           if constexpr (D == 2 && NL == 2) {
             if (a.b.tpc == kGreen729T && a.b.stride_i == a.b.Q) {  // the 729^2 two-load tiles
               if (a.b.Q == 4) {
-                k_col<T, D, kColGreen, P, 4, kGreen729T><<<L.grid, L.block, L.smem, st>>>(a);
+                seq_launch(k_col<T, D, kColGreen, P, 4, kGreen729T>, L, L.smem, st, a);
                 return cudaGetLastError();
               }
               if (a.b.Q == 8) {
-                k_col<T, D, kColGreen, P, 8, kGreen729T><<<L.grid, L.block, L.smem, st>>>(a);
+                seq_launch(k_col<T, D, kColGreen, P, 8, kGreen729T>, L, L.smem, st, a);
                 return cudaGetLastError();
               }
             }
           }
           if constexpr (D == 2 && NL == 1) {
             if (a.b.Q == kGreenQ && a.b.tpc == kGreenT && a.b.stride_i == kGreenQ) {  // the tuned 2187^2 tile shape
-              k_col<T, D, kColGreen, P, kGreenQ, kGreenT><<<L.grid, L.block, L.smem, st>>>(a);
+              seq_launch(k_col<T, D, kColGreen, P, kGreenQ, kGreenT>, L, L.smem, st, a);
               return cudaGetLastError();
             }
           }
-          k_col<T, D, kColGreen, P><<<L.grid, L.block, L.smem, st>>>(a);
+          seq_launch(k_col<T, D, kColGreen, P>, L, L.smem, st, a);
           return cudaGetLastError();
         }
         if constexpr (D == 3) {
           if (mode == kColFwd) {
-            k_col<T, D, kColFwd, P><<<L.grid, L.block, L.smem, st>>>(a);
+            seq_launch(k_col<T, D, kColFwd, P>, L, L.smem, st, a);
             return cudaGetLastError();
           }
           if (mode == kColInv) {
-            k_col<T, D, kColInv, P><<<L.grid, L.block, L.smem, st>>>(a);
+            seq_launch(k_col<T, D, kColInv, P>, L, L.smem, st, a);
             return cudaGetLastError();
           }
         }
@@ -352,10 +352,10 @@ struct Launchers {
     if (a.b.plan.ext == kRadixSpread) {
       if constexpr (kHasSpread<T, NL>) {
         switch (mode) {
-          case kColFwd: k_col<T, D, kColFwd, DynPlanW><<<L.grid, L.block, L.smem, st>>>(a); break;
-          case kColInv: k_col<T, D, kColInv, DynPlanW><<<L.grid, L.block, L.smem, st>>>(a); break;
-          case kColGreen: k_col<T, D, kColGreen, DynPlanW><<<L.grid, L.block, L.smem, st>>>(a); break;
-          case kColEta: k_col<T, D, kColEta, DynPlanW><<<L.grid, L.block, L.smem, st>>>(a); break;
+          case kColFwd: seq_launch(k_col<T, D, kColFwd, DynPlanW>, L, L.smem, st, a); break;
+          case kColInv: seq_launch(k_col<T, D, kColInv, DynPlanW>, L, L.smem, st, a); break;
+          case kColGreen: seq_launch(k_col<T, D, kColGreen, DynPlanW>, L, L.smem, st, a); break;
+          case kColEta: seq_launch(k_col<T, D, kColEta, DynPlanW>, L, L.smem, st, a); break;
           default: return cudaErrorInvalidValue;
         }
         return cudaGetLastError();
@@ -365,10 +365,10 @@ struct Launchers {
     if (a.b.plan.ext) {  // a length with a prime factor 11, 13 or 17
       if constexpr (NL == 1) {
         switch (mode) {
-          case kColFwd: k_col<T, D, kColFwd, DynPlanX><<<L.grid, L.block, L.smem, st>>>(a); break;
-          case kColInv: k_col<T, D, kColInv, DynPlanX><<<L.grid, L.block, L.smem, st>>>(a); break;
-          case kColGreen: k_col<T, D, kColGreen, DynPlanX><<<L.grid, L.block, L.smem, st>>>(a); break;
-          case kColEta: k_col<T, D, kColEta, DynPlanX><<<L.grid, L.block, L.smem, st>>>(a); break;
+          case kColFwd: seq_launch(k_col<T, D, kColFwd, DynPlanX>, L, L.smem, st, a); break;
+          case kColInv: seq_launch(k_col<T, D, kColInv, DynPlanX>, L, L.smem, st, a); break;
+          case kColGreen: seq_launch(k_col<T, D, kColGreen, DynPlanX>, L, L.smem, st, a); break;
+          case kColEta: seq_launch(k_col<T, D, kColEta, DynPlanX>, L, L.smem, st, a); break;
           default: return cudaErrorInvalidValue;
         }
         return cudaGetLastError();
@@ -376,10 +376,10 @@ struct Launchers {
       return cudaErrorInvalidValue;
     }
     switch (mode) {
-      case kColFwd: k_col<T, D, kColFwd><<<L.grid, L.block, L.smem, st>>>(a); break;
-      case kColInv: k_col<T, D, kColInv><<<L.grid, L.block, L.smem, st>>>(a); break;
-      case kColGreen: k_col<T, D, kColGreen><<<L.grid, L.block, L.smem, st>>>(a); break;
-      case kColEta: k_col<T, D, kColEta><<<L.grid, L.block, L.smem, st>>>(a); break;
+      case kColFwd: seq_launch(k_col<T, D, kColFwd>, L, L.smem, st, a); break;
+      case kColInv: seq_launch(k_col<T, D, kColInv>, L, L.smem, st, a); break;
+      case kColGreen: seq_launch(k_col<T, D, kColGreen>, L, L.smem, st, a); break;
+      case kColEta: seq_launch(k_col<T, D, kColEta>, L, L.smem, st, a); break;
       default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
@@ -399,7 +399,7 @@ struct Launchers {
   }
   static cudaError_t col_df(const Launch& L, const ColArgs<T>& a, const void* tw, cudaStream_t st) {
     if constexpr (kHasDf<T, D>) {
-      k_col_green_df<><<<L.grid, L.block, L.smem, st>>>(a, static_cast<const dfc*>(tw));
+      seq_launch(k_col_green_df<>, L, L.smem, st, a, static_cast<const dfc*>(tw));
       return cudaGetLastError();
     }
     return cudaErrorInvalidValue;
@@ -417,7 +417,7 @@ struct Launchers {
     return cudaErrorInvalidValue;
   }
   static cudaError_t cg_update(const Launch& L, const VecArgs<T>& v, cudaStream_t st) {
-#define FH_CGU(PP, XM) k_cg_update<T, NL, PP, XM><<<L.grid, L.block, 0, st>>>(v)
+#define FH_CGU(PP, XM) seq_launch(k_cg_update<T, NL, PP, XM>, L, 0, st, v)
     switch (v.xmode * 2 + (v.want_pp ? 1 : 0)) {
       case 0: FH_CGU(false, 0); break;
       case 1: FH_CGU(true, 0); break;
@@ -431,11 +431,11 @@ struct Launchers {
     return cudaGetLastError();
   }
   static cudaError_t cg_flush(const Launch& L, const VecArgs<T>& v, cudaStream_t st) {
-    k_cg_flush<T, NL><<<L.grid, L.block, 0, st>>>(v);
+    seq_launch(k_cg_flush<T, NL>, L, 0, st, v);
     return cudaGetLastError();
   }
   static cudaError_t bicg_update(const Launch& L, const VecArgs<T>& v, cudaStream_t st) {
-    k_bicg_update<T, NL><<<L.grid, L.block, 0, st>>>(v);
+    seq_launch(k_bicg_update<T, NL>, L, 0, st, v);
     return cudaGetLastError();
   }
   static cudaError_t current_sum(const Launch& L, const T* e, const uint8_t* ph, const double* tab,

@@ -272,6 +272,7 @@ struct Pipeline {
   // steps alternates the two direction buffers and settles x every second
   // iteration)
   cudaError_t enqueue_iter(int method, int j = 0);
+  cudaError_t field_iter(int method, int j);  // the same on the fields
   // CG items that stopped with an x step owed receive it (after the loop)
   cudaError_t enqueue_x_flush();
   bool has_after_loop() const { return defer_x_ || spec_run_; }

@@ -603,8 +603,8 @@ template <typename T>
 cudaError_t Pipeline<T>::spec_iter() {
   FH_CK(spec_passes());
   ++launches;
-  k_scal_spec<<<item_blocks(items), kSpecScalThreads, 0, st>>>(
-      scal, reinterpret_cast<const float2*>(part), scol.grid, ncell, nloads, (double)g.cell_nodes);
+  seq_launch(k_scal_spec, chain_launch(item_blocks(items), kSpecScalThreads), 0, st, scal,
+             reinterpret_cast<const float2*>(part), scol.grid, ncell, nloads, (double)g.cell_nodes);
   return cudaGetLastError();
 }
 
@@ -778,7 +778,17 @@ int Pipeline<T>::chunk_size(int method) const {
 
 template <typename T>
 cudaError_t Pipeline<T>::enqueue_iter(int method, int j) {
-  if (spec_run_) return spec_iter();
+  auto chain = [&](bool on) {
+    for (Launch* L : {&row, &col0, &col1, &vec, &scol, &smid, &srow}) L->chain = on;
+  };
+  chain(true);
+  const cudaError_t e = spec_run_ ? spec_iter() : field_iter(method, j);
+  chain(false);
+  return e;
+}
+
+template <typename T>
+cudaError_t Pipeline<T>::field_iter(int method, int j) {
   RowArgs<T> a = row_args();
   a.scal = scal;
   if (method == kCG) {
@@ -798,7 +808,7 @@ cudaError_t Pipeline<T>::enqueue_iter(int method, int j) {
     }
     FH_CK(passes(kProDir, kEpiDir, f, i, scal));
     ++launches;
-    k_scal_alpha<<<item_blocks(items), kRedThreads, 0, st>>>(scal, part, row.grid, ncell, nloads, 0);
+    seq_launch(k_scal_alpha, chain_launch(item_blocks(items), kRedThreads), 0, st, scal, part, row.grid, ncell, nloads, 0);
     FH_CK(cudaGetLastError());
     VecArgs<T> v;
     std::memset(&v, 0, sizeof(v));
@@ -822,7 +832,7 @@ cudaError_t Pipeline<T>::enqueue_iter(int method, int j) {
     ++launches;
     FH_CK(lt.cg_update(vec, v, st));
     ++launches;
-    k_scal_beta<<<item_blocks(items), kRedThreads, 0, st>>>(scal, part, vec.grid, ncell, nloads, 0,
+    seq_launch(k_scal_beta, chain_launch(item_blocks(items), kRedThreads), 0, st, scal, part, vec.grid, ncell, nloads, 0,
                                                             !defer_x_ ? -1 : (odd ? 1 : 0));
     FH_CK(cudaGetLastError());
     return hist_eta_e != nullptr && items == 1 ? enqueue_eta_record() : cudaSuccess;
@@ -844,7 +854,7 @@ cudaError_t Pipeline<T>::enqueue_iter(int method, int j) {
     FH_CK(passes(kProDirPlain, kEpiApplyT, ft, it, scal));
     FH_CK(passes(kProDir, kEpiDirShadow, f, i, scal));
     ++launches;
-    k_scal_alpha<<<item_blocks(items), kRedThreads, 0, st>>>(scal, part, row.grid, ncell, nloads, 1);
+    seq_launch(k_scal_alpha, chain_launch(item_blocks(items), kRedThreads), 0, st, scal, part, row.grid, ncell, nloads, 1);
     FH_CK(cudaGetLastError());
     VecArgs<T> v;
     std::memset(&v, 0, sizeof(v));
@@ -867,7 +877,7 @@ cudaError_t Pipeline<T>::enqueue_iter(int method, int j) {
     ++launches;
     FH_CK(lt.bicg_update(vec, v, st));
     ++launches;
-    k_scal_beta<<<item_blocks(items), kRedThreads, 0, st>>>(scal, part, vec.grid, ncell, nloads, 1, -1);
+    seq_launch(k_scal_beta, chain_launch(item_blocks(items), kRedThreads), 0, st, scal, part, vec.grid, ncell, nloads, 1, -1);
     FH_CK(cudaGetLastError());
     return hist_eta_e != nullptr && items == 1 ? enqueue_eta_record() : cudaSuccess;
   }
@@ -881,7 +891,7 @@ cudaError_t Pipeline<T>::enqueue_iter(int method, int j) {
   }
   FH_CK(passes(kProApply, kEpiFixed, f, i, scal));
   ++launches;
-  k_scal_fixed<<<item_blocks(items), kRedThreads, 0, st>>>(scal, part, row.grid, ncell, nloads);
+  seq_launch(k_scal_fixed, chain_launch(item_blocks(items), kRedThreads), 0, st, scal, part, row.grid, ncell, nloads);
   FH_CK(cudaGetLastError());
   return hist_eta_e != nullptr && items == 1 ? enqueue_eta_record() : cudaSuccess;
 }

@@ -6,11 +6,11 @@ namespace fh {
 cudaError_t spec_inv(int mode, const Launch& L, const SpecArgs& a, cudaStream_t st) {
   if (mode == kSpecFinish)
     return on_plan<PlanList<>, true>(a.plan, [&](auto t) {
-      k_spec_inv<kSpecFinish, decltype(t)><<<L.grid, L.block, L.smem, st>>>(a);
+      seq_launch(k_spec_inv<kSpecFinish, decltype(t)>, L, L.smem, st, a);
       return cudaGetLastError();
     });
   return on_plan<SpecPlans, true>(a.plan, [&](auto t) {
-    k_spec_inv<kSpecUpdate, decltype(t)><<<L.grid, L.block, L.smem, st>>>(a);
+    seq_launch(k_spec_inv<kSpecUpdate, decltype(t)>, L, L.smem, st, a);
     return cudaGetLastError();
   });
 }
@@ -18,18 +18,18 @@ cudaError_t spec_inv(int mode, const Launch& L, const SpecArgs& a, cudaStream_t 
 cudaError_t spec_fwd(int mode, const Launch& L, const SpecArgs& a, cudaStream_t st) {
   if (mode == kSpecProject)
     return on_plan<PlanList<>, true>(a.plan, [&](auto t) {
-      k_spec_fwd<kSpecProject, decltype(t)><<<L.grid, L.block, L.smem, st>>>(a);
+      seq_launch(k_spec_fwd<kSpecProject, decltype(t)>, L, L.smem, st, a);
       return cudaGetLastError();
     });
   return on_plan<SpecPlans, true>(a.plan, [&](auto t) {
-    k_spec_fwd<kSpecApply, decltype(t)><<<L.grid, L.block, L.smem, st>>>(a);
+    seq_launch(k_spec_fwd<kSpecApply, decltype(t)>, L, L.smem, st, a);
     return cudaGetLastError();
   });
 }
 
 cudaError_t spec_green(const Launch& L, const SpecArgs& a, cudaStream_t st) {
   return on_plan<SpecPlans, true>(a.plan, [&](auto t) {
-    k_spec_green<decltype(t)><<<L.grid, L.block, L.smem, st>>>(a);
+    seq_launch(k_spec_green<decltype(t)>, L, L.smem, st, a);
     return cudaGetLastError();
   });
 }

@@ -6,9 +6,9 @@ namespace fh {
 cudaError_t spec_mid(bool inv, const Launch& L, const SpecMidArgs& a, cudaStream_t st) {
   return on_plan<SpecPlans3D, true>(a.plan, [&](auto t) {
     if (inv)
-      k_spec_mid<true, decltype(t)><<<L.grid, L.block, L.smem, st>>>(a);
+      seq_launch(k_spec_mid<true, decltype(t)>, L, L.smem, st, a);
     else
-      k_spec_mid<false, decltype(t)><<<L.grid, L.block, L.smem, st>>>(a);
+      seq_launch(k_spec_mid<false, decltype(t)>, L, L.smem, st, a);
     return cudaGetLastError();
   });
 }

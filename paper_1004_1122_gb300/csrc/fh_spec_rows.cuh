@@ -21,14 +21,14 @@ template <int D, int NL, typename Plans> struct SpecRows {
   static cudaError_t run(int mode, const Launch& L, const SpecRowArgs& a, cudaStream_t st) {
     if (mode == kSpecRowTau)
       return hot(a.plan, L, [&](auto t) {
-        k_spec_row<D, NL, kSpecRowTau, decltype(t)><<<L.grid, L.block, L.smem, st>>>(a);
+        seq_launch(k_spec_row<D, NL, kSpecRowTau, decltype(t)>, L, L.smem, st, a);
         return cudaGetLastError();
       });
     return ends(a.plan, L, [&](auto t) {
       if (mode == kSpecRowLoad)
-        k_spec_row<D, NL, kSpecRowLoad, decltype(t)><<<L.grid, L.block, L.smem, st>>>(a);
+        seq_launch(k_spec_row<D, NL, kSpecRowLoad, decltype(t)>, L, L.smem, st, a);
       else
-        k_spec_row<D, NL, kSpecRowAdd, decltype(t)><<<L.grid, L.block, L.smem, st>>>(a);
+        seq_launch(k_spec_row<D, NL, kSpecRowAdd, decltype(t)>, L, L.smem, st, a);
       return cudaGetLastError();
     });
   }

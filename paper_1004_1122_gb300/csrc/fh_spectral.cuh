@@ -232,6 +232,7 @@ inline size_t spec_col_smem(int ss, int Q, int rows, int block) {
 // the new direction.  kSpecFinish: the inverse FFT of x + (owed step).
 template <int MODE, typename PS = DynPlan>
 __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_inv(SpecArgs a) {
+  seq_begin();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* sm = reinterpret_cast<float2*>(smem_raw);
   const int n = plan_len<PS>(a.plan), C = a.sg.C, csh = a.sg.csh, nl = a.nl;
@@ -329,6 +330,7 @@ __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_inv(SpecArgs a
 // kSpecProject: the scalars of a real residual field's spectrum into r.
 template <int MODE, typename PS = DynPlan>
 __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_fwd(SpecArgs a) {
+  seq_begin();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* sm = reinterpret_cast<float2*>(smem_raw);
   const int n = plan_len<PS>(a.plan), C = a.sg.C, csh = a.sg.csh, nl = a.nl;
@@ -425,6 +427,7 @@ __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_fwd(SpecArgs a
 // pass took 21 us; 2-D 49 us on 2187^2, bound by the shared-memory stages.
 template <typename PS = DynPlan>
 __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_green(SpecArgs a) {
+  seq_begin();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* sm = reinterpret_cast<float2*>(smem_raw);
   const int n = plan_len<PS>(a.plan), C = a.sg.C, nl = a.nl;
@@ -500,6 +503,7 @@ struct SpecMidArgs {
 
 template <bool INV, typename PS = DynPlan>
 __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_mid(SpecMidArgs a) {
+  seq_begin();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* sm = reinterpret_cast<float2*>(smem_raw);
   const Geom& g = a.g;
@@ -612,6 +616,7 @@ inline size_t spec_row_smem(int d, int nl, int lpc, int n, int ss, int nphase) {
 
 template <int D, int NL, int MODE, typename PS = DynPlan>
 __global__ void __launch_bounds__(SpecRowBounds<PS>::threads, SpecRowBounds<PS>::blocks) k_spec_row(SpecRowArgs a) {
+  seq_begin();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* sm = reinterpret_cast<float2*>(smem_raw);
   const Geom& g = a.g;
@@ -896,6 +901,7 @@ __global__ void __launch_bounds__(SpecRowBounds<PS>::threads, SpecRowBounds<PS>:
 constexpr int kSpecScalThreads = 512;
 static __global__ void __launch_bounds__(kSpecScalThreads) k_scal_spec(Scal* scal, const float2* part, int np, int ncell,
                                                                        int nl, double nfac) {
+  seq_begin();
   const ItemRef r = item_ref(np, ncell, nl);
   if (!r.valid) return;
   Scal& s = scal[r.item];
