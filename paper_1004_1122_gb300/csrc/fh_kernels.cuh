@@ -226,6 +226,7 @@ template <typename T> struct ColArgs {
   Scal* scal;
   double* part;
   const double* L0cell;  // per-cell reference medium [ncell][9], or nullptr for g.L0
+  const T* green;        // spread plans: table of k_green_tab
   int* err;              // device error word (bounded waits that expired), or nullptr
   unsigned long long wait_ns;  // limit of the bounded waits (0: tma::kWaitLimitNs)
 };
@@ -573,6 +574,56 @@ struct GreenPoint2 {
   }
 };
 
+// GreenPoint2 from a table: [cell][frequency of the last axis][row] of
+// 1 / (xi . L0 . xi) / |N| (zero where the operator is), then xi_0 of every
+// row.  The factor's division, products and integer conversions take ~25
+// float64 operations per value, as many as a radix-3 stage; from the table it
+// takes 7 and a load.  Only for spread plans, whose tables stay in L2.
+static __global__ void k_green_tab(Geom g, const double* L0cell, double* tab) {
+  const int n = g.n[0], TC = g.Tt * g.C;
+  const long long len = (long long)g.ncell * TC * n;
+  const long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  if (idx >= len + n) return;
+  const int i = (int)(idx % n);
+  const double xi0 = (double)signed_freq(i, n) * g.invY[0];
+  if (idx >= len) {
+    tab[idx] = xi0;
+    return;
+  }
+  const int kl = (int)(idx / n % TC);
+  const double* const L0 = L0cell ? L0cell + 9 * (idx / n / TC) : g.L0;
+  const double xi1 = (double)kl * g.invY[1];
+  const bool zero = kl >= g.H || nyquist_bin(kl, g.nlast) || nyquist_bin(i, n) || (i == 0 && kl == 0);
+  const double den = xi0 * (L0[0] * xi0 + L0[1] * xi1) + xi1 * (L0[3] * xi0 + L0[4] * xi1);
+  tab[idx] = zero ? 0.0 : g.inv_nodes / den;
+}
+template <typename T>
+struct GreenPointTab {
+  const T *f, *x0;
+  T xi1;
+  int a;
+  __device__ __forceinline__ void init(const ColArgs<T>& c, int t, int q, int cell, int n) {
+    const Geom& g = c.b.g;
+    const int TC = g.Tt * g.C, kl = t * g.C + (q / g.M) % g.C;
+    f = c.green + ((long long)cell * TC + kl) * n;
+    x0 = c.green + (long long)g.ncell * TC * n;
+    xi1 = T(kl) * T(g.invY[1]);
+    a = q & 1;
+  }
+  __device__ __forceinline__ cplx<T> operator()(cplx<T> v, int i, bool act) const {
+    cplx<T> o;
+    o.x = __shfl_xor_sync(0xffffffffu, v.x, 1);
+    o.y = __shfl_xor_sync(0xffffffffu, v.y, 1);
+    const T xi0 = act ? __ldg(x0 + i) : T(0), fk = act ? __ldg(f + i) : T(0);
+    const T own = a == 0 ? xi0 : xi1, oth = a == 0 ? xi1 : xi0;
+    const T w = own * fk;
+    cplx<T> y;
+    y.x = w * (own * v.x + oth * o.x);
+    y.y = w * (own * v.y + oth * o.y);
+    return y;
+  }
+};
+
 // Green projection of one column tile held in shared memory (after the
 // forward FFT along axis 0): y^(k) = xi (xi . tau^(k)) / (xi . L0 . xi) / |N|,
 // zero at k = 0 and on padded frequencies (kColGreen), or the equilibrium-norm
@@ -730,10 +781,16 @@ __global__ void __launch_bounds__(ColBounds<PS>::threads, ColBounds<PS>::blocks)
     // inverse FFTs.  Q = C * M is even and the two components of a frequency
     // sit in columns q and q ^ 1, i.e. adjacent lanes of one warp.
     const int t = blk_outer;
-    const double* L0src = a.L0cell ? a.L0cell + 9 * cell : g.L0;
-    GreenPoint2<T, QC ? PlanLen<PS>::value : 0> gp;
-    gp.init(g, L0src, t, q, n);
-    fft_fused_plan<T, PS>(sm + q, Q, b.plan, u, tpc, a.tw, gp);
+    if constexpr (std::is_same<PS, DynPlanW>::value) {
+      GreenPointTab<T> gp;
+      gp.init(a, t, q, cell, n);
+      fft_fused_plan<T, PS>(sm + q, Q, b.plan, u, tpc, a.tw, gp);
+    } else {
+      const double* L0src = a.L0cell ? a.L0cell + 9 * cell : g.L0;
+      GreenPoint2<T, QC ? PlanLen<PS>::value : 0> gp;
+      gp.init(g, L0src, t, q, n);
+      fft_fused_plan<T, PS>(sm + q, Q, b.plan, u, tpc, a.tw, gp);
+    }
   } else {
   if (CM_ == kColFwd || CM_ == kColGreen || CM_ == kColEta)
     fft_plan<false, T, PS>(sm + q, Q, b.plan, u, tpc, a.tw);

@@ -155,6 +155,7 @@ struct Pipeline {
   int ncell = 1;
   int items = 1;             // ncell * nloads
   double* L0cell_dev = nullptr;
+  T* green_tab = nullptr;      // 2-D spread plans: the Green operator's factors (k_green_tab)
   long long vlen = 0;        // d * nodes
   T* x[kMaxLoads] = {};
   T* r[kMaxLoads] = {};

@@ -335,6 +335,14 @@ int Pipeline<T>::init(const Problem& pb, int nloads_, bool krylov, cudaStream_t 
     if ((rc = dev_alloc(allocs, &L0cell_dev, (size_t)9 * ncell, err))) return rc;
     FH_CKS(cudaMemcpy(L0cell_dev, pb.L0cell.data(), 9 * ncell * sizeof(double), cudaMemcpyHostToDevice));
   }
+  if constexpr (std::is_same<T, double>::value) {
+    if (d == 2 && pcol0.ext == kRadixSpread) {
+      const size_t len = (size_t)ncell * g.Tt * g.C * g.n[0] + g.n[0];
+      if ((rc = dev_alloc(allocs, &green_tab, len, err))) return rc;
+      k_green_tab<<<(int)((len + 255) / 256), 256, 0, st>>>(g, L0cell_dev, green_tab);
+      FH_CKS(cudaGetLastError());
+    }
+  }
   if (krylov) {
     // one block for the field vectors, each on a 256-byte boundary (with p2,
     // the second direction buffer of CG, where it is needed from the start)
@@ -707,6 +715,7 @@ cudaError_t Pipeline<T>::launch_green(int mode, Scal* sc, double* pt) {
   a.scal = sc;
   a.part = pt;
   a.L0cell = L0cell_dev;
+  a.green = green_tab;
   a.err = dev_err;
   m.err = dev_err;
   a.wait_ns = m.wait_ns = tma::wait_limit_ns();
