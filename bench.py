@@ -404,7 +404,8 @@ def run_reference(args):
 # capture of these kernels measured).
 KERNEL_SOURCES = ("fh_fft.cuh", "fh_dfloat.cuh", "fh_kernels.cuh", "fh_tma.cuh", "fh_plan.h",
                   "fh_launch.cuh", "fh_launch_impl.cuh", "fh_launch_f32_d2.cu", "fh_pipeline.cuh",
-                  "fh_pipeline_impl.cuh")
+                  "fh_pipeline_impl.cuh", "fh_spectral.cuh", "fh_spec_plans.cuh", "fh_spec_cols.cu",
+                  "fh_spec_mids.cu", "fh_spec_rows.cuh", "fh_spec_rows_d2.cu", "fh_spec_rows_d3.cu")
 
 
 def csrc_digest() -> str:

@@ -114,7 +114,7 @@ typedef struct {
 #define FH_INFO_ETA_E 1
 
 /* fh_info.ct_plans bits: compile-time plans of the float32 CG-iteration passes */
-#define FH_CT_2187 1      /* 2-D, one load per launch, 2187 = 27 * 27 * 3 along both axes */
+#define FH_CT_2187 1      /* 2-D, one load per launch, 2187 = 27 * 3 * 27 along both axes */
 #define FH_CT_729 2       /* 2-D, two loads per launch, 729 = 27 * 27 along both axes */
 #define FH_CT_243 4       /* 3-D, one or three loads per launch, 243 = 27 * 9 along every axis */
 
@@ -212,7 +212,10 @@ fh_status fh_eta_e(fh_ctx* ctx, const double* e, double* eta);
  * launches of one piece of the CG iteration on the context stream with CUDA
  * events after 3 warm-up launches, and writes the average milliseconds per
  * launch to *ms.  The context's Krylov vectors are overwritten (zeroed); any
- * solve state is lost.
+ * solve state is lost.  The pieces are those of the iteration on fields
+ * (FH_FP64 and FH_FP32 contexts, BiCG and the fixed point); the CG iterations
+ * of FH_FP32_REFINED contexts run in the frequency domain and have passes of
+ * their own, and so has the float32 product (5).
  *  dtype  FH_FP64 or FH_FP32 (pipeline to time)
  *  what   0 row-forward pass (p = r + beta p, dL p, forward line FFTs)
  *         1 column passes with the Green projection

@@ -10,10 +10,9 @@
  *
  * Network (all kernels hand-written, float32 activations, bfloat16-rounded
  * weights, float32 accumulation; levels N, N/3, N/9, N/27; channels c0..c3;
- * layers 0..10 in parameter order).  The forward convolutions and the data
- * gradients run on the tensor cores (tcgen05, each float32 activation or
- * gradient split into two bfloat16 halves), the weight gradients on the CUDA
- * cores:
+ * layers 0..10 in parameter order).  The convolutions, the data gradients and
+ * the weight gradients run on the tensor cores (tcgen05, each float32
+ * activation or gradient split into two bfloat16 halves):
  *   a0 = leaky(conv0(x))            a1 = leaky(conv1(pool(a0)))
  *   a2 = leaky(conv2(pool(a1)))     a3 = leaky(conv3(pool(a2)))
  *   v2 = up(leaky(conv4(a3))) + a2  u2 = leaky(conv5(v2))
