@@ -1533,7 +1533,9 @@ int Pipeline<T>::profile(int what, int reps, double* ms, std::string& err) {
       case 1: return launch_green(kColGreen, scal, nullptr);
       case 2: return launch_row_inv(kEpiDir, i);
       case 3: ++launches; return lt.cg_update(vec, v, st);
-      case 5: return passes(kProApply, kEpiApply, app, app, nullptr);
+      case 5:
+        if (nloads == 1) return apply(app.in[0], app.out[0], false);
+        return passes(kProApply, kEpiApply, app, app, nullptr);
       default: return cudaErrorInvalidValue;
     }
   };
