@@ -380,8 +380,9 @@ int Pipeline<T>::upload_twiddles(const FFTPlan& pl, W** dst, std::string& err) {
   return 0;
 }
 
-// Launch shapes and buffers of the frequency-domain CG iteration.  Left off
-// (spectral = false) where a tile or line does not fit one CTA.
+// Launch shapes and buffers of the frequency-layout passes and the CG iteration
+// in the frequency domain.  Left off (spec_ops, spectral false: passes on
+// fields) where a tile or a line does not fit one CTA.
 template <typename T>
 int Pipeline<T>::init_spectral(const Problem& pb, std::string& err) {
   if constexpr (std::is_same<T, float>::value) {
@@ -470,7 +471,11 @@ int Pipeline<T>::init_spectral(const Problem& pb, std::string& err) {
       });
     });
     srow.smem = spec_row_smem(d, nl, slpc, g.nlast, ssrow, nphase);
-    if (srow.smem > cap || srow.block > 768 || scol.smem > cap) return 0;
+    // kRowMaxThreads bounds the run-time-plan kernels, which run every launch
+    // above kSpecRowCtThreads; a pair of 3-D lines of 2640 nodes and more can
+    // need more threads, and the passes on fields (which pack the channels of
+    // one line) then do the work.
+    if (srow.smem > cap || srow.block > kRowMaxThreads || scol.smem > cap) return 0;
     const bool more_part = scol.grid > part_stride;
     part_stride = std::max(part_stride, scol.grid);
     FH_CKS(spec_col_set_smem(spec_args(), scol.smem));
