@@ -770,9 +770,13 @@ fh_status fh_solve(fh_ctx* c, const double* E, double tol, int method, int max_i
       double M[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
       for (int i = 0; i < d; ++i)
         for (int j = 0; j < d; ++j) M[i * 3 + j] = c->pb.L0[i * d + j];
-      double n2;
-      rc = P->spec_run_ ? P->spec_dir_norm2(M, &n2, err) : P->matnorm2(P->p[0], M, &n2, err);
-      if (rc) return from_rc(c, rc, err);
+      double n2 = 0.0;
+      // no iteration: there was no step (and the frequency-domain solve has not
+      // written its direction)
+      if (res.iters > 0) {
+        rc = P->spec_run_ ? P->spec_dir_norm2(M, &n2, err) : P->matnorm2(P->p[0], M, &n2, err);
+        if (rc) return from_rc(c, rc, err);
+      }
       eta_r = std::fabs(last_alpha) * std::sqrt(n2 / e2);
     }
     fh_status fs = finish_info(c, P, info, hist_len);
