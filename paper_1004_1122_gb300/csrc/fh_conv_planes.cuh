@@ -381,22 +381,28 @@ template <int T, int NT> __global__ void __launch_bounds__(kConvThreads) k_conv_
         }
         commit(&tfull[buf]);
       }
-      // every issued MMA has finished before tensor memory is released
+      // every issued MMA has finished before tensor memory is released, and every
+      // commit has arrived before the CTA leaves (the epilogue, which waits for
+      // the accumulators' commits, may have given up)
       for (int st = 0; st < nstage; ++st) {
         const int cnt = (it + nstage - 1 - st) >> ssh;
         if (cnt > 0) tma::mbar_wait(&empty[st], (cnt - 1) & 1);
+      }
+      for (int b = 0; b < 2; ++b) {
+        const int cnt = (nt + 1 - b) >> 1;  // commits of this accumulator
+        if (cnt > 0) tma::mbar_wait(&tfull[b], (cnt - 1) & 1);
       }
     }
   } else {
     const long long V = g.v();
     int nt = 0;
-    for (int tile = blockIdx.x; tile < ntile && !s_fail; tile += gridDim.x, ++nt) {
+    // a warp goes on or gives up as a whole (its tensor-memory loads need all lanes)
+    for (int tile = blockIdx.x; tile < ntile && !__any_sync(0xffffffffu, s_fail); tile += gridDim.x, ++nt) {
       const int buf = nt & 1;
-      if (!tma::mbar_wait(&tfull[buf], (nt >> 1) & 1, a.wait_ns)) {
+      if (!__all_sync(0xffffffffu, tma::mbar_wait(&tfull[buf], (nt >> 1) & 1, a.wait_ns))) {
         s_fail = 1;
         break;
       }
-      __syncwarp();
       fence_after();
       const int z = tile / a.tiles_z, k = tile - z * a.tiles_z;
       constexpr int K16 = NT / 16;
