@@ -41,8 +41,7 @@ typedef struct fh_nn fh_nn;
  * cout output channels (each <= 64), channels[4] = (c0, c1, c2, c3), each
  * <= 64, or NULL for (16, 32, 48, 64).  Parameters start at zero (set them
  * with fh_nn_set_params).  stream: cudaStream_t or NULL.
- * Errors: FH_ERR_ARG, FH_ERR_OOM, FH_ERR_CUDA (FH_ERR_TIMEOUT from the
- * synchronising calls if a tensor-core kernel's bounded wait expired). */
+ * Errors: FH_ERR_ARG, FH_ERR_OOM, FH_ERR_CUDA. */
 fh_status fh_nn_create(fh_nn** out, const int* N, int cin, int cout, const int* channels, void* stream);
 
 /* Number of float32 parameters. */
@@ -60,11 +59,16 @@ fh_status fh_nn_forward(fh_nn* nn, const float* x, float* y);
 
 /* Forward, mean-squared-error loss against target (device [cout][N...]) and
  * backward.  *loss (host, may be NULL) receives the loss; grad_host (host,
- * param_count floats, may be NULL) receives the gradient.  Synchronises. */
+ * param_count floats, may be NULL) receives the gradient.  Synchronises.
+ * FH_ERR_TIMEOUT: a tensor-core kernel's bounded wait expired in this call or
+ * in an fh_nn_forward before it; reported once, with *loss and grad_host left
+ * as they were. */
 fh_status fh_nn_gradients(fh_nn* nn, const float* x, const float* target, double* loss, float* grad_host);
 
 /* One Adam step (beta1 0.9, beta2 0.999, eps 1e-8, bias correction with the
- * 1-based step count) on the gradients of the MSE loss at (x, target). */
+ * 1-based step count) on the gradients of the MSE loss at (x, target).  After
+ * an error of fh_nn_gradients (FH_ERR_TIMEOUT among them) the parameters and
+ * moments are as before. */
 fh_status fh_nn_train_step(fh_nn* nn, const float* x, const float* target, float lr, int step, double* loss);
 
 void fh_nn_destroy(fh_nn* nn);

@@ -199,7 +199,7 @@ struct fh_nn {
   float *gy = nullptr, *gu[3] = {}, *gv[3] = {}, *ga3 = nullptr, *gp[3] = {}, *gt = nullptr;
   uint4 *GA = nullptr, *GB[kLayers] = {};
   double* part = nullptr;
-  double* h_part = nullptr;
+  double* h_part = nullptr;                      // pinned: loss partials, error word
   int npart = 0;
   void* slab = nullptr;                          // the one allocation behind all of it
   long long launches = 0;
@@ -423,27 +423,31 @@ cudaError_t backward(fh_nn* n) {
 }
 #undef FH_NN
 
-// true when a kernel's bounded wait expired (synchronises the stream)
-bool device_error(fh_nn* n) {
-  int h = 0;
-  if (cudaMemcpyAsync(&h, n->dev_err, sizeof(int), cudaMemcpyDeviceToHost, n->st) != cudaSuccess ||
-      cudaStreamSynchronize(n->st) != cudaSuccess)
-    return true;
-  return h != 0;
+// gy = gradient of the mean squared error of y, partial sums of the loss in part
+cudaError_t loss_gradient(fh_nn* n, const float* target) {
+  const long long cnt = n->lv[0].v() * n->cout;
+  ++n->launches;
+  k_mse<<<std::min(n->npart, grid1(cnt)), kThreads, 0, n->st>>>(n->y, target, n->gy, cnt, n->part);
+  return cudaGetLastError();
 }
 
-int loss_grad(fh_nn* n, const float* target, double* loss) {
+// Waits for what is queued, reads the loss and the device error word (bounded
+// waits that expired, in this call or an earlier forward); a word that was set
+// is reported once and cleared.
+int finish(fh_nn* n, double* loss) {
   const long long cnt = n->lv[0].v() * n->cout;
   const int g = std::min(n->npart, grid1(cnt));
-  ++n->launches;
-  k_mse<<<g, kThreads, 0, n->st>>>(n->y, target, n->gy, cnt, n->part);
-  if (cudaMemcpyAsync(n->h_part, n->part, g * sizeof(double), cudaMemcpyDeviceToHost, n->st) != cudaSuccess)
+  int* const h_err = reinterpret_cast<int*>(n->h_part + n->npart);
+  if (cudaMemcpyAsync(n->h_part, n->part, g * sizeof(double), cudaMemcpyDeviceToHost, n->st) != cudaSuccess ||
+      cudaMemcpyAsync(h_err, n->dev_err, sizeof(int), cudaMemcpyDeviceToHost, n->st) != cudaSuccess ||
+      cudaStreamSynchronize(n->st) != cudaSuccess)
     return FH_ERR_CUDA;
-  if (cudaStreamSynchronize(n->st) != cudaSuccess) return FH_ERR_CUDA;
+  if (*h_err != 0)
+    return cudaMemsetAsync(n->dev_err, 0, sizeof(int), n->st) == cudaSuccess ? FH_ERR_TIMEOUT : FH_ERR_CUDA;
   double s = 0.0;
   for (int i = 0; i < g; ++i) s += n->h_part[i];
   if (loss) *loss = s / (double)cnt;
-  return device_error(n) ? FH_ERR_TIMEOUT : 0;
+  return 0;
 }
 
 }  // namespace
@@ -580,7 +584,7 @@ fh_status fh_nn_create(fh_nn** out, const int* N, int cin, int cout, const int* 
   for (int k = 0; k <= kLayers && !rc; ++k)
     if (cudaEventCreateWithFlags(k < kLayers ? &n->fork[k] : &n->join, cudaEventDisableTiming) != cudaSuccess) rc = FH_ERR_CUDA;
   if (!rc && cudaStreamCreateWithFlags(&n->side, cudaStreamNonBlocking) != cudaSuccess) rc = FH_ERR_CUDA;
-  if (!rc && cudaMallocHost(&n->h_part, n->npart * sizeof(double)) != cudaSuccess) rc = FH_ERR_OOM;
+  if (!rc && cudaMallocHost(&n->h_part, (n->npart + 1) * sizeof(double)) != cudaSuccess) rc = FH_ERR_OOM;
   if (!rc && (cudaMemsetAsync(n->slab, 0, planes, n->st) != cudaSuccess ||
               cudaMemsetAsync(n->dev_err, 0, sizeof(int), n->st) != cudaSuccess ||
               cudaMemsetAsync(n->Mo, 0, off * sizeof(float), n->st) != cudaSuccess ||
@@ -624,10 +628,13 @@ fh_status fh_nn_forward(fh_nn* n, const float* x, float* y) {
 
 fh_status fh_nn_gradients(fh_nn* n, const float* x, const float* target, double* loss, float* grad_host) {
   if (!n || !x || !target) return FH_ERR_ARG;
-  if (forward(n, x, n->y) != cudaSuccess) return FH_ERR_CUDA;
-  int rc = loss_grad(n, target, loss);
+  // the error word is read behind the backward pass: its waits are bounded too
+  if (forward(n, x, n->y) != cudaSuccess || loss_gradient(n, target) != cudaSuccess || backward(n) != cudaSuccess) {
+    cudaStreamSynchronize(n->side);  // weight gradients that were launched read this call's planes
+    return FH_ERR_CUDA;
+  }
+  const int rc = finish(n, loss);
   if (rc) return (fh_status)rc;
-  if (backward(n) != cudaSuccess) return FH_ERR_CUDA;
   if (grad_host) {
     if (cudaMemcpyAsync(grad_host, n->G, n->nparam * sizeof(float), cudaMemcpyDeviceToHost, n->st) != cudaSuccess ||
         cudaStreamSynchronize(n->st) != cudaSuccess)
