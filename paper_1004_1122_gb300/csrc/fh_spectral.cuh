@@ -16,16 +16,21 @@
 //   spec_mid  3-D: inverse FFT along axis 1 of (v_0, xi_1 g, xi_2 g).
 //   spec_row  lines: inverse FFT, tau = dL v at the nodes, forward FFT, in place.
 //   spec_mid  3-D: forward FFT along axis 1, (tau_0, xi_1 tau_1 + xi_2 tau_2).
-//   spec_fwd  columns along axis 0: forward FFT, projection, A p, (p, A p), (A p, A p).
+//   spec_fwd  columns along axis 0: forward FFT, projection, A p, (p, A p), (A p, A p),
+//             (r, A p).
 //   k_scal_spec  alpha, beta and the stopping tests from one reduction.
 //
 // The next (r, r) follows from the reductions of spec_fwd,
-// (r+, r+) = alpha^2 (A p, A p) - (r, r) since (r, A p) = (p, A p), and the
-// stored residual's own (r, r) replaces it one iteration later as the
-// numerator of alpha, so rounding does not accumulate.
+//   (r+, r+) = (r, r) - 2 alpha (r, A p) + alpha^2 (A p, A p),
+// and the stored residual's own (r, r) replaces it one iteration later as the
+// numerator of alpha, so rounding does not accumulate.  All three products are
+// measured: the expansion is then within 1e-7 of the (r+, r+) of the stored
+// residual (the rounding of its elements; contrast 10 to 1e4 in a float32
+// model of the iteration), where (p, A p) in place of (r, A p), its value for a
+// symmetric A in exact arithmetic, is 1e-6 off.
 //
-// Memory moved per iteration in units of one real scalar per node: 18.25 in
-// 2-D (113 / 4 = 28.25 with the fields' passes), 31.25 in 3-D (59.25).
+// Memory moved per iteration in units of one real scalar per node: 19.25 in
+// 2-D (113 / 4 = 28.25 with the fields' passes), 32.25 in 3-D (59.25).
 // Measured per iteration, against the passes on fields: 2187^2 168 -> 127 us
 // (row 44, inv 43, fwd 33, scalars 7; 349 MB, 51 us at the copy rate), 243^3
 // with three loads 2.54 -> 1.43 ms (row 402, inv 284, mid 271 + 253, fwd 217;
@@ -78,7 +83,7 @@ struct SpecArgs {
   float2* x[kMaxLoads];
   Scal* scal;
   // partial sums as two-float values, one per CTA: (p, A p) rows 0..,
-  // (A p, A p) rows kMaxLoads.., (r, r) rows 2 kMaxLoads..
+  // (A p, A p) rows kMaxLoads.., (r, A p) rows 2 kMaxLoads.., (r, r) rows 3 kMaxLoads..
   float2* part;
   const SpecMedium* med;       // per cell
 };
@@ -329,10 +334,10 @@ __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_inv(SpecArgs a
     S[w.i * rs + w.j] = make_float4(v0.x, v0.y, v1.x, v1.y);
   }
   if (MODE == kSpecUpdate)
-    ff_rows_store(red, nl, [&](int k, float2 v) { a.part[(size_t)(2 * kMaxLoads + k) * gridDim.x + tl.slot] = v; });
+    ff_rows_store(red, nl, [&](int k, float2 v) { a.part[(size_t)(3 * kMaxLoads + k) * gridDim.x + tl.slot] = v; });
 }
 
-// kSpecApply: A p of the direction's tau spectrum, with (p, A p) and (A p, A p).
+// kSpecApply: A p of the direction's tau spectrum, with (p, A p), (A p, A p) and (r, A p).
 // kSpecProject: the scalars of a real residual field's spectrum into r.
 template <int MODE, typename PS = DynPlan>
 __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_fwd(SpecArgs a) {
@@ -375,21 +380,24 @@ __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_fwd(SpecArgs a
   fq[0].init(a, a.med[tl.cell], n, tl.t * C + e, tl.inner);
   fq[1].init(a, a.med[tl.cell], n, tl.t * C + e + 1, tl.inner);
   for (int l = 0; l < nl; ++l) {
-    DotAcc<float> d1[2], d2[2];
+    DotAcc<float> d1[2], d2[2], d3[2];
     if (MODE == kSpecProject || sc[l].done == kRunning) {
       const float4* const p = reinterpret_cast<const float4*>(a.p[l] + tl.sbase + e);
+      const float4* const r = reinterpret_cast<const float4*>(a.r[l] + tl.sbase + e);
       float4* const out = reinterpret_cast<float4*>((MODE == kSpecApply ? a.ap[l] : a.r[l]) + tl.sbase + e);
       const float2* const ch = sm + (size_t)(e * nl + l) * 2 * a.ss;
       const int next = 2 * nl * a.ss;
-      for (int i0 = row0; i0 < n; i0 += kUnroll * drow) {
-        float4 vp[kUnroll];
+      constexpr int kUnrollA = 2;  // 4 spill
+      for (int i0 = row0; i0 < n; i0 += kUnrollA * drow) {
+        float4 vp[kUnrollA], vr[kUnrollA];
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
+        for (int u = 0; u < kUnrollA; ++u) {
           const int i = i0 + u * drow;
           vp[u] = (MODE == kSpecApply && i < n) ? __ldg(p + (i << (csh - 1))) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+          vr[u] = (MODE == kSpecApply && i < n) ? __ldg(r + (i << (csh - 1))) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         }
 #pragma unroll
-        for (int u = 0; u < kUnroll; ++u) {
+        for (int u = 0; u < kUnrollA; ++u) {
           const int i = i0 + u * drow;
           if (i >= n) continue;
           const float x0 = fq[0].xi0(i);
@@ -403,8 +411,10 @@ __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_fwd(SpecArgs a
             y[h] = make_float2(w0 * v0.x + w1 * v1.x, w0 * v0.y + w1 * v1.y);
             if (MODE == kSpecApply) {
               const float2 q = h ? make_float2(vp[u].z, vp[u].w) : make_float2(vp[u].x, vp[u].y);
+              const float2 rv = h ? make_float2(vr[u].z, vr[u].w) : make_float2(vr[u].x, vr[u].y);
               y[h].x += q.x;
               y[h].y += q.y;
+              d3[h].add(rv.x * y[h].x + rv.y * y[h].y);
               d1[h].add(q.x * y[h].x + q.y * y[h].y);
               d2[h].add(y[h].x * y[h].x + y[h].y * y[h].y);
             }
@@ -416,12 +426,13 @@ __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_fwd(SpecArgs a
     if (MODE == kSpecApply) {
       red[l * blockDim.x + threadIdx.x] = ff_add(ff_of(d1[0], fq[0].wgt), ff_of(d1[1], fq[1].wgt));
       red[(nl + l) * blockDim.x + threadIdx.x] = ff_add(ff_of(d2[0], fq[0].wgt), ff_of(d2[1], fq[1].wgt));
+      red[(2 * nl + l) * blockDim.x + threadIdx.x] = ff_add(ff_of(d3[0], fq[0].wgt), ff_of(d3[1], fq[1].wgt));
     }
   }
   if (MODE == kSpecApply) {
     __syncthreads();
-    ff_rows_store(red, 2 * nl, [&](int k, float2 v) {
-      a.part[(size_t)(k < nl ? k : kMaxLoads + k - nl) * gridDim.x + tl.slot] = v;
+    ff_rows_store(red, 3 * nl, [&](int k, float2 v) {
+      a.part[(size_t)(k / nl * kMaxLoads + k % nl) * gridDim.x + tl.slot] = v;
     });
   }
 }
@@ -914,44 +925,41 @@ static __global__ void __launch_bounds__(kSpecScalThreads) k_scal_spec(Scal* sca
   // what thread 0 needs afterwards is loaded together with the partial sums
   const int done = s.done, iter = s.iter, max_iter = s.max_iter;
   const double b2 = s.b2, tol2 = s.tol2, ib2 = s.ib2;
-  float2 v[3];
+  float2 v[4];
 #pragma unroll
-  for (int k = 0; k < 3; ++k) {
+  for (int k = 0; k < 4; ++k) {
     const float2* const p = part + (long long)(k * kMaxLoads + r.l) * np + (long long)r.cell * r.bpc;
     v[k] = make_float2(0.0f, 0.0f);
 #pragma unroll 4
     for (int i = threadIdx.x; i < r.bpc; i += kSpecScalThreads) v[k] = ff_add(v[k], p[i]);
   }
-  __shared__ float2 red[3][kSpecScalThreads / 32];
+  __shared__ float2 red[4][kSpecScalThreads / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-  for (int k = 0; k < 3; ++k) {
+  for (int k = 0; k < 4; ++k) {
     v[k] = ff_warp_sum(v[k]);
     if (lane == 0) red[k][warp] = v[k];
   }
   __syncthreads();
   if (warp != 0) return;
 #pragma unroll
-  for (int k = 0; k < 3; ++k) v[k] = ff_warp_sum(lane < kSpecScalThreads / 32 ? red[k][lane] : make_float2(0.0f, 0.0f));
+  for (int k = 0; k < 4; ++k) v[k] = ff_warp_sum(lane < kSpecScalThreads / 32 ? red[k][lane] : make_float2(0.0f, 0.0f));
   if (lane != 0 || done != kRunning) return;
   const double den = nfac * ((double)v[0].x + v[0].y), aa = nfac * ((double)v[1].x + v[1].y),
-               rr = nfac * ((double)v[2].x + v[2].y);
+               ra = nfac * ((double)v[2].x + v[2].y), rr = nfac * ((double)v[3].x + v[3].y);
   s.xpend = 0;
   s.den = den;
-  if (!finite_d(den) || !finite_d(aa) || !finite_d(rr) || den <= 0.0) {
+  if (!finite_d(den) || !finite_d(aa) || !finite_d(ra) || !finite_d(rr) || den <= 0.0) {
     s.done = kBreakdown;
     return;
   }
-  // one float64 division and one square root: a float64 operation of one
-  // thread costs tens of cycles here, and every kernel of the next iteration
-  // waits for this one
-  const double inv = 1.0 / den, alpha = rr * inv;
+  const double alpha = rr / den;
   s.alpha = alpha;
   s.alpha_f = (float)alpha;
   s.xpend = 1;
-  // the sums carry float32 products: below 1e-8 of (r, r) the difference is rounding
-  const double beta = fmax(alpha * (aa * inv) - 1.0, 1e-8);
-  const double rr_new = beta * rr;
+  // below 1e-8 of (r, r) the expansion is the rounding of its float32 products
+  const double rr_new = fmax(rr + alpha * (alpha * aa - 2.0 * ra), 1e-8 * rr);
+  const double beta = rr > 0.0 ? rr_new / rr : 0.0;
   s.iter = iter + 1;
   s.beta_f = (float)beta;
   s.rr = rr_new;
