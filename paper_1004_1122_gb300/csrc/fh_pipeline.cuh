@@ -250,6 +250,7 @@ struct Pipeline {
   float2 *stw_row = nullptr, *stw_col = nullptr, *stw_mid = nullptr;
   Launch scol{}, smid{}, srow{};
   T* S2 = nullptr;             // 3-D: two-channel spectrum
+  float4* spart = nullptr;     // partial sums of the iteration
   SpecMedium* smed = nullptr;  // reference medium per cell
   int init_spectral(const Problem& pb, std::string& err);
   SpecArgs spec_args() const;

@@ -325,7 +325,7 @@ int Pipeline<T>::init(const Problem& pb, int nloads_, bool krylov, cudaStream_t 
   const int nred = std::max(std::max(items, ncell * d), 16);
   if ((rc = dev_alloc(allocs, &scal, nscal, err))) return rc;
   if ((rc = dev_alloc(allocs, &scal_aux, nscal, err))) return rc;
-  if ((rc = dev_alloc(allocs, &part, (size_t)4 * kMaxLoads * part_stride, err))) return rc;
+  if ((rc = dev_alloc(allocs, &part, (size_t)3 * kMaxLoads * part_stride, err))) return rc;
   if ((rc = dev_alloc(allocs, &d_red, nred, err))) return rc;
   const size_t scal_bytes = 2 * nscal * sizeof(Scal), red_bytes = nred * sizeof(double);
   FH_CKS(cudaMallocHost(&h_pinned, scal_bytes + red_bytes + 4 * sizeof(int)));
@@ -445,7 +445,7 @@ int Pipeline<T>::init_spectral(const Problem& pb, std::string& err) {
     sscol = seq_stride(spcol, stpc, Cc * 2 * nl, 2, [&](int ss) {
       return 2 * walk(scol.block, nl * Cc, 2, ss) + 2 * walk(scol.block, Cc / 2, 4 * nl, ss);
     });
-    scol.smem = spec_col_smem(sscol, Cc * 2 * nl, 3 * nl, scol.block);
+    scol.smem = spec_col_smem(sscol, Cc * 2 * nl, nl, scol.block);
     if (d == 3) {
       smid.block = round_up(std::max(64, Cc * 3 * nl * stpm), 32);
       smid.grid = sg.Tt * g.n[0];
@@ -513,7 +513,8 @@ int Pipeline<T>::init_spectral(const Problem& pb, std::string& err) {
       if ((rc = dev_alloc(allocs, &smed, ncell, err))) return rc;
       FH_CKS(cudaMemcpy(smed, hm.data(), ncell * sizeof(SpecMedium), cudaMemcpyHostToDevice));
     }
-    if (more_part && (rc = dev_alloc(allocs, &part, (size_t)4 * kMaxLoads * part_stride, err))) return rc;
+    if (more_part && (rc = dev_alloc(allocs, &part, (size_t)3 * kMaxLoads * part_stride, err))) return rc;
+    if ((rc = dev_alloc(allocs, &spart, (size_t)4 * kMaxLoads * scol.grid, err))) return rc;
     spec_ops = true;
     if (!want_spectral) return 0;
     if (2 * lines > (size_t)vlen)  // padded scalar arrays do not fit the field buffers
@@ -550,7 +551,7 @@ SpecArgs Pipeline<T>::spec_args() const {
   a.scal = scal;
   a.nl = nloads;
   a.three = g.d == 3;
-  a.part = reinterpret_cast<float2*>(part);
+  a.part = spart;
   a.med = smed;
   return a;
 }
@@ -620,7 +621,7 @@ cudaError_t Pipeline<T>::spec_iter() {
   FH_CK(spec_passes());
   ++launches;
   seq_launch(k_scal_spec, chain_launch(item_blocks(items), kSpecScalThreads), 0, st, scal,
-             reinterpret_cast<const float2*>(part), scol.grid, ncell, nloads, (double)g.cell_nodes);
+             spart, scol.grid, ncell, nloads, (double)g.cell_nodes);
   return cudaGetLastError();
 }
 

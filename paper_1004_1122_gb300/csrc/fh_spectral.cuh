@@ -82,39 +82,73 @@ struct SpecArgs {
   float2* ap[kMaxLoads];
   float2* x[kMaxLoads];
   Scal* scal;
-  // partial sums as two-float values, one per CTA: (p, A p) rows 0..,
-  // (A p, A p) rows kMaxLoads.., (r, A p) rows 2 kMaxLoads.., (r, r) rows 3 kMaxLoads..
-  float2* part;
+  // partial sums (Sum3), one per CTA: (p, A p) rows 0.., (A p, A p) rows kMaxLoads..,
+  // (r, A p) rows 2 kMaxLoads.., (r, r) rows 3 kMaxLoads..
+  float4* part;
   const SpecMedium* med;       // per cell
 };
 
 // ----------------------------------------------------------------------------
-// two-float sums (value s + c): exact to ~2^-48 of the sum of |terms|
+// sums over a CTA
 // ----------------------------------------------------------------------------
-__device__ __forceinline__ float2 ff_add(float2 a, float2 b) {
-  const float s = __fadd_rn(a.x, b.x);
-  const float bb = __fsub_rn(s, a.x);
-  const float e = __fadd_rn(__fsub_rn(a.x, __fsub_rn(s, bb)), __fsub_rn(b.x, bb));
-  return make_float2(s, __fadd_rn(__fadd_rn(a.y, b.y), e));
+// a + b = s + e exactly
+__device__ __forceinline__ float two_sum(float a, float b, float& e) {
+  const float s = __fadd_rn(a, b);
+  const float bb = __fsub_rn(s, a);
+  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+  return s;
 }
-__device__ __forceinline__ float2 ff_warp_sum(float2 v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1)
-    v = ff_add(v, make_float2(__shfl_down_sync(0xffffffffu, v.x, o), __shfl_down_sync(0xffffffffu, v.y, o)));
-  return v;
-}
-__device__ __forceinline__ float2 ff_of(const DotAcc<float>& d, float w) { return make_float2(w * d.s, -w * d.c); }
+// Sum held in three float32 parts s + c + r (the K-fold compensated summation
+// of Ogita, Rump and Oishi with K = 3): more bits than float64, on the float32
+// units.  A float64 instruction holds an SM's unit for 16 cycles per warp, and a
+// tree of them at the end of every kernel is a chain that the next kernel waits
+// for.
+struct Sum3 {
+  float s, c, r;
+  __device__ __forceinline__ void low(float v) {
+    float e;
+    c = two_sum(c, v, e);
+    r = __fadd_rn(r, e);
+  }
+  __device__ __forceinline__ void add(float vs, float vc, float vr) {
+    float e;
+    s = two_sum(s, vs, e);
+    low(e);
+    low(vc);
+    r = __fadd_rn(r, vr);
+  }
+  // over groups of `width` lanes
+  __device__ __forceinline__ void warp_sum(int width = 32) {
+    for (int o = width >> 1; o > 0; o >>= 1)
+      add(__shfl_down_sync(0xffffffffu, s, o), __shfl_down_sync(0xffffffffu, c, o), __shfl_down_sync(0xffffffffu, r, o));
+  }
+  __device__ __forceinline__ double get() const { return (double)s + ((double)c + (double)r); }
+};
+__device__ __forceinline__ float2 dot_parts(const DotAcc<float>& d) { return make_float2(d.s, -d.c); }
 
-// Sums of `rows` rows of blockDim values in shared memory, one warp per row;
-// row k goes to out[map(k)].  Call after a barrier behind the writes.
-template <typename F>
-__device__ __forceinline__ void ff_rows_store(const float2* red, int rows, F&& out) {
-  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  for (int k = threadIdx.x >> 5; k < rows; k += nw) {
-    float2 v = make_float2(0.0f, 0.0f);
-    for (int i = lane; i < (int)blockDim.x; i += 32) v = ff_add(v, red[k * blockDim.x + i]);
-    v = ff_warp_sum(v);
-    if (lane == 0) out(k, v);
+// Sums of `rows` rows of `count` values (a thread's two parts each) in shared
+// memory, row k at src(k)[at(i)]; its sum goes to *out(k).  Call after a barrier behind the
+// writes.  A row is summed by 32 lanes, or by 8 where a kernel carries several
+// loads: there the CTAs are small and many, and the trees' instructions count
+// more than the length of the chain (243^3, three loads: 644 -> 610 ms per tensor
+// with that and the sums kept in the tile instead of behind it).
+template <typename S, typename A, typename F>
+__device__ __forceinline__ void rows_store(int rows, int count, int nl, S&& src, A&& at, F&& out) {
+  const int width = nl > 1 ? 8 : 32, per = 32 / width;  // lanes per row, rows per warp
+  const int lane = threadIdx.x & 31, sub = lane & (width - 1), nw = blockDim.x >> 5;
+  for (int k0 = (threadIdx.x >> 5) * per; k0 < rows; k0 += nw * per) {
+    const int k = k0 + lane / width;
+    Sum3 t{0.0f, 0.0f, 0.0f};
+    if (k < rows) {
+      const float2* const row = src(k);
+#pragma unroll 4
+      for (int i = sub; i < count; i += width) {
+        const float2 v = row[at(i)];
+        t.add(v.x, v.y, 0.0f);
+      }
+    }
+    t.warp_sum(width);
+    if (sub == 0 && k < rows) *out(k) = make_float4(t.s, t.c, t.r, 0.0f);
   }
 }
 
@@ -270,7 +304,7 @@ __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_inv(SpecArgs a
     const float4* const ap = reinterpret_cast<const float4*>(a.ap[l] + tl.sbase + e);
     float2* const ch = sm + (size_t)(e * nl + l) * 2 * a.ss;
     const int next = 2 * nl * a.ss;  // the second frequency's columns
-    DotAcc<float> dot[2];
+    DotAcc<float> dot;
     for (int i0 = row0; i0 < n; i0 += kUnroll * drow) {
       float4 vr[kUnroll], vp[kUnroll], va[kUnroll], vx[kUnroll];
 #pragma unroll
@@ -309,8 +343,8 @@ __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_inv(SpecArgs a
             p[k] = v;
             __stcs(x + k, vx[u]);
           }
-          dot[0].add(vr[u].x * vr[u].x + vr[u].y * vr[u].y);
-          dot[1].add(vr[u].z * vr[u].z + vr[u].w * vr[u].w);
+          dot.add(fq[0].wgt * (vr[u].x * vr[u].x + vr[u].y * vr[u].y));
+          dot.add(fq[1].wgt * (vr[u].z * vr[u].z + vr[u].w * vr[u].w));
         }
         const float x0 = fq[0].xi0(i);
         const float s0 = fq[0].rnorm(i, x0), s1 = fq[1].rnorm(i, x0);
@@ -322,7 +356,7 @@ __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_inv(SpecArgs a
       }
     }
     if (MODE == kSpecUpdate)
-      red[l * blockDim.x + threadIdx.x] = ff_add(ff_of(dot[0], fq[0].wgt), ff_of(dot[1], fq[1].wgt));
+      red[l * blockDim.x + threadIdx.x] = dot_parts(dot);
   }
   __syncthreads();
   spec_col_fft<true, PS>(sm, a.ss, n, Q, a.plan, a.tpc, a.tw);
@@ -334,7 +368,9 @@ __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_inv(SpecArgs a
     S[w.i * rs + w.j] = make_float4(v0.x, v0.y, v1.x, v1.y);
   }
   if (MODE == kSpecUpdate)
-    ff_rows_store(red, nl, [&](int k, float2 v) { a.part[(size_t)(3 * kMaxLoads + k) * gridDim.x + tl.slot] = v; });
+    rows_store(
+        nl, blockDim.x, nl, [&](int k) { return red + k * blockDim.x; }, [](int i) { return i; },
+        [&](int k) { return a.part + (size_t)(3 * kMaxLoads + k) * gridDim.x + tl.slot; });
 }
 
 // kSpecApply: A p of the direction's tau spectrum, with (p, A p), (A p, A p) and (r, A p).
@@ -346,7 +382,6 @@ __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_fwd(SpecArgs a
   float2* sm = reinterpret_cast<float2*>(smem_raw);
   const int n = plan_len<PS>(a.plan), C = a.sg.C, csh = a.sg.csh, nl = a.nl;
   const int Q = 2 * nl * C;
-  float2* const red = sm + (size_t)a.ss * Q;
   const SpecTile tl = spec_tile(a, n);
   Scal* const sc = a.scal + tl.cell * nl;
   if (MODE == kSpecApply && all_done(sc, nl)) return;
@@ -380,7 +415,7 @@ __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_fwd(SpecArgs a
   fq[0].init(a, a.med[tl.cell], n, tl.t * C + e, tl.inner);
   fq[1].init(a, a.med[tl.cell], n, tl.t * C + e + 1, tl.inner);
   for (int l = 0; l < nl; ++l) {
-    DotAcc<float> d1[2], d2[2], d3[2];
+    DotAcc<float> d1, d2, d3;
     if (MODE == kSpecProject || sc[l].done == kRunning) {
       const float4* const p = reinterpret_cast<const float4*>(a.p[l] + tl.sbase + e);
       const float4* const r = reinterpret_cast<const float4*>(a.r[l] + tl.sbase + e);
@@ -414,26 +449,34 @@ __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_fwd(SpecArgs a
               const float2 rv = h ? make_float2(vr[u].z, vr[u].w) : make_float2(vr[u].x, vr[u].y);
               y[h].x += q.x;
               y[h].y += q.y;
-              d3[h].add(rv.x * y[h].x + rv.y * y[h].y);
-              d1[h].add(q.x * y[h].x + q.y * y[h].y);
-              d2[h].add(y[h].x * y[h].x + y[h].y * y[h].y);
+              d1.add(fq[h].wgt * (q.x * y[h].x + q.y * y[h].y));
+              d2.add(fq[h].wgt * (y[h].x * y[h].x + y[h].y * y[h].y));
+              d3.add(fq[h].wgt * (rv.x * y[h].x + rv.y * y[h].y));
             }
           }
           out[i << (csh - 1)] = make_float4(y[0].x, y[0].y, y[1].x, y[1].y);
         }
       }
     }
-    if (MODE == kSpecApply) {
-      red[l * blockDim.x + threadIdx.x] = ff_add(ff_of(d1[0], fq[0].wgt), ff_of(d1[1], fq[1].wgt));
-      red[(nl + l) * blockDim.x + threadIdx.x] = ff_add(ff_of(d2[0], fq[0].wgt), ff_of(d2[1], fq[1].wgt));
-      red[(2 * nl + l) * blockDim.x + threadIdx.x] = ff_add(ff_of(d3[0], fq[0].wgt), ff_of(d3[1], fq[1].wgt));
+    // the sums take the place of the thread's first row, which only it has read
+    if (MODE == kSpecApply && row0 < n) {
+      float2* const own = sm + (size_t)(e * nl + l) * 2 * a.ss + row0;
+      own[0] = dot_parts(d1);
+      own[a.ss] = dot_parts(d2);
+      own[2 * nl * a.ss] = dot_parts(d3);
     }
   }
   if (MODE == kSpecApply) {
     __syncthreads();
-    ff_rows_store(red, 3 * nl, [&](int k, float2 v) {
-      a.part[(size_t)(k / nl * kMaxLoads + k % nl) * gridDim.x + tl.slot] = v;
-    });
+    const int half = csh - 1, count = n << half < (int)blockDim.x ? n << half : (int)blockDim.x;
+    rows_store(
+        3 * nl, count, nl,
+        [&](int k) {
+          const int kind = k / nl;
+          return sm + (k - kind * nl) * 2 * a.ss + (kind == 2 ? 2 * nl : kind) * a.ss;
+        },
+        [&](int i) { return 4 * nl * a.ss * (i & ((1 << half) - 1)) + (i >> half); },
+        [&](int k) { return a.part + (size_t)(k / nl * kMaxLoads + k % nl) * gridDim.x + tl.slot; });
   }
 }
 
@@ -916,7 +959,7 @@ __global__ void __launch_bounds__(SpecRowBounds<PS>::threads, SpecRowBounds<PS>:
 // ((v, w) = nfac sum_k conj(psi_v) psi_w).  A step's x update is applied by
 // the next spec_inv, so a stopping item leaves it owed (xpend).
 constexpr int kSpecScalThreads = 512;
-static __global__ void __launch_bounds__(kSpecScalThreads) k_scal_spec(Scal* scal, const float2* part, int np, int ncell,
+static __global__ void __launch_bounds__(kSpecScalThreads) k_scal_spec(Scal* scal, const float4* part, int np, int ncell,
                                                                        int nl, double nfac) {
   seq_begin();
   const ItemRef r = item_ref(np, ncell, nl);
@@ -925,41 +968,47 @@ static __global__ void __launch_bounds__(kSpecScalThreads) k_scal_spec(Scal* sca
   // what thread 0 needs afterwards is loaded together with the partial sums
   const int done = s.done, iter = s.iter, max_iter = s.max_iter;
   const double b2 = s.b2, tol2 = s.tol2, ib2 = s.ib2;
-  float2 v[4];
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const float2* const p = part + (long long)(k * kMaxLoads + r.l) * np + (long long)r.cell * r.bpc;
-    v[k] = make_float2(0.0f, 0.0f);
+  // warp w sums a share of row w % 4
+  constexpr int kRows = 4, kShares = kSpecScalThreads / 32 / kRows;
+  __shared__ Sum3 red[kRows][kShares];
+  __shared__ double tot[kRows], inv[kRows];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, row = warp % kRows, share = warp / kRows;
+  Sum3 v{0.0f, 0.0f, 0.0f};
+  {
+    const float4* const p = part + (long long)(row * kMaxLoads + r.l) * np + (long long)r.cell * r.bpc;
 #pragma unroll 4
-    for (int i = threadIdx.x; i < r.bpc; i += kSpecScalThreads) v[k] = ff_add(v[k], p[i]);
+    for (int i = share * 32 + lane; i < r.bpc; i += kShares * 32) {
+      const float4 q = p[i];
+      v.add(q.x, q.y, q.z);
+    }
   }
-  __shared__ float2 red[4][kSpecScalThreads / 32];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    v[k] = ff_warp_sum(v[k]);
-    if (lane == 0) red[k][warp] = v[k];
+  v.warp_sum();
+  if (lane == 0) red[row][share] = v;
+  __syncthreads();
+  // each row's float64 value and reciprocal in a warp of its own: a float64
+  // operation of one thread costs tens of cycles here, and every kernel of the
+  // next iteration waits for this one
+  if (warp < kRows && lane == 0) {
+    for (int q = 1; q < kShares; ++q) v.add(red[warp][q].s, red[warp][q].c, red[warp][q].r);
+    tot[warp] = nfac * v.get();
+    inv[warp] = 1.0 / tot[warp];
   }
   __syncthreads();
-  if (warp != 0) return;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) v[k] = ff_warp_sum(lane < kSpecScalThreads / 32 ? red[k][lane] : make_float2(0.0f, 0.0f));
-  if (lane != 0 || done != kRunning) return;
-  const double den = nfac * ((double)v[0].x + v[0].y), aa = nfac * ((double)v[1].x + v[1].y),
-               ra = nfac * ((double)v[2].x + v[2].y), rr = nfac * ((double)v[3].x + v[3].y);
+  if (threadIdx.x != 0 || done != kRunning) return;
+  const double den = tot[0], aa = tot[1], ra = tot[2], rr = tot[3];
   s.xpend = 0;
   s.den = den;
   if (!finite_d(den) || !finite_d(aa) || !finite_d(ra) || !finite_d(rr) || den <= 0.0) {
     s.done = kBreakdown;
     return;
   }
-  const double alpha = rr / den;
+  const double alpha = rr * inv[0];
   s.alpha = alpha;
   s.alpha_f = (float)alpha;
   s.xpend = 1;
   // below 1e-8 of (r, r) the expansion is the rounding of its float32 products
   const double rr_new = fmax(rr + alpha * (alpha * aa - 2.0 * ra), 1e-8 * rr);
-  const double beta = rr > 0.0 ? rr_new / rr : 0.0;
+  const double beta = rr > 0.0 ? rr_new * inv[3] : 0.0;
   s.iter = iter + 1;
   s.beta_f = (float)beta;
   s.rr = rr_new;
