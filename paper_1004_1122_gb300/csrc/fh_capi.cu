@@ -248,10 +248,6 @@ int init_tuned(Pipeline<T>* P, const Problem& pb, bool krylov, cudaStream_t st, 
 // float64 outer residual then decides whether another refinement step helps.
 constexpr int kInnerStallWindow = 100;
 
-// Relative residual at which the first float32 solve of a refined solve hands
-// over to the float64 outer residual.
-constexpr double kFirstEta = 1e-3;
-
 bool l0_isotropic(const Problem& pb, double& l0) {
   const int d = pb.d;
   l0 = pb.L0[0];
@@ -683,15 +679,16 @@ fh_status fh_solve(fh_ctx* c, const double* E, double tol, int method, int max_i
     SolveResult res;
     double last_alpha = 0.0;
     bool done_first = false;
+    const double first = P->first_eta(method);
     if (!e_init) {
       // From e = E the first correction solves A d = -B E, whose complement
       // part is zero (B maps into the compatible fields): that is the float32
       // solve of A x = E from x = E itself, with no float64 residual before it.
-      // It stops at kFirstEta (or 0.3 tol if that is looser): float32 CG
+      // It stops at first_eta (or 0.3 tol if that is looser): float32 CG
       // tracks float64 CG closely that far, and restarting from the float64
       // residual there took fewer iterations in total than pushing float32 to
       // its limit first (2187^2, contrast 1e4: 395 instead of 446).
-      double eta = std::max(0.3 * tol, kFirstEta);
+      double eta = std::max(0.3 * tol, first);
       if (eta > 0.1) eta = 0.1;
       rc = P->solve(method, Ev, false, fh::kX0Const, nullptr, eta, max_iter, &res, err, nullptr,
                     kInnerStallWindow);
@@ -729,8 +726,8 @@ fh_status fh_solve(fh_ctx* c, const double* E, double tol, int method, int max_i
       // the target, never below what float32 can resolve
       double eta = 0.3 * tol / rel_true;
       // a first step from a given initial field far from the solution hands
-      // over at kFirstEta |E| too, as the direct first step from e = E does
-      if (outer == 0 && rel_true > 10.0 * kFirstEta) eta = std::max(eta, kFirstEta / rel_true);
+      // over at first_eta |E| too, as the direct first step from e = E does
+      if (outer == 0 && rel_true > 10.0 * first) eta = std::max(eta, first / rel_true);
       if (eta < 2e-6) eta = 2e-6;
       if (eta > 0.1) eta = 0.1;
       ++c->own_launches;

@@ -252,6 +252,19 @@ struct Pipeline {
   T* S2 = nullptr;             // 3-D: two-channel spectrum
   float4* spart = nullptr;     // partial sums of the iteration
   SpecMedium* smed = nullptr;  // reference medium per cell
+  // Relative residual at which the first refinement step hands over to the
+  // float64 residual.  A restart there takes fewer iterations than pushing
+  // float32 to its limit.  The distance between the float32 solution and the
+  // recursive residual, which the next step starts and ends with, is
+  // proportional to it; in the frequency domain it is twice that of the
+  // iteration on fields (the correction's large low-frequency coefficients
+  // round in every step, where a field's values round at their own size: 8.1e-6
+  // against 4.4e-6 of the starting residual in a float32 model of 147x189 at
+  // contrast 267), so these solves hand over at half the residual.
+  // Error of the field against float64, 39 drawn refined solves, geometric
+  // mean over that of the iteration on fields: 1.02 at 1e-3, 0.75 at 5e-4, 0.76 at
+  // 3e-4, with 10356, 10168 and 10078 iterations in total.
+  double first_eta(int method) const { return spectral && method == kCG ? 5e-4 : 1e-3; }
   int init_spectral(const Problem& pb, std::string& err);
   SpecArgs spec_args() const;
   SpecRowArgs spec_row_args() const;

@@ -213,10 +213,19 @@ struct SpecFreq {
   __device__ __forceinline__ float rnorm(int i, float x0) const {
     return dead || i == nyq || (i == 0 && zero0) ? 0.0f : rsqrtf(x0 * x0 + q1);
   }
-  // |xi| / (xi . L0 . xi) / |N| from rn = 1 / |xi|
+  // 1 / (|xi|^2 rn), which takes xi . v back to psi where v = xi rn psi: the two
+  // maps are inverse to each other to float32 rounding whatever the error of
+  // rn is (rsqrtf's, squared, would be an error of the operator).  One Newton
+  // step from rn; its defect |xi|^2 rn^2 - 1 is formed exactly.
+  __device__ __forceinline__ float inverse(float x0, float rn) const {
+    const float q = x0 * x0 + q1, t = q * rn;
+    const float e = fmaf(t, rn, -1.0f) + fmaf(q, rn, -t) * rn;
+    return rn == 0.0f ? 0.0f : fmaf(-rn, e, rn);
+  }
+  // 1 / (xi . L0 . xi rn) / |N|: the projection's factor
   __device__ __forceinline__ float project(float x0, float rn) const {
-    if (iso) return rn * scale;
-    return rn == 0.0f ? 0.0f : scale * (x0 * x0 + q1) * rn / (x0 * (L00 * x0 + L01) + L11);
+    if (iso) return inverse(x0, rn) * scale;
+    return rn == 0.0f ? 0.0f : scale / ((x0 * (L00 * x0 + L01) + L11) * rn);
   }
 };
 
@@ -441,7 +450,7 @@ __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_fwd(SpecArgs a
           for (int h = 0; h < 2; ++h) {
             const float2 v0 = ch[h * next + i], v1 = ch[h * next + a.ss + i];
             const float rn = fq[h].rnorm(i, x0);
-            const float w = MODE == kSpecApply ? fq[h].project(x0, rn) : rn * a.sg.inv_nodes;
+            const float w = MODE == kSpecApply ? fq[h].project(x0, rn) : fq[h].inverse(x0, rn) * a.sg.inv_nodes;
             const float w0 = x0 * w, w1 = fq[h].c1 * w;
             y[h] = make_float2(w0 * v0.x + w1 * v1.x, w0 * v0.y + w1 * v1.y);
             if (MODE == kSpecApply) {
