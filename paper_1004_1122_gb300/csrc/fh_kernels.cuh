@@ -141,6 +141,7 @@ struct Scal {
   int xpend;
   // frequency-domain CG (fh_spectral.cuh): alpha and beta as its kernels use them
   float alpha_f, beta_f;
+  float psi_f, psi_b;  // powers of two: scalars = psi_f * those of the fields, and back
   double ib2;      // 1 / b2
 };
 
@@ -1550,6 +1551,9 @@ static __global__ void k_scal_start(Scal* scal, const double* part, int np, int 
     s.rel_true = s.rel;
     s.best_rel = s.rel;
     s.best_iter = 0;
+    const int h = rr > 0.0 && finite_d(rr) ? max(-120, min(120, ilogb(rr) / 2)) : 0;
+    s.psi_f = ldexpf(1.0f, -h);
+    s.psi_b = ldexpf(1.0f, h);
     record_hist(s);
     if (!finite_d(rr)) s.done = kBreakdown;
     else if (rr <= s.tol2 * s.b2) s.done = kConverged;

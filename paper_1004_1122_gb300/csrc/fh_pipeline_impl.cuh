@@ -652,8 +652,12 @@ cudaError_t Pipeline<T>::spec_finish() {
 
 template <typename T>
 int Pipeline<T>::spec_dir_norm2(const double* Mx, double* out, std::string& err) {
+  // the kernel's float32 squares see M with entries up to 1
+  double top = 0.0;
+  for (int i = 0; i < 9; ++i) top = std::max(top, std::fabs(Mx[i]));
+  const int e = top > 0.0 ? std::ilogb(top) : 0;
   Mat3 m;
-  for (int i = 0; i < 9; ++i) m.v[i] = Mx[i];
+  for (int i = 0; i < 9; ++i) m.v[i] = std::ldexp(Mx[i], -e);
   ++launches;
   k_spec_matnorm2<<<scol.grid, 256, 0, st>>>(spec_args(), m, part);
   FH_CKS(cudaGetLastError());
@@ -662,7 +666,8 @@ int Pipeline<T>::spec_dir_norm2(const double* Mx, double* out, std::string& err)
   FH_CKS(cudaGetLastError());
   FH_CKS(cudaMemcpyAsync(h_red, d_red, sizeof(double), cudaMemcpyDeviceToHost, st));
   FH_CKS(cudaStreamSynchronize(st));
-  *out = h_red[0] * (double)g.nodes;
+  const double back = std::ldexp((double)h_scal[0].psi_b, e);
+  *out = h_red[0] * (double)g.nodes * back * back;
   return 0;
 }
 

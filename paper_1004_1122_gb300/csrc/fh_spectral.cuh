@@ -29,6 +29,10 @@
 // model of the iteration), where (p, A p) in place of (r, A p), its value for a
 // symmetric A in exact arithmetic, is 1e-6 off.
 //
+// The scalars of a solve are those of its fields times a power of two that
+// brings the initial residual's norm to about 1 (psi_f, exact): psi is 1 / sqrt|N|
+// of a field, and its squares would leave float32's range for loads of 1e-11.
+//
 // Memory moved per iteration in units of one real scalar per node: 19.25 in
 // 2-D (113 / 4 = 28.25 with the fields' passes), 32.25 in 3-D (59.25).
 // Measured per iteration, against the passes on fields: 2187^2 168 -> 127 us
@@ -307,6 +311,7 @@ __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_inv(SpecArgs a
     const float al = MODE == kSpecUpdate || s.xpend ? s.alpha_f : 0.0f;
     const float be = s.beta_f;
     const bool live = MODE == kSpecUpdate ? s.done == kRunning : !fresh;
+    const float back = s.psi_b;  // kSpecFinish: to the fields' scale
     float4* const r = reinterpret_cast<float4*>(a.r[l] + tl.sbase + e);
     float4* const p = reinterpret_cast<float4*>(a.p[l] + tl.sbase + e);
     float4* const x = reinterpret_cast<float4*>(a.x[l] + tl.sbase + e);
@@ -342,7 +347,7 @@ __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_inv(SpecArgs a
           y.w += c * z.w;
         };
         axpy(vx[u], al, vp[u]);
-        float4 v = vx[u];
+        float4 v = make_float4(back * vx[u].x, back * vx[u].y, back * vx[u].z, back * vx[u].w);
         if (MODE == kSpecUpdate) {
           axpy(vr[u], -al, va[u]);
           v = vr[u];
@@ -424,6 +429,7 @@ __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_fwd(SpecArgs a
   fq[0].init(a, a.med[tl.cell], n, tl.t * C + e, tl.inner);
   fq[1].init(a, a.med[tl.cell], n, tl.t * C + e + 1, tl.inner);
   for (int l = 0; l < nl; ++l) {
+    const float toscale = a.sg.inv_nodes * sc[l].psi_f;  // kSpecProject
     DotAcc<float> d1, d2, d3;
     if (MODE == kSpecProject || sc[l].done == kRunning) {
       const float4* const p = reinterpret_cast<const float4*>(a.p[l] + tl.sbase + e);
@@ -450,7 +456,7 @@ __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_fwd(SpecArgs a
           for (int h = 0; h < 2; ++h) {
             const float2 v0 = ch[h * next + i], v1 = ch[h * next + a.ss + i];
             const float rn = fq[h].rnorm(i, x0);
-            const float w = MODE == kSpecApply ? fq[h].project(x0, rn) : fq[h].inverse(x0, rn) * a.sg.inv_nodes;
+            const float w = MODE == kSpecApply ? fq[h].project(x0, rn) : fq[h].inverse(x0, rn) * toscale;
             const float w0 = x0 * w, w1 = fq[h].c1 * w;
             y[h] = make_float2(w0 * v0.x + w1 * v1.x, w0 * v0.y + w1 * v1.y);
             if (MODE == kSpecApply) {
@@ -965,7 +971,7 @@ __global__ void __launch_bounds__(SpecRowBounds<PS>::threads, SpecRowBounds<PS>:
 }
 
 // alpha, beta and the stopping tests of one iteration; nfac = nodes per cell
-// ((v, w) = nfac sum_k conj(psi_v) psi_w).  A step's x update is applied by
+// ((v, w) = nfac psi_b^2 sum_k conj(psi_v) psi_w).  A step's x update is applied by
 // the next spec_inv, so a stopping item leaves it owed (xpend).
 constexpr int kSpecScalThreads = 512;
 static __global__ void __launch_bounds__(kSpecScalThreads) k_scal_spec(Scal* scal, const float4* part, int np, int ncell,
@@ -976,7 +982,7 @@ static __global__ void __launch_bounds__(kSpecScalThreads) k_scal_spec(Scal* sca
   Scal& s = scal[r.item];
   // what thread 0 needs afterwards is loaded together with the partial sums
   const int done = s.done, iter = s.iter, max_iter = s.max_iter;
-  const double b2 = s.b2, tol2 = s.tol2, ib2 = s.ib2;
+  const double b2 = s.b2, tol2 = s.tol2, ib2 = s.ib2, back = s.psi_b;
   // warp w sums a share of row w % 4
   constexpr int kRows = 4, kShares = kSpecScalThreads / 32 / kRows;
   __shared__ Sum3 red[kRows][kShares];
@@ -999,7 +1005,7 @@ static __global__ void __launch_bounds__(kSpecScalThreads) k_scal_spec(Scal* sca
   // next iteration waits for this one
   if (warp < kRows && lane == 0) {
     for (int q = 1; q < kShares; ++q) v.add(red[warp][q].s, red[warp][q].c, red[warp][q].r);
-    tot[warp] = nfac * v.get();
+    tot[warp] = nfac * back * back * v.get();
     inv[warp] = 1.0 / tot[warp];
   }
   __syncthreads();
@@ -1030,7 +1036,7 @@ static __global__ void __launch_bounds__(kSpecScalThreads) k_scal_spec(Scal* sca
 }
 
 // Partial sums of |M u psi|^2 over the full spectrum (single-cell, one load):
-// |N| times their sum is |M v|^2 of the field v.
+// |N| psi_b^2 times their sum is |M v|^2 of the field v.
 static __global__ void k_spec_matnorm2(SpecArgs a, Mat3 m, double* part) {
   const int n = a.plan.n, C = a.sg.C, csh = a.sg.csh;
   const SpecTile tl = spec_tile(a, n);
