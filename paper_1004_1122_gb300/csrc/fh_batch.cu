@@ -593,6 +593,11 @@ int solve_all_loads(const Problem& pb, int precision, double tol, int method, in
       g->p64 = new (std::nothrow) Pipeline<double>();
       rc = g->p64 ? g->p64->init(pb, d, precision == FH_FP64, g->st, err) : FH_ERR_OOM;
     }
+    // before the float32 pipeline, whose optional buffers take what is left
+    for (int l = 0; l < d && !rc; ++l)
+      if (cudaMalloc(&g->x64[l], (size_t)d * pb.nodes * sizeof(double)) != cudaSuccess ||
+          cudaMalloc(&g->r64[l], (size_t)d * pb.nodes * sizeof(double)) != cudaSuccess)
+        rc = FH_ERR_OOM;
     if (!rc && precision != FH_FP64) {
       g->p32 = new (std::nothrow) Pipeline<float>();
       if (!g->p32) {
@@ -613,10 +618,6 @@ int solve_all_loads(const Problem& pb, int precision, double tol, int method, in
         if (rc) rc = g->p32->init(pb, d, true, g->st, err);
       }
     }
-    for (int l = 0; l < d && !rc; ++l)
-      if (cudaMalloc(&g->x64[l], (size_t)d * pb.nodes * sizeof(double)) != cudaSuccess ||
-          cudaMalloc(&g->r64[l], (size_t)d * pb.nodes * sizeof(double)) != cudaSuccess)
-        rc = FH_ERR_OOM;
     if (rc) {
       release_loads_group(g);
       return rc;

@@ -421,15 +421,16 @@ fh_status fh_create(fh_ctx** out, int d, const int* N, const double* Y, const ui
     if (!c->p64) rc = FH_ERR_OOM;
     if (!rc) rc = init_tuned(c->p64, pb, precision == FH_FP64, c->st, err);
   }
+  // before the float32 pipeline, whose optional buffers take what is left
+  const size_t vbytes = (size_t)d * pb.nodes * sizeof(double);
+  if (!rc && cudaMalloc(&c->d_x64, vbytes) != cudaSuccess) rc = FH_ERR_OOM;
+  if (!rc && cudaMalloc(&c->d_r64, vbytes) != cudaSuccess) rc = FH_ERR_OOM;
   if (!rc && (precision == FH_FP32 || precision == FH_FP32_REFINED)) {
     c->p32 = new (std::nothrow) Pipeline<float>();
     if (!c->p32) rc = FH_ERR_OOM;
     else c->p32->want_spectral = precision == FH_FP32_REFINED;
     if (!rc) rc = init_tuned(c->p32, pb, true, c->st, err);
   }
-  const size_t vbytes = (size_t)d * pb.nodes * sizeof(double);
-  if (!rc && cudaMalloc(&c->d_x64, vbytes) != cudaSuccess) rc = FH_ERR_OOM;
-  if (!rc && cudaMalloc(&c->d_r64, vbytes) != cudaSuccess) rc = FH_ERR_OOM;
   if (rc) {
     fh_destroy(c);
     return (fh_status)rc;

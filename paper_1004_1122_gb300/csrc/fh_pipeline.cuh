@@ -90,6 +90,21 @@ struct DevPool {
   char* cur = nullptr;
   size_t left = 0;
   void push_back(void* p) { blocks.push_back(p); }
+  // what was allocated behind a mark goes back
+  struct Mark {
+    size_t count;
+    char* cur;
+    size_t left;
+  };
+  Mark mark() const { return {blocks.size(), cur, left}; }
+  void rollback(const Mark& m) {
+    while (blocks.size() > m.count) {
+      cudaFree(blocks.back());
+      blocks.pop_back();
+    }
+    cur = m.cur;
+    left = m.left;
+  }
   void release() {
     for (void* p : blocks) cudaFree(p);
     blocks.clear();

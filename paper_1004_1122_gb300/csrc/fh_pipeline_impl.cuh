@@ -360,7 +360,39 @@ int Pipeline<T>::init(const Problem& pb, int nloads_, bool krylov, cudaStream_t 
         v += len;
       }
   }
-  return krylov ? init_spectral(pb, err) : 0;
+  if (!krylov) return 0;
+  // Without the memory for the buffers of the frequency-layout passes (3-D: a
+  // spectrum of 8 bytes per node and load; padded scalar arrays) the passes on
+  // fields, which need none of them, do the work.
+  const DevPool::Mark m = allocs.mark();
+  struct {
+    C* S;
+    double* part;
+    T *r[kMaxLoads], *p[kMaxLoads], *ap[kMaxLoads], *p2[kMaxLoads];
+  } fields;
+  fields.S = S;
+  fields.part = part;
+  for (int l = 0; l < kMaxLoads; ++l) {
+    fields.r[l] = r[l];
+    fields.p[l] = p[l];
+    fields.ap[l] = ap[l];
+    fields.p2[l] = p2[l];
+  }
+  rc = init_spectral(pb, err);
+  if (rc != 4) return rc;  // 4: FH_ERR_OOM
+  cudaGetLastError();
+  allocs.rollback(m);
+  S = fields.S;
+  S2 = nullptr;
+  part = fields.part;
+  for (int l = 0; l < kMaxLoads; ++l) {
+    r[l] = fields.r[l];
+    p[l] = fields.p[l];
+    ap[l] = fields.ap[l];
+    p2[l] = fields.p2[l];
+  }
+  spec_ops = spectral = false;
+  return 0;
 }
 
 // A plan's stage twiddles (fh_fft.cuh) on the device.
