@@ -23,7 +23,7 @@ e2e    = the same through the public API with host buffers: every step copies
          the phase image from pinned host memory and reads every solved field
          (float64) back into pinned host memory.
 Also reported: the matvec (operator application) throughput and its HBM
-bandwidth, the roofline of the dominant kernel, the plain float64 CG on cuFFT
+bandwidth, the roofline of one CG iteration, the plain float64 CG on cuFFT
 (torch.fft) as the comparison baseline, and the CPU oracle timed on the host.
 
 --impl reference times the CPU oracle (the reference arm of this repository).
@@ -62,7 +62,9 @@ def parse():
     ap.add_argument("--impl", default="fh", choices=["fh", "reference"])
     ap.add_argument("--no-baseline", action="store_true", help="skip the cuFFT float64 CG baseline")
     ap.add_argument("--no-cpu", action="store_true", help="skip the CPU oracle baseline")
-    ap.add_argument("--no-tune", action="store_true", help="skip the launch-shape autotuner")
+    ap.add_argument("--no-tune", action="store_true",
+                    help="accepted, no effect: the autotuner shapes the passes on fields, which these workloads' "
+                         "CG iterations do not run")
     ap.add_argument("--serial", action="store_true",
                     help="run the step's solves one after another on one host thread (same contexts and "
                          "kernels; for profilers, which serialise kernels anyway)")
@@ -468,6 +470,31 @@ def pass_bytes(n, d, s):
     }
 
 
+def iteration_bytes(nodes, d, loads=1):
+    """Bytes one frequency-domain CG iteration (float32) reads and writes, in
+    scalars per node: r, p, A p, x read and r, p, x written by the update, A p
+    written and r, p read by the projection, the two-channel and (3-D) the
+    three-component spectra written and read between the passes; a byte of
+    phase."""
+    return (18 if d == 2 else 30) * 4 * nodes * loads + nodes
+
+
+def iteration_ms(solve, k0, k1):
+    """Time of one CG iteration: the difference of two solves that stop at k0 and
+    k1 iterations of their first refinement step.  solve(k) returns its info."""
+    def median_time(k):
+        t = []
+        for _ in range(5):
+            t0 = time.perf_counter()
+            info = solve(k)
+            t.append(time.perf_counter() - t0)
+            if info["iters"] != k:
+                raise RuntimeError(f"expected {k} iterations: {info}")
+        return statistics.median(t[1:])
+
+    return 1e3 * (median_time(k1) - median_time(k0)) / (k1 - k0)
+
+
 def run_fh(args):
     import numpy as np
     import torch
@@ -488,11 +515,6 @@ def run_fh(args):
     # solves of a step run concurrently, one host thread each (a context is
     # used by one thread at a time), as a serving loop would run them.
     first = fh.Solver(phase, tables[0], precision="fp32_refined", stream=torch.cuda.Stream())
-    tune = None
-    if not args.no_tune:
-        before, after = first.autotune("fp32")
-        tune = {"ms_per_iter_before": before, "ms_per_iter_after": after,
-                "cache": os.environ.get("FH_TUNE_CACHE")}
     units = [(first, 0, LOADS[0])]
     for i, L in enumerate(tables):
         for j, E in enumerate(LOADS):
@@ -606,7 +628,11 @@ def run_fh(args):
     h2d, d2h = bytes_moved["h2d"], bytes_moved["d2h"]
     solvers = [u[0] for u in units]
 
-    # ---- matvec and per-kernel roofline (float32 pipeline, rho = 1e2 context)
+    # ---- roofline of the CG iteration the timed step runs (rho = 1e4 context),
+    # matvec, and the passes of the iteration on fields (rho = 1e2 context)
+    it_ms = iteration_ms(lambda k: solvers[6].solve(LOADS[0], tol=1e-12, method="cg", max_iter=k, want_field=False)[2],
+                         20, 100)
+    it_bytes = iteration_bytes(N * N, 2)
     prof = solvers[2]  # rho = 1e2, E = (1, 0)
     s4, d = 4, 2
     nodes = N * N
@@ -615,11 +641,9 @@ def run_fh(args):
     times = {k: prof.profile(w, reps=30) for k, (w, _) in kern.items()}
     t_apply = prof.profile(5, reps=30)
     peak, peak_src = load_peaks()
-    dom = max(times, key=lambda k: times[k])
-    achieved = kern[dom][1] / (times[dom] * 1e-3) / 1e9
+    achieved = it_bytes / (it_ms * 1e-3) / 1e9
     b_min = (2 * d * s4 + 1) * nodes
     b_apply = (d * s4 + 1) * nodes + spec + 2 * spec + spec + 2 * d * s4 * nodes
-    traffic = recorded_traffic(dom)
 
     # ---- CG on cuFFT (baselines, measured once) ----------------------------
     base = base32 = None
@@ -710,15 +734,11 @@ def run_fh(args):
                     "d2h_bytes_per_step": d2h // args.steps},
             "gpu_launches": launches,
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                         "frac": achieved / peak, "traffic": traffic, "kernel": dom,
-                         "traffic_source": (f"recorded, not measured by this run: ncu dram__bytes_read.sum + "
-                                            f"dram__bytes_write.sum of a cold-L2 launch ({TRAFFIC_SUMMARY}, "
-                                            f"kernel sources {csrc_digest()})") if traffic else None,
-                         "peak_source": peak_src,
-                         "algorithmic_bytes_per_launch": kern[dom][1],
-                         "ms_per_launch": times[dom]},
-            "kernels_ms": times,
-            "autotune": tune,
+                         "frac": achieved / peak, "traffic": None,
+                         "kernel": "one CG iteration (k_spec_inv, k_spec_row, k_spec_fwd, k_scal_spec)",
+                         "peak_source": peak_src, "algorithmic_bytes_per_launch": it_bytes,
+                         "ms_per_launch": it_ms},
+            "field_passes_ms": times,
             "matvec": {"ms": t_apply, "matvecs_per_s": 1e3 / t_apply,
                        "dof_per_s": d * nodes * 1e3 / t_apply,
                        "alg_gbs_B_min": b_min / (t_apply * 1e-3) / 1e9,
@@ -809,11 +829,6 @@ def run_c4(args):
     gen_s = time.perf_counter() - t0
     nodes = sum(c[2] * c[2] for c in cells)
     b = fh.Batch([c[0] for c in cells], [c[1] for c in cells], nloads=2, precision="fp32_refined")
-    tune = None
-    if not args.no_tune:
-        t0 = time.perf_counter()
-        before, after = b.autotune()
-        tune = {"ms_per_iter_before": before, "ms_per_iter_after": after, "s": time.perf_counter() - t0}
     E = np.eye(2)
     for _ in range(args.warmup):
         b.solve(E, tol=TOL, method="cg", max_iter=MAX_ITER)
@@ -841,7 +856,6 @@ def run_c4(args):
         "config": {"workload": f"{len(cells)} 2-D cells, N in {C4_SIZES}, disks/ellipses/laminates vf 0.3, "
                                f"rho log-U[1e1,1e4], 2 loads, CG fp32 + fp64 refinement to {TOL:g}",
                    "total_nodes": nodes, "generation_s": gen_s},
-        "autotune": tune,
         "clocks": clk,
         "dof_iter_per_s": float(np.sum(iters * np.repeat([c[2] * c[2] * 2 for c in cells], 2)))
                           / (t_ms / args.steps * 1e-3),
@@ -874,10 +888,6 @@ def run_c3(args):
     gen_s = time.perf_counter() - t0
     L = micro.isotropic_table([1.0, 1e3], 3)
     s = fh.Solver(phase, L, precision="fp32_refined")
-    tune = None
-    if not args.no_tune:
-        before, after = s.autotune(loads=True)
-        tune = {"ms_per_iter_before": before, "ms_per_iter_after": after}
     for _ in range(args.warmup):
         s.solve_all(tol=TOL, max_iter=MAX_ITER)
     clocks = Clocks(local)
@@ -891,20 +901,11 @@ def run_c3(args):
     ev1.synchronize()
     clk = clocks.stop()
     t_ms = ev0.elapsed_time(ev1)
-    # roofline of the 3-D float32 CG-iteration passes (the context's one-load
-    # pipeline, the 243-point compile-time plan): algorithmic bytes per launch
-    n3 = 243 ** 3
-    d3, s4 = 3, 4
-    spec3 = 2 * s4 * d3 * ((243 + 1) // 2) * 243 * 243
-    kern3 = {"row_fwd": (0, (3 * d3 * s4 + 1) * n3 + spec3),
-             "col_mid_green_mid": (1, 6 * spec3),  # middle-axis forward, Green pass, middle-axis inverse
-             "row_inv": (2, spec3 + 2 * d3 * s4 * n3),
-             "cg_update": (3, 6 * d3 * s4 * n3)}
-    times3 = {k: s.profile(w, reps=20) for k, (w, _) in kern3.items()}
+    # roofline of one CG iteration of all three loads
+    it_ms = iteration_ms(lambda k: s.solve_all(tol=1e-12, max_iter=k)[1][0], 10, 60)
+    it_bytes = iteration_bytes(243 ** 3, 3, loads=3)
+    ach3 = it_bytes / (it_ms * 1e-3) / 1e9
     peak, peak_src = load_peaks()
-    dom3 = max(times3, key=lambda k: times3[k])
-    ach3 = kern3[dom3][1] / (times3[dom3] * 1e-3) / 1e9
-    traffic3 = recorded_traffic(dom3, TRAFFIC_SUMMARY_3D)
     s.close()
     line = {
         "metric": "3-D full effective tensor: time per load solve to true rel.res 1e-6 (3 loads per launch)",
@@ -913,20 +914,16 @@ def run_c3(args):
         "vs_baseline": None, "dtype": "f32 (f64 refinement)", "data": "synthetic",
         "config": {"workload": "3-D N=243^3 Boolean spheres r=12 vf>=0.25, rho=1e3, loads e1,e2,e3 batched",
                    "vf": float(micro.digital_fraction(phase)), "generation_s": gen_s},
-        "autotune": tune,
         "clocks": clk,
         "gpu_launches": sum(i["launches"] for i in infos[:1]) * args.steps,
         "solver": {"iters": [i["iters"] for i in infos], "outer_iters": infos[0]["outer_iters"],
                    "rel_res_true": [i["rel_res_true"] for i in infos], "status": [i["status"] for i in infos],
                    "L_eff": Le.tolist(), "ct_plans": infos[0]["ct_plans"]},
         "roofline": {"bound": "hbm", "achieved": ach3, "peak": peak, "unit": "GB/s", "frac": ach3 / peak,
-                     "traffic": traffic3, "kernel": dom3, "peak_source": peak_src,
-                     "traffic_source": (f"recorded, not measured by this run: ncu dram__bytes_read.sum + "
-                                        f"dram__bytes_write.sum of cold-L2 launches ({TRAFFIC_SUMMARY_3D}, "
-                                        f"kernel sources {csrc_digest()})") if traffic3 else None,
-                     "algorithmic_bytes_per_launch": kern3[dom3][1], "ms_per_launch": times3[dom3],
-                     "note": "one-load float32 pipeline of the same context (fh_profile)"},
-        "kernels_ms": times3,
+                     "traffic": None,
+                     "kernel": "one CG iteration, 3 loads (k_spec_inv, k_spec_mid x 2, k_spec_row, k_spec_fwd, "
+                               "k_scal_spec)",
+                     "peak_source": peak_src, "algorithmic_bytes_per_launch": it_bytes, "ms_per_launch": it_ms},
     }
     print(json.dumps(line), flush=True)
 

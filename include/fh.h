@@ -225,27 +225,31 @@ fh_status fh_eta_e(fh_ctx* ctx, const double* e, double* eta);
  * Synchronises.  Errors: FH_ERR_ARG, FH_ERR_CUDA. */
 fh_status fh_profile(fh_ctx* ctx, int dtype, int what, int reps, double* ms);
 
-/* fh_autotune -- choose the launch shapes of the context's pipeline of the
- * given precision (FH_FP32 or FH_FP64) by timing candidates: half-spectrum
- * tile width, lines per CTA of the row passes, and the radix plan (threads per
- * line / column FFT).  Each candidate is a temporary set of buffers of the
+/* fh_autotune -- choose the launch shapes of the passes on fields in the
+ * context's pipeline of the given precision (FH_FP32 or FH_FP64) by timing
+ * candidates: half-spectrum tile width, lines per CTA of the row passes, and
+ * the radix plan (threads per line / column FFT).  These passes run every solve
+ * and product in float64, CG of FH_FP32 contexts, BiCG and the fixed point;
+ * CG of FH_FP32_REFINED contexts and the float32 product run frequency-layout
+ * passes, whose shapes are chosen by rule, and do not change.  Each candidate is a temporary set of buffers of the
  * same size as the context's; its four CG-iteration pass kernels are timed
  * with CUDA events (10 launches each).  If a faster shape is found the
  * pipeline is rebuilt with it (its Krylov vectors are reallocated, so any
  * solve state is lost).  When the environment variable FH_TUNE_CACHE names a
  * file, the result is appended to it, and fh_create reads that file to start
  * every later context of the same shape with the tuned launch shapes.
- *  ms_before / ms_after  host, may be NULL: summed pass time per CG iteration
- *                        before and after.
+ *  ms_before / ms_after  host, may be NULL: summed time of the passes on fields
+ *                        per CG iteration before and after.
  * Synchronises.  Errors: FH_ERR_ARG, FH_ERR_OOM, FH_ERR_CUDA, FH_ERR_UNSUPPORTED. */
 fh_status fh_autotune(fh_ctx* ctx, int dtype, double* ms_before, double* ms_after);
 
 /* fh_autotune_loads -- the same search for the pipeline of fh_solve_all,
  * which carries all d unit loads in every launch (float32; FH_FP32 and
- * FH_FP32_REFINED contexts).  The best shapes are appended to the tuning
+ * FH_FP32_REFINED contexts); its BiCG and fixed-point iterations run the passes
+ * on fields.  The best shapes are appended to the tuning
  * cache under this grid with d loads, and the next fh_solve_all uses them.
- * ms_before / ms_after (host, or NULL): float32 CG-iteration time of the
- * default and of the chosen shapes.  Errors: FH_ERR_ARG (FH_FP64 context),
+ * ms_before / ms_after (host, or NULL): time of the float32 passes on fields
+ * per CG iteration with the default and the chosen shapes.  Errors: FH_ERR_ARG (FH_FP64 context),
  * FH_ERR_OOM, FH_ERR_CUDA. */
 fh_status fh_autotune_loads(fh_ctx* ctx, double* ms_before, double* ms_after);
 
@@ -292,11 +296,12 @@ fh_status fh_batch_create(fh_batch** out, int ncells, const int* N, const uint8_
 fh_status fh_batch_solve(fh_batch* b, const double* E, double tol, int method, int max_iter,
                          double* Leff, int* status, int* iters, fh_info* summary);
 
-/* fh_batch_autotune -- pick the launch shapes of every size group's float32
- * pipeline (FH_FP32_REFINED batches) by timing a bounded set of candidates
- * on the group itself, as fh_autotune does for one cell.  ms_before /
- * ms_after (host, or NULL): the summed float32 CG-iteration time of all
- * groups before and after.  Synchronises.  Errors: FH_ERR_ARG, FH_ERR_OOM,
+/* fh_batch_autotune -- pick the launch shapes of the passes on fields in every
+ * size group's float32 pipeline (FH_FP32_REFINED batches; their BiCG and
+ * fixed-point iterations) by timing a bounded set of candidates on the group
+ * itself, as fh_autotune does for one cell.  ms_before / ms_after (host, or
+ * NULL): the summed time of those passes per CG iteration of all groups before
+ * and after.  Synchronises.  Errors: FH_ERR_ARG, FH_ERR_OOM,
  * FH_ERR_CUDA. */
 fh_status fh_batch_autotune(fh_batch* b, double* ms_before, double* ms_after);
 

@@ -895,7 +895,6 @@ fh_status fh_project_compatible(fh_ctx* c, const double* in, double* out) {
 
 fh_status fh_profile(fh_ctx* c, int dtype, int what, int reps, double* ms) {
   if (!c || !ms || reps < 1) return FH_ERR_ARG;
-  if (what > 5) what = 4;  // no such piece
   std::string err;
   int rc;
   if (dtype == FH_FP64 && c->p64 && c->p64->x[0]) {

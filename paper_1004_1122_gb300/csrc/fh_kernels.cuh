@@ -300,7 +300,9 @@ __device__ __forceinline__ void block_reduce_store(double (&v)[NV], int nv, doub
 }
 
 // First statement of the kernels of a chain (seq_launch): wait for the kernel
-// before this one and its writes, then let the next one's CTAs in.
+// before this one and its writes.  No launch trigger follows, so the next
+// kernel's CTAs start only when all of this one's have ended; buffers that the
+// chain updates in place (spectra, r, p) depend on that.
 __device__ __forceinline__ void seq_begin() {
   cudaGridDependencySynchronize();
 }

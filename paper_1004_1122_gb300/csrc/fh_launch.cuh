@@ -21,7 +21,7 @@ struct Launch {
 // of 4 to 10 short kernels gains 2 to 4 % (405x675 refined 8.19 -> 7.85 ms,
 // 81^2 float64 CG 1.44 -> 1.41 ms); single products gain nothing and launch
 // plainly.  Letting the next kernel's CTAs in before this one's have ended was
-// worse on small grids (405x675: 9.73 ms, 255^2 BiCGSTAB 10.6 instead of
+// worse on small grids (405x675: 9.73 ms, 255^2 BiCG 10.6 instead of
 // 9.9 ms): they take the SMs that are free, two to an SM, and leave the others
 // idle.
 template <typename... P, typename... A>

@@ -48,7 +48,7 @@ template <typename T, int D>
 constexpr bool kHasDf = std::is_same<T, double>::value && D == 2;
 
 // Spread plans: float64, one load per launch (grids too small to give every
-// SM scheduler a warp; see spread_plans in the pipeline).
+// SM scheduler a warp; the rule is in Pipeline::init).
 template <typename T, int NL>
 constexpr bool kHasSpread = std::is_same<T, double>::value && NL == 1;
 

@@ -203,11 +203,13 @@ struct Pipeline {
   unsigned long long uid = 0;  // next_pipeline_uid() of the last init
   int init(const Problem& pb, int nloads_, bool krylov, cudaStream_t stream, std::string& err,
            const Tuning* want = nullptr);
-  // Time the CG-iteration pass kernels for candidate tunings (temporary
-  // pipelines) and return the fastest; `ms` receives its time per iteration.
+  // Time the pass kernels of the iteration on fields for candidate tunings
+  // (temporary pipelines) and return the fastest; `ms` receives its time per
+  // iteration.
   static int autotune(const Problem& pb, int nloads, cudaStream_t stream, Tuning& best, double& ms,
                       std::string& err, int max_candidates = 256, bool want_spectral = false);
-  // device time of one CG iteration's kernels (what autotune compares)
+  // device time of the four pass kernels of one CG iteration on the fields (what
+  // autotune compares; the frequency-domain passes take their shapes by rule)
   int iteration_time(double* ms, std::string& err);
   template <typename W> int upload_twiddles(const FFTPlan& pl, W** dst, std::string& err);
   void release();

@@ -106,7 +106,7 @@ int Pipeline<T>::init(const Problem& pb, int nloads_, bool krylov, cudaStream_t 
   // pipelines whose passes would leave SM schedulers without a warp.  A float64
   // warp instruction occupies its scheduler's unit for 64 cycles on this part,
   // so a pass then takes one thread's chain of float64 operations: the more
-  // threads share a sequence, the shorter (255^2 BiCGSTAB 20.2 -> 10.0 ms, 81^2
+  // threads share a sequence, the shorter (255^2 BiCG 20.2 -> 10.0 ms, 81^2
   // CG 2.04 -> 1.43 ms).  From one warp per scheduler on (128 threads per SM)
   // the pass is bound by the operations' total, which the standard plans'
   // fewer and longer stages keep smaller.
@@ -464,7 +464,6 @@ int Pipeline<T>::init_spectral(const Problem& pb, std::string& err) {
     sg.csh = 0;
     while ((1 << sg.csh) < Cc) ++sg.csh;
     sg.Tt = (g.H + Cc - 1) / Cc;
-    if (sg.Tt * Cc % 2) ++sg.Tt;  // 16-byte aligned lines
     sg.Hp = sg.Tt * Cc;
     for (int k = 0; k < 3; ++k) sg.invY[k] = (float)g.invY[k];
     sg.inv_nodes = (float)g.inv_nodes;

@@ -3,8 +3,11 @@
 //
 // Which lengths: the odd lengths whose only prime factors are 3 and 5, from 75
 // nodes (shorter axes belong to grids that launch latency bounds); each entry
-// is the plan make_fft_plan picks for that length, in mirror_order.  Other lengths, and the
-// small-radix plans of small grids, run the run-time-plan kernels.
+// is the plan make_fft_plan picks for that length, in mirror_order.  Other
+// lengths, and the small-radix plans of small grids, run the run-time-plan
+// kernels.  Lengths with a factor 7 are left out to keep the compile time: some
+// twenty-five more plans would instantiate three column, two middle and up to
+// six row kernels each; what they would gain has not been measured.
 #pragma once
 
 #include "fh_launch_impl.cuh"

@@ -33,8 +33,9 @@
 // brings the initial residual's norm to about 1 (psi_f, exact): psi is 1 / sqrt|N|
 // of a field, and its squares would leave float32's range for loads of 1e-11.
 //
-// Memory moved per iteration in units of one real scalar per node: 19.25 in
-// 2-D (113 / 4 = 28.25 with the fields' passes), 32.25 in 3-D (59.25).
+// Memory moved per iteration in units of one real scalar per node: 18.25 in
+// 2-D (update 7, spectra 6, projection 5, phase 1/4; 28.25 with the fields'
+// passes), 30.25 in 3-D (54.25).
 // Measured per iteration, against the passes on fields: 2187^2 168 -> 127 us
 // (row 44, inv 43, fwd 33, scalars 7; 349 MB, 51 us at the copy rate), 243^3
 // with three loads 2.54 -> 1.43 ms (row 402, inv 284, mid 271 + 253, fwd 217;
