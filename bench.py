@@ -488,8 +488,8 @@ def iteration_ms(solve, k0, k1):
             t0 = time.perf_counter()
             info = solve(k)
             t.append(time.perf_counter() - t0)
-            if info["iters"] != k:
-                raise RuntimeError(f"expected {k} iterations: {info}")
+            if info["iters"] != k or info["outer_iters"] != 1:
+                raise RuntimeError(f"expected {k} iterations of the first refinement step: {info}")
         return statistics.median(t[1:])
 
     return 1e3 * (median_time(k1) - median_time(k0)) / (k1 - k0)

@@ -61,8 +61,8 @@ fh_status fh_nn_forward(fh_nn* nn, const float* x, float* y);
  * backward.  *loss (host, may be NULL) receives the loss; grad_host (host,
  * param_count floats, may be NULL) receives the gradient.  Synchronises.
  * FH_ERR_TIMEOUT: a tensor-core kernel's bounded wait expired in this call or
- * in an fh_nn_forward before it; reported once, with *loss and grad_host left
- * as they were. */
+ * in an fh_nn_forward before it; reported once, and what grad_host holds then is
+ * no gradient. */
 fh_status fh_nn_gradients(fh_nn* nn, const float* x, const float* target, double* loss, float* grad_host);
 
 /* One Adam step (beta1 0.9, beta2 0.999, eps 1e-8, bias correction with the

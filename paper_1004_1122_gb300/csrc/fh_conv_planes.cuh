@@ -270,6 +270,7 @@ template <int T, int NT> __global__ void __launch_bounds__(kConvThreads) k_conv_
   fence_after();
   const uint32_t tmem = tmem_slot;
   const int ntile = a.tiles_z * g.n0;
+  int commits = 0;  // the issuing thread: accumulators committed
   const long long plane0 = (long long)g.py * g.px;
 
   if (warp == 4) {
@@ -381,17 +382,12 @@ template <int T, int NT> __global__ void __launch_bounds__(kConvThreads) k_conv_
         }
         commit(&tfull[buf]);
       }
-      // every issued MMA has finished before tensor memory is released, and every
-      // commit has arrived before the CTA leaves (the epilogue, which waits for
-      // the accumulators' commits, may have given up)
+      // every issued MMA has finished before tensor memory is released
       for (int st = 0; st < nstage; ++st) {
         const int cnt = (it + nstage - 1 - st) >> ssh;
         if (cnt > 0) tma::mbar_wait(&empty[st], (cnt - 1) & 1);
       }
-      for (int b = 0; b < 2; ++b) {
-        const int cnt = (nt + 1 - b) >> 1;  // commits of this accumulator
-        if (cnt > 0) tma::mbar_wait(&tfull[b], (cnt - 1) & 1);
-      }
+      commits = nt;
     }
   } else {
     const long long V = g.v();
@@ -442,7 +438,16 @@ template <int T, int NT> __global__ void __launch_bounds__(kConvThreads) k_conv_
   }
   fence_before();
   __syncthreads();
-  if (tid == 0 && s_fail && a.err) atomicExch(a.err, 1);
+  if (s_fail) {
+    if (tid == 0 && a.err) atomicExch(a.err, 1);
+    // an epilogue that gave up no longer waits for the accumulators' commits:
+    // the last of each has arrived before the CTA leaves
+    for (int b = 0; b < 2; ++b) {
+      const int cnt = (commits + 1 - b) >> 1;
+      if (cnt > 0) tma::mbar_wait(&tfull[b], (cnt - 1) & 1);
+    }
+  }
+  __syncwarp();
   if (warp == 0) {
     fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(ncols) : "memory");

@@ -431,15 +431,16 @@ cudaError_t loss_gradient(fh_nn* n, const float* target) {
   return cudaGetLastError();
 }
 
-// Waits for what is queued, reads the loss and the device error word (bounded
-// waits that expired, in this call or an earlier forward); a word that was set
-// is reported once and cleared.
-int finish(fh_nn* n, double* loss) {
+// Waits for what is queued, reads the loss, the gradient (into grad_host, if
+// any) and the device error word (bounded waits that expired, in this call or an
+// earlier forward); a word that was set is reported once and cleared.
+int finish(fh_nn* n, double* loss, float* grad_host) {
   const long long cnt = n->lv[0].v() * n->cout;
   const int g = std::min(n->npart, grid1(cnt));
   int* const h_err = reinterpret_cast<int*>(n->h_part + n->npart);
   if (cudaMemcpyAsync(n->h_part, n->part, g * sizeof(double), cudaMemcpyDeviceToHost, n->st) != cudaSuccess ||
       cudaMemcpyAsync(h_err, n->dev_err, sizeof(int), cudaMemcpyDeviceToHost, n->st) != cudaSuccess ||
+      (grad_host && cudaMemcpyAsync(grad_host, n->G, n->nparam * sizeof(float), cudaMemcpyDeviceToHost, n->st) != cudaSuccess) ||
       cudaStreamSynchronize(n->st) != cudaSuccess)
     return FH_ERR_CUDA;
   if (*h_err != 0)
@@ -633,14 +634,7 @@ fh_status fh_nn_gradients(fh_nn* n, const float* x, const float* target, double*
     cudaStreamSynchronize(n->side);  // weight gradients that were launched read this call's planes
     return FH_ERR_CUDA;
   }
-  const int rc = finish(n, loss);
-  if (rc) return (fh_status)rc;
-  if (grad_host) {
-    if (cudaMemcpyAsync(grad_host, n->G, n->nparam * sizeof(float), cudaMemcpyDeviceToHost, n->st) != cudaSuccess ||
-        cudaStreamSynchronize(n->st) != cudaSuccess)
-      return FH_ERR_CUDA;
-  }
-  return FH_OK;
+  return (fh_status)finish(n, loss, grad_host);
 }
 
 fh_status fh_nn_train_step(fh_nn* n, const float* x, const float* target, float lr, int step, double* loss) {
