@@ -34,12 +34,12 @@
 // of a field, and its squares would leave float32's range for loads of 1e-11.
 //
 // Memory moved per iteration in units of one real scalar per node: 18.25 in
-// 2-D (update 7, spectra 6, projection 5, phase 1/4; 28.25 with the fields'
+// 2-D (update 7, spectra 8, projection 3, phase 1/4; 28.25 with the fields'
 // passes), 30.25 in 3-D (54.25).
-// Measured per iteration, against the passes on fields: 2187^2 168 -> 127 us
-// (row 44, inv 43, fwd 33, scalars 7; 349 MB, 51 us at the copy rate), 243^3
-// with three loads 2.54 -> 1.43 ms (row 402, inv 284, mid 271 + 253, fwd 217;
-// 5.4 GB, 0.79 ms at the copy rate).  Bound by the FFT stages' shared-memory
+// Measured per iteration, against the passes on fields: 2187^2 168 -> 125 us
+// (row 44, inv 42, fwd 38; 349 MB, 51 us at the copy rate), 243^3 with three
+// loads 2.54 -> 1.46 ms (row 403, inv 287, mid 270 + 254, fwd 234; 5.2 GB,
+// 0.76 ms at the copy rate).  Bound by the FFT stages' shared-memory
 // round trips and barriers at 24 warps per SM (45 % of the issue slots); small
 // grids (405x675: 25 us) by the length of one thread's chain per kernel.
 //
@@ -64,7 +64,7 @@ struct SpecGeom {
 // factor of the projection.  float32: the kernels of an iteration do no
 // float64 work per element or per thread (a warp's float64 instruction holds
 // the pipe for 16 cycles; the conversions and the float64 block reductions of
-// an earlier version kept that pipe 73 % busy in spec_fwd).
+// an earlier version kept that pipe 73 % busy in spec_fwd; sums are Sum3).
 struct SpecMedium {
   float L00, s01, s02, L11, s12, L22;  // sij = L0ij + L0ji
   float scale;                         // 1 / (|N| l0) for isotropic L0, else 1 / |N|
@@ -132,8 +132,8 @@ struct Sum3 {
 __device__ __forceinline__ float2 dot_parts(const DotAcc<float>& d) { return make_float2(d.s, -d.c); }
 
 // Sums of `rows` rows of `count` values (a thread's two parts each) in shared
-// memory, row k at src(k)[at(i)]; its sum goes to *out(k).  Call after a barrier behind the
-// writes.  A row is summed by 32 lanes, or by 8 where a kernel carries several
+// memory, row k at src(k)[at(i)]; its sum goes to *out(k).  Call after a barrier
+// behind the writes.  A row is summed by 32 lanes, or by 8 where a kernel carries several
 // loads: there the CTAs are small and many, and the trees' instructions count
 // more than the length of the chain (243^3, three loads: 644 -> 610 ms per tensor
 // with that and the sums kept in the tile instead of behind it).
@@ -327,8 +327,9 @@ __global__ void __launch_bounds__(SpecBounds<PS>::threads) k_spec_inv(SpecArgs a
         const int i = i0 + u * drow, k = i << (csh - 1);
         vr[u] = vp[u] = va[u] = vx[u] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         if (i < n && live) {
-          // r and x are touched once per iteration: kept out of the way of
-          // what the next passes read again (S, p, A p)
+          // r and x are kept out of the way of what the next passes read again
+          // (S, p, A p; r too is read by the projection, but storing it the
+          // ordinary way made no difference: 2187^2 14.36 and 14.28 ms)
           if (MODE == kSpecUpdate) vr[u] = __ldcs(r + k);
           if (!fresh) {
             if (MODE == kSpecUpdate) va[u] = __ldg(ap + k);
