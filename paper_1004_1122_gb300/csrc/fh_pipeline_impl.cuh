@@ -348,11 +348,19 @@ int Pipeline<T>::init(const Problem& pb, int nloads_, bool krylov, cudaStream_t 
   }
   if (krylov) {
     // one block for the field vectors, each on a 256-byte boundary (with p2,
-    // the second direction buffer of CG, where it is needed from the start)
-    const int per = want_spectral ? 6 : 5;
+    // the second direction buffer of CG, where it is needed from the start and
+    // there is the memory for it)
+    int per = want_spectral ? 6 : 5;
     const size_t len = ((size_t)vlen + 64 + 63) / 64 * 64;
     T* v = nullptr;
-    if ((rc = dev_alloc(allocs, &v, len * per * nloads, err))) return rc;
+    rc = dev_alloc(allocs, &v, len * per * nloads, err);
+    if (rc && per == 6) {
+      cudaGetLastError();
+      want_spectral = false;
+      per = 5;
+      rc = dev_alloc(allocs, &v, len * per * nloads, err);
+    }
+    if (rc) return rc;
     for (int l = 0; l < nloads; ++l)
       for (T** b : {&x[l], &r[l], &p[l], &ap[l], &rhs[l], &p2[l]}) {
         if (b == &p2[l] && per == 5) continue;

@@ -20,8 +20,8 @@ N = (243, 243, 243)
 KEEP = 60 << 20
 
 
-def _tight(torch, fh, args, kw):
-    """A context created in the memory an ordinary one takes, less KEEP."""
+def _tight(torch, fh, args, kw, less=KEEP):
+    """A context created in the memory an ordinary one takes, less `less` bytes."""
     torch.cuda.synchronize()
     torch.cuda.empty_cache()
     before = torch.cuda.mem_get_info()[0]
@@ -29,7 +29,7 @@ def _tight(torch, fh, args, kw):
         torch.cuda.synchronize()
         took = before - torch.cuda.mem_get_info()[0]
     free = torch.cuda.mem_get_info()[0]
-    junk = torch.empty(free - took + KEEP, dtype=torch.uint8, device="cuda")
+    junk = torch.empty(free - took + less, dtype=torch.uint8, device="cuda")
     try:
         return fh.Solver(*args, **kw)
     finally:
@@ -59,3 +59,16 @@ def test_a_context_without_the_frequency_buffers(precision):
             y, _, info = s.solve([1.0, 0.5, 0.25], tol=1e-8)
             assert info["status"] == "FH_OK"
             assert float((y - x).norm()) <= 2 * 20 * 1e-8 * float(x.norm())
+
+
+def test_a_context_without_the_second_direction_buffer():
+    """Refined contexts allocate CG's second direction (12 bytes per node) with
+    the others; methods that need none run where it does not fit."""
+    torch = cuda_or_skip()
+    from paper_1004_1122_gb300 import fh
+
+    phase = (np.random.default_rng(2).random(N) < 0.3).astype(np.uint8)
+    args, kw = (phase, micro.isotropic_table([1.0, 4.0], 3)), {"precision": "fp32_refined"}
+    with _tight(torch, fh, args, kw, less=220 << 20) as s:
+        _, _, info = s.solve([1.0, 0.5, 0.25], tol=1e-6, method="fixed_point")
+    assert info["status"] == "FH_OK"
